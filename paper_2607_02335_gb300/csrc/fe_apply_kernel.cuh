@@ -1,5 +1,5 @@
-// fe_apply_kernel.cuh -- sum-factorized cell-wise operator apply (one template, three
-// arithmetics).
+// fe_apply_kernel.cuh -- sum-factorized cell-wise operator apply (one template for the FP64 pipe, FP32
+// and 16-bit operands; the FP64-accurate double-word path is fe_apply_pair.cuh).
 //
 // Per cell K the kernel computes y_K = A_K x_K, the unassembled dual output of the local
 // operator (Sec. 3.1), with the sum factorization of Sec. 2.3 extended to general
@@ -15,15 +15,14 @@
 // data sits in registers (global load/store, pointwise geometry, z sweeps), the x-line
 // (j,k) = (t % n, t / n) and the y-line (i,k) = (t % n, t / n) for the x and y sweeps, which
 // read and write the cell's tile in shared memory.  Rows of the tile are padded to n+1 entries,
-// which keeps the line accesses of a warp free of bank conflicts (double-word values are stored
-// as interleaved hi/lo pairs, one 64-bit access each).
+// which keeps the line accesses of a warp free of bank conflicts.
 //
 // Every 1D contraction uses the even-odd form of the matrix (the reflection symmetry of the GLL
 // nodes and Gauss points; the even-odd decomposition named in Sec. 2.3 "Initial performance
 // measurements"), which halves the multiply-adds.
 // Up to n = FE_ROLL_MINN - 1 all loops unroll with compile-time indices, so the 1D tables (kernel
 // parameters) are read from the constant bank as instruction operands; from n = FE_ROLL_MINN on
-// the double-word and FP64 kernels keep the output loop of each contraction a run-time loop
+// the FP64-pipe kernels keep the output loop of each contraction a run-time loop
 // (apply_cells_rolled), because fully unrolled they no longer fit the instruction cache.
 #pragma once
 #include <type_traits>
@@ -80,19 +79,6 @@ template <>
 struct Sm<hfv> : Sm16<hfv> {
   using Sm16<hfv>::Sm16;
 };
-template <>
-struct Sm<dw> {  // hi and lo interleaved: one 64-bit shared-memory access per value
-  float2* p;
-  __device__ __forceinline__ Sm(unsigned char* base, int, int arr, int tile)
-      : p(reinterpret_cast<float2*>(base) + (size_t)arr * tile) {}
-  __device__ __forceinline__ dw get(int e) const {
-    const float2 v = p[e];
-    return {v.x, v.y};
-  }
-  __device__ __forceinline__ void put(int e, dw v) const { p[e] = make_float2(v.h, v.l); }
-  static constexpr int BYTES = 8;
-};
-
 // One 1D contraction of a line in even-odd form (the EO comment in fe_internal.h):
 // put(q, value) receives output q.  ROLLED: the output pairs are a run-time loop (outputs must
 // go to shared memory); otherwise everything unrolls and put may write a register array.
@@ -107,24 +93,24 @@ __device__ __forceinline__ void eo_line(const EO<N, V>& t, const V (&in)[N], Put
     o[r] = T::subk(in[r], in[N - 1 - r]);
   }
   if constexpr (N & 1) {
-    V acc;
     if constexpr (SIG > 0) {
-      acc = T::prod(t.mm, in[MID]);
+      auto acc = T::prod(t.mm, in[MID]);
 #pragma unroll
       for (int r = 0; r < H; ++r) acc = T::mac(acc, t.cr[r], e[r]);
+      put(MID, T::keep(acc));
     } else {
-      acc = T::prod(t.cr[0], o[0]);
+      auto acc = T::prod(t.cr[0], o[0]);
 #pragma unroll
       for (int r = 1; r < H; ++r) acc = T::mac(acc, t.cr[r], o[r]);
+      put(MID, T::keep(acc));
     }
-    put(MID, T::keep(acc));
   }
   auto pair = [&](int q) {
-    V a = T::prod(t.A[q][0], e[0]);
+    auto a = T::prod(t.A[q][0], e[0]);
 #pragma unroll
     for (int r = 1; r < H; ++r) a = T::mac(a, t.A[q][r], e[r]);
     if constexpr (N & 1) a = T::mac(a, t.cm[q], in[MID]);
-    V b = T::prod(t.B[q][0], o[0]);
+    auto b = T::prod(t.B[q][0], o[0]);
 #pragma unroll
     for (int r = 1; r < H; ++r) b = T::mac(b, t.B[q][r], o[r]);
     put(q, T::addk(a, b));
@@ -154,25 +140,24 @@ __device__ __forceinline__ void eob_line(const EOB<N, V>& t, const V (&d)[N - 1]
     o[s] = T::subk(d[s], d[NI - 1 - s]);
   }
   if constexpr (N & 1) {  // middle output (no middle difference for odd n)
-    V acc = T::prod(t.cr[0], e[0]);
+    auto acc = T::prod(t.cr[0], e[0]);
 #pragma unroll
     for (int s = 1; s < HI; ++s) acc = T::mac(acc, t.cr[s], e[s]);
     put(N / 2, T::keep(acc));
   }
   auto pair = [&](int q) {
-    V a;
     if constexpr (HI > 0) {
-      a = T::prod(t.A[q][0], e[0]);
+      auto a = T::prod(t.A[q][0], e[0]);
 #pragma unroll
       for (int s = 1; s < HI; ++s) a = T::mac(a, t.A[q][s], e[s]);
       if constexpr (NI & 1) a = T::mac(a, t.cm[q], d[NI / 2]);
-      V b = T::prod(t.B[q][0], o[0]);
+      auto b = T::prod(t.B[q][0], o[0]);
 #pragma unroll
       for (int s = 1; s < HI; ++s) b = T::mac(b, t.B[q][s], o[s]);
       put(q, T::addk(a, b));
       put(N - 1 - q, T::subk(a, b));
     } else {  // n = 2: one difference, a constant derivative
-      a = T::keep(T::prod(t.cm[q], d[0]));
+      const V a = T::keep(T::prod(t.cm[q], d[0]));
       put(q, a);
       put(N - 1 - q, a);
     }
@@ -185,92 +170,6 @@ __device__ __forceinline__ void eob_line(const EOB<N, V>& t, const V (&d)[N - 1]
 #pragma unroll
     for (int q = 0; q < HO; ++q) pair(q);
   }
-}
-
-// Exponent shift of the FP64 path: the CTA's inputs enter the double-word arithmetic scaled by
-// 2^-sh, sh = (binary exponent of the largest finite |x| of the CTA), and every output is scaled
-// back by 2^sh.  Powers of two are exact, so the result is the same operator applied to x; the
-// scaling keeps every intermediate double-word value (and its low part) inside the float range
-// whatever the magnitude of x.  Scaled values below 2^-74 (of the CTA's largest) are flushed to
-// zero.  All threads of the CTA call it; it holds a __syncthreads.
-template <int N>
-__device__ __forceinline__ int cta_exp_shift(const double (&xr)[N]) {
-  __shared__ unsigned s_wmax[32];
-  unsigned em = 0;
-#pragma unroll
-  for (int k = 0; k < N; ++k) {
-    unsigned e = ((unsigned)__double2hiint(xr[k]) >> 20) & 0x7FFu;
-    em = max(em, e == 0x7FFu ? 0u : e);  // infinities and NaNs keep their own value
-  }
-  const unsigned warp = threadIdx.x >> 5;
-  const unsigned lanes = min(32u, blockDim.x - warp * 32u);
-  em = __reduce_max_sync(lanes == 32u ? 0xFFFFFFFFu : ((1u << lanes) - 1u), em);
-  if ((threadIdx.x & 31u) == 0u) s_wmax[warp] = em;
-  __syncthreads();
-  unsigned m = 0;
-  const unsigned nw = (blockDim.x + 31u) >> 5;
-  for (unsigned w = 0; w < nw; ++w) m = max(m, s_wmax[w]);
-  return (int)m - 1023;
-}
-
-// Reference gradient at the Gauss points from differences of the stored inputs (the FP64 path:
-// binary64 inputs into double-word differences; also written for float values): component a is
-// B'_a (the derivative from the differences along axis a) followed by V along the two other axes.
-// Every value the sweeps carry is of the size of a difference of neighbouring nodal values, not of
-// x itself, so the rounding of the sweeps does not meet the cancellation of the derivative (a
-// smooth field's Laplacian).  Three phases, each the same contraction on three lines of the thread
-// (an axis loop, not unrolled, which keeps the kernel's code within the instruction cache):
-//   1  B' on the x-, y- and z-line of the inputs (raw tile)  -> s1, s2, s0
-//   2  V  along z of s1 and s2, along x of s0
-//   3  V  along y of s1, along x of s2, along y of s0
-// On return s1, s2, s0 hold d/dx, d/dy, d/dz of u at the Gauss points and sh the exponent shift
-// (FP64 path; 0 otherwise).
-template <int N, class V, int RU>
-__device__ __forceinline__ void diff_gradient(const typename NT<V>::SV (&xr)[N],
-                                              const Sm<typename NT<V>::SV>& raw, const Sm<V>& s0,
-                                              const Sm<V>& s1, const Sm<V>& s2, int cb, int la,
-                                              int lb, const Tab1D<N, V>& tab, int& sh) {
-  constexpr bool DW = std::is_same<V, dw>::value;
-  using SV = typename NT<V>::SV;
-  constexpr int RS = Cfg<N>::RS, PS = Cfg<N>::PS;
-  const int bx = cb + lb * PS + la * RS, by = cb + lb * PS + la, bz = cb + lb * RS + la;
-#pragma unroll
-  for (int k = 0; k < N; ++k) raw.put(bz + k * PS, xr[k]);
-  if constexpr (DW)
-    sh = cta_exp_shift<N>(xr);  // its barrier also publishes the raw tile
-  else
-    __syncthreads();
-#pragma unroll 1
-  for (int ax = 0; ax < 3; ++ax) {
-    const int base = ax == 0 ? bx : (ax == 1 ? by : bz);
-    const int st = ax == 0 ? 1 : (ax == 1 ? RS : PS);
-    const Sm<V> o = ax == 0 ? s1 : (ax == 1 ? s2 : s0);
-    SV dd[N - 1];
-#pragma unroll
-    for (int r = 0; r < N - 1; ++r) dd[r] = raw.get(base + (r + 1) * st) - raw.get(base + r * st);
-    V d[N - 1];
-#pragma unroll
-    for (int r = 0; r < N - 1; ++r) {
-      if constexpr (DW)
-        d[r] = dw_from_double_ftz(dd[r], sh);
-      else
-        d[r] = dd[r];
-    }
-    eob_line<N, V, RU>(tab.eB, d, [&](int q, V v) { o.put(base + q * st, v); });
-  }
-  __syncthreads();
-#pragma unroll 1
-  for (int ax = 0; ax < 6; ++ax) {
-    if (ax == 3) __syncthreads();
-    const Sm<V> o = (ax == 0 || ax == 3) ? s1 : ((ax == 1 || ax == 4) ? s2 : s0);
-    const int base = ax < 2 ? bz : ((ax == 2 || ax == 4) ? bx : by);
-    const int st = ax < 2 ? PS : ((ax == 2 || ax == 4) ? 1 : RS);
-    V in[N];
-#pragma unroll
-    for (int r = 0; r < N; ++r) in[r] = o.get(base + r * st);
-    eo_line<N, V, 1, RU>(tab.eV, in, [&](int q, V v) { o.put(base + q * st, v); });
-  }
-  __syncthreads();
 }
 
 // register line -> register line
@@ -437,10 +336,10 @@ __device__ __forceinline__ void brick_sums(const Sm<V>& s, int cb, int cl, int l
 
 // ---------------------------------------------------------------------------------------------
 // High degrees: the same sweeps with the output index of every 1D contraction as a run-time loop.
-// Fully unrolled n x n contractions in double-word arithmetic outgrow the instruction cache from
-// n ~ 6 on (the unrolled kernel then waits on instruction fetch); here each sweep is one unrolled
-// n-term dot product per output, the coefficients come from the constant bank with a
-// warp-uniform index, and every output goes straight to the shared-memory tile.
+// Fully unrolled n x n contractions outgrow the instruction cache from n ~ 6 on (the unrolled kernel
+// then waits on instruction fetch); here each sweep is one unrolled n-term dot product per output,
+// the coefficients come from the constant bank with a warp-uniform index, and every output goes
+// straight to the shared-memory tile.
 // ---------------------------------------------------------------------------------------------
 #ifndef FE_PREFETCH_MASS_MAXN  // mass: fetch w detJ of the z-line at the start up to this n
 #define FE_PREFETCH_MASS_MAXN 6
@@ -449,15 +348,14 @@ __device__ __forceinline__ void brick_sums(const Sm<V>& s, int cb, int cl, int l
 #define FE_ROLL_MINN 5
 #endif
 // single-float arithmetics (FP32, 16-bit operands) stay unrolled at every degree: a float
-// contraction is a fraction of the double-word one, the unrolled kernels fit the instruction cache,
+// contraction is one FMA per term, the unrolled kernels fit the instruction cache,
 // and they ran faster (FP32 Laplace at 32^3 Q7 0.113 against 0.138 ms, 48^3 Q5 0.171 against 0.210)
 #ifndef FE_ROLL_MINN_F32
 #define FE_ROLL_MINN_F32 9
 #endif
 template <class V>
 __host__ __device__ constexpr int roll_minn() {
-  return (std::is_same<V, dw>::value || std::is_same<V, double>::value) ? FE_ROLL_MINN
-                                                                         : FE_ROLL_MINN_F32;
+  return std::is_same<V, double>::value ? FE_ROLL_MINN : FE_ROLL_MINN_F32;
 }
 
 // s[base + q * stride] = (M in)_q, R output pairs per loop iteration
@@ -467,21 +365,15 @@ __device__ __forceinline__ void sweep_rolled(const EO<N, V>& M, const V (&in)[N]
   eo_line<N, V, SIG, R>(M, in, [&](int q, V v) { s.put(base + q * stride, v); });
 }
 
-// Output pairs per loop iteration of the run-time contraction loops (measured, double-word, GB300):
-// all of them (the loop unrolled) except the Laplace kernels at n = 6 and 8, where the unrolled
-// loops ran 7.5% slower (n = 6) and no faster (n = 8: equal at 32^3 cells, 10% slower at 16^3);
-// unrolled, the mass kernels gain 5-16% at n = 5..8 and the Laplace kernels 6% at n = 5 and 7.
+// output pairs per loop iteration of the run-time contraction loops: all of them except the Laplace
+// kernels at n = 6 and 8
 template <int N, int OP>
 __host__ __device__ constexpr int roll_unroll() {
   return (OP == FE_LAPLACE && (N == 6 || N == 8)) ? 1 : N / 2;
 }
 
-// Arrays of the shared-memory tile: Laplace 3 (the FP64 path a fourth for the binary64 inputs
-// that are differenced), mass 1.
-template <class V>
-__host__ __device__ constexpr int apply_narr(int op) {
-  return op == FE_LAPLACE ? (std::is_same<V, dw>::value ? 4 : 3) : 1;
-}
+// arrays of the shared-memory tile
+__host__ __device__ constexpr int apply_narr(int op) { return op == FE_LAPLACE ? 3 : 1; }
 
 template <int N, class V, int OP, int GEOM, int MODE>
 __device__ __forceinline__ void apply_cells_rolled(const CellArgs<N, V>& a, const Tab1D<N, V>& tab,
@@ -522,26 +414,11 @@ __device__ __forceinline__ void apply_cells_rolled(const CellArgs<N, V>& a, cons
     for (int r = 0; r < N; ++r) v[r] = s.get(base + r * stride);
   };
 
-  // FP64 path: binary64 inputs until they are differenced, CTA exponent shift (as apply_cells)
-  constexpr bool DW = std::is_same<V, dw>::value;
-  // FP64 path: Laplace gradient from differences of the binary64 inputs (diff_gradient)
-  constexpr bool DIFF = DW && OP == FE_LAPLACE;
-  using SV = typename NT<V>::SV;
-  int sh = 0;
   V in[N];
-  SV xr[(DW || DIFF) ? N : 1];
-  if constexpr (DW || DIFF) {
 #pragma unroll
-    for (int k = 0; k < N; ++k) {
-      const SV v = active ? __ldcs(a.x + gbase + k * N2 + lt) : SV(0);
-      xr[k] = masked(k) ? SV(0) : v;
-    }
-  } else {
-#pragma unroll
-    for (int k = 0; k < N; ++k) {
-      V v = active ? T::load_stream(a.x + gbase + k * N2 + lt) : T::zero();
-      in[k] = masked(k) ? T::zero() : v;
-    }
+  for (int k = 0; k < N; ++k) {
+    V v = active ? T::load_stream(a.x + gbase + k * N2 + lt) : T::zero();
+    in[k] = masked(k) ? T::zero() : v;
   }
   constexpr bool PREF_M = (OP == FE_MASS) && (GEOM == GEOM_STORED_K) && (N <= FE_PREFETCH_MASS_MAXN);
   V jpre[PREF_M ? N : 1];
@@ -551,32 +428,23 @@ __device__ __forceinline__ void apply_cells_rolled(const CellArgs<N, V>& a, cons
 #pragma unroll
     for (int k = 0; k < N; ++k) jpre[k] = active ? T::geo(g6 + k * N2) : T::zero();
   }
-  if constexpr (DIFF) {
-    diff_gradient<N, V, RU>(xr, Sm<SV>(smraw, 4, 3, tile_stride), s0, s1, s2, cb, la, lb, tab, sh);
-  } else {
-    if constexpr (DW) {
-      sh = cta_exp_shift<N>(xr);
-#pragma unroll
-      for (int k = 0; k < N; ++k) in[k] = dw_from_double_ftz(xr[k], sh);
-    }
-    sweep_rolled<N, V, 1, RU>(tab.eV, in, s0, bz, PS);  // z
-    __syncthreads();
+  sweep_rolled<N, V, 1, RU>(tab.eV, in, s0, bz, PS);  // z
+  __syncthreads();
+  load_line(s0, bx, 1, in);
+  sweep_rolled<N, V, 1, RU>(tab.eV, in, s0, bx, 1);  // x
+  __syncthreads();
+  load_line(s0, by, RS, in);
+  sweep_rolled<N, V, 1, RU>(tab.eV, in, s0, by, RS);  // y
+  __syncthreads();
+  if constexpr (OP == FE_LAPLACE) {
+    V inz[N];
+    load_line(s0, bz, PS, inz);
     load_line(s0, bx, 1, in);
-    sweep_rolled<N, V, 1, RU>(tab.eV, in, s0, bx, 1);  // x
-    __syncthreads();
+    sweep_rolled<N, V, -1, RU>(tab.eD, in, s1, bx, 1);  // d/dx -> s1
     load_line(s0, by, RS, in);
-    sweep_rolled<N, V, 1, RU>(tab.eV, in, s0, by, RS);  // y
+    sweep_rolled<N, V, -1, RU>(tab.eD, in, s2, by, RS);  // d/dy -> s2
     __syncthreads();
-    if constexpr (OP == FE_LAPLACE) {
-      V inz[N];
-      load_line(s0, bz, PS, inz);
-      load_line(s0, bx, 1, in);
-      sweep_rolled<N, V, -1, RU>(tab.eD, in, s1, bx, 1);  // d/dx -> s1
-      load_line(s0, by, RS, in);
-      sweep_rolled<N, V, -1, RU>(tab.eD, in, s2, by, RS);  // d/dy -> s2
-      __syncthreads();
-      sweep_rolled<N, V, -1, RU>(tab.eD, inz, s0, bz, PS);  // d/dz -> s0 (own z-line)
-    }
+    sweep_rolled<N, V, -1, RU>(tab.eD, inz, s0, bz, PS);  // d/dz -> s0 (own z-line)
   }
 
   if constexpr (OP == FE_LAPLACE) {
@@ -659,15 +527,12 @@ __device__ __forceinline__ void apply_cells_rolled(const CellArgs<N, V>& a, cons
       V v = s0.get(bz + k * PS);
       if (masked(k)) v = T::zero();
       if constexpr (T::LOWP) v.v *= a.oscale;
-      T::store(a.y + gbase + k * N2 + lt, v, sh);
+      T::store(a.y + gbase + k * N2 + lt, v);
     }
   }
 }
 
-// The cells cell0 .. cell0 + CPB - 1 (those below ncells), applied by the CTA's first CPB*n^2
-// threads.  Threads beyond that (a CTA wider than the tile, as in the batched persistent kernel)
-// work on a spare slot of the tile that nobody reads and still reach every barrier; the caller
-// then sizes each array tile_stride = TILE + CS.
+// The cells cell0 .. cell0 + CPB - 1 (those below ncells), applied by the CTA's CPB*n^2 threads.
 template <int N, class V, int OP, int GEOM, int MODE = MODE_CELLS>
 __device__ __forceinline__ void apply_cells(const CellArgs<N, V>& a, const Tab1D<N, V>& tab,
                                             long long cell0, unsigned char* smraw,
@@ -675,7 +540,7 @@ __device__ __forceinline__ void apply_cells(const CellArgs<N, V>& a, const Tab1D
                                             ZCarry<typename NT<V>::SV>* zc = nullptr) {
   static_assert(MODE != MODE_PACKED || N < FE_ROLL_MINN, "packed units: unrolled degrees only");
   static_assert(MODE != MODE_BRICKZ || (N < FE_ROLL_MINN && !NT<V>::LOWP),
-                "z-carry bricks: unrolled degrees, FP64 / double-word / FP32 values");
+                "z-carry bricks: unrolled degrees, FP64 / FP32 values");
   if constexpr (N >= roll_minn<V>() && MODE != MODE_PACKED) {
     apply_cells_rolled<N, V, OP, GEOM, MODE>(a, tab, cell0, smraw, tile_stride);
     return;
@@ -723,27 +588,11 @@ __device__ __forceinline__ void apply_cells(const CellArgs<N, V>& a, const Tab1D
       return gbase + k * N2 + lt;
     }
   };
-  // FP64 path (double-word values): the inputs stay binary64 until they are differenced, and the
-  // CTA's values are scaled by a power of two (cta_exp_shift)
-  constexpr bool DW = std::is_same<V, dw>::value;
-  // FP64 path: Laplace gradient from differences of the binary64 inputs (diff_gradient)
-  constexpr bool DIFF = DW && OP == FE_LAPLACE;
-  using SV = typename NT<V>::SV;
-  int sh = 0;
   V u[N], w[N];
-  SV xr[(DW || DIFF) ? N : 1];
-  if constexpr (DW || DIFF) {
 #pragma unroll
-    for (int k = 0; k < N; ++k) {
-      const SV v = active ? __ldcs(a.x + xaddr(k)) : SV(0);
-      xr[k] = masked(k) ? SV(0) : v;
-    }
-  } else {
-#pragma unroll
-    for (int k = 0; k < N; ++k) {
-      V v = active ? T::load_stream(a.x + xaddr(k)) : T::zero();
-      u[k] = masked(k) ? T::zero() : v;
-    }
+  for (int k = 0; k < N; ++k) {
+    V v = active ? T::load_stream(a.x + xaddr(k)) : T::zero();
+    u[k] = masked(k) ? T::zero() : v;
   }
   // low degrees: issue the metric loads now so that their latency hides behind the sweeps
 #ifndef FE_PREFETCH_MAXN
@@ -767,44 +616,32 @@ __device__ __forceinline__ void apply_cells(const CellArgs<N, V>& a, const Tab1D
 #pragma unroll
       for (int c = 0; c < 6; ++c) gpre[c * N + k] = active ? T::geo(g0 + c * N3 + k * N2) : T::zero();
   }
-  if constexpr (DIFF) {
-    diff_gradient<N, V, 0>(xr, Sm<SV>(smraw, 4, 3, tile_stride), s0, s1, s2, cb, la, lb, tab, sh);
-    // s1, s2, s0: d/dx, d/dy, d/dz of u at the Gauss points
+  eo_regs<N, V, 1>(tab.eV, u, w);
 #pragma unroll
-    for (int k = 0; k < N; ++k) u[k] = s0.get(cb + zl<N>(la, lb, k));
-  } else {
-    if constexpr (DW) {
-      sh = cta_exp_shift<N>(xr);
+  for (int k = 0; k < N; ++k) s0.put(cb + zl<N>(la, lb, k), w[k]);
+  __syncthreads();
+  tile_sweep<N, V, 0, 1>(s0, cb, la, lb, tab.eV);  // x
+  __syncthreads();
+  tile_sweep<N, V, 1, 1>(s0, cb, la, lb, tab.eV);  // y
+  __syncthreads();
+  // s0 now holds u at the Gauss points
+  if constexpr (OP == FE_LAPLACE) {
+    // ---- reference gradient at the Gauss points (collocation derivative)
+    V in[N], out[N];
 #pragma unroll
-      for (int k = 0; k < N; ++k) u[k] = dw_from_double_ftz(xr[k], sh);
-    }
-    eo_regs<N, V, 1>(tab.eV, u, w);
+    for (int r = 0; r < N; ++r) in[r] = s0.get(cb + xl<N>(la, lb, r));
+    eo_regs<N, V, -1>(tab.eD, in, out);
 #pragma unroll
-    for (int k = 0; k < N; ++k) s0.put(cb + zl<N>(la, lb, k), w[k]);
+    for (int r = 0; r < N; ++r) s1.put(cb + xl<N>(la, lb, r), out[r]);
+#pragma unroll
+    for (int r = 0; r < N; ++r) in[r] = s0.get(cb + yl<N>(la, lb, r));
+    eo_regs<N, V, -1>(tab.eD, in, out);
+#pragma unroll
+    for (int r = 0; r < N; ++r) s2.put(cb + yl<N>(la, lb, r), out[r]);
+#pragma unroll
+    for (int r = 0; r < N; ++r) in[r] = s0.get(cb + zl<N>(la, lb, r));
+    eo_regs<N, V, -1>(tab.eD, in, u);  // u := d/dz along the z-line
     __syncthreads();
-    tile_sweep<N, V, 0, 1>(s0, cb, la, lb, tab.eV);  // x
-    __syncthreads();
-    tile_sweep<N, V, 1, 1>(s0, cb, la, lb, tab.eV);  // y
-    __syncthreads();
-    // s0 now holds u at the Gauss points
-    if constexpr (OP == FE_LAPLACE) {
-      // ---- reference gradient at the Gauss points (collocation derivative)
-      V in[N], out[N];
-#pragma unroll
-      for (int r = 0; r < N; ++r) in[r] = s0.get(cb + xl<N>(la, lb, r));
-      eo_regs<N, V, -1>(tab.eD, in, out);
-#pragma unroll
-      for (int r = 0; r < N; ++r) s1.put(cb + xl<N>(la, lb, r), out[r]);
-#pragma unroll
-      for (int r = 0; r < N; ++r) in[r] = s0.get(cb + yl<N>(la, lb, r));
-      eo_regs<N, V, -1>(tab.eD, in, out);
-#pragma unroll
-      for (int r = 0; r < N; ++r) s2.put(cb + yl<N>(la, lb, r), out[r]);
-#pragma unroll
-      for (int r = 0; r < N; ++r) in[r] = s0.get(cb + zl<N>(la, lb, r));
-      eo_regs<N, V, -1>(tab.eD, in, u);  // u := d/dz along the z-line
-      __syncthreads();
-    }
   }
 
   if constexpr (OP == FE_LAPLACE) {
@@ -900,7 +737,7 @@ __device__ __forceinline__ void apply_cells(const CellArgs<N, V>& a, const Tab1D
     // The x/y sums inside the brick came first, as they do before the pass.
     if (active) {
       using SV = typename NT<V>::SV;
-      SV bottom = T::to_sv(masked(0) ? T::zero() : s0.get(cb + zl<N>(la, lb, 0)), sh);
+      SV bottom = T::to_sv(masked(0) ? T::zero() : s0.get(cb + zl<N>(la, lb, 0)));
       if (zc->pending) {
         bottom = zc->top + bottom;
         T::store_sv(a.y + gbase - (long long)a.mx * a.my * N3 + (N - 1) * N2 + lt, bottom);
@@ -910,9 +747,9 @@ __device__ __forceinline__ void apply_cells(const CellArgs<N, V>& a, const Tab1D
       for (int k = 1; k < N - 1; ++k) {
         V v = s0.get(cb + zl<N>(la, lb, k));
         if (masked(k)) v = T::zero();
-        T::store(a.y + gbase + k * N2 + lt, v, sh);
+        T::store(a.y + gbase + k * N2 + lt, v);
       }
-      const SV top = T::to_sv(masked(N - 1) ? T::zero() : s0.get(cb + zl<N>(la, lb, N - 1)), sh);
+      const SV top = T::to_sv(masked(N - 1) ? T::zero() : s0.get(cb + zl<N>(la, lb, N - 1)));
       if (zc->last) {
         T::store_sv(a.y + gbase + (N - 1) * N2 + lt, top);
         zc->pending = false;
@@ -952,7 +789,7 @@ __device__ __forceinline__ void apply_cells(const CellArgs<N, V>& a, const Tab1D
         V v = s0.get(cb + zl<N>(la, lb, k));
         if (masked(k)) v = T::zero();
         if constexpr (T::LOWP) v.v *= a.oscale;
-        T::store(yu + (long long)(sz * P + k) * NU * NU, v, sh);
+        T::store(yu + (long long)(sz * P + k) * NU * NU, v);
       }
     }
     return;
@@ -963,54 +800,11 @@ __device__ __forceinline__ void apply_cells(const CellArgs<N, V>& a, const Tab1D
       V v = s0.get(cb + zl<N>(la, lb, k));
       if (masked(k)) v = T::zero();
       if constexpr (T::LOWP) v.v *= a.oscale;
-      T::store(a.y + gbase + k * N2 + lt, v, sh);
+      T::store(a.y + gbase + k * N2 + lt, v);
     }
   }
 }
 
-// Resident CTAs per SM the one-layer kernels are compiled for: the double-word kernels are held
-// to the register budget of 3 (Laplace, unrolled degrees: 80 registers; n = 3: 4), 4 (Laplace,
-// rolled: 64; n = 7: 3, n = 8: 5) or 6 (mass: 40; up to n = 4: 8, n = 6: 5) CTAs per SM; the rest
-// are left to the compiler.
-// n = 3 double-word Laplace: 4 CTAs per SM (64 registers, no spills); its kernel waits on shared
-// memory rather than on issue, and the extra CTA took Q2 48^3 from 0.0887 to 0.0846 ms (assembled
-// 0.1184 to 0.1133 ms)
-#ifndef FE_DW_LAPLACE_MINB_N3
-#define FE_DW_LAPLACE_MINB_N3 4
-#endif
-// n = 8 double-word Laplace: 5 CTAs per SM (51 registers, no spills): Q7 32^3 0.621 -> 0.601 ms
-#ifndef FE_DW_LAPLACE_MINB_N8
-#define FE_DW_LAPLACE_MINB_N8 5
-#endif
-// n = 7 Laplace at 3 CTAs per SM and n = 6 mass at 5: the budgets of 4 and 6 spilled (100 and 16
-// bytes); Q6 32^3 Laplace 0.443 -> 0.437 ms, Q5 40^3 mass 0.171 -> 0.168 ms
-#ifndef FE_DW_LAPLACE_MINB_N7
-#define FE_DW_LAPLACE_MINB_N7 3
-#endif
-#ifndef FE_DW_MASS_MINB_N6
-#define FE_DW_MASS_MINB_N6 5
-#endif
-// double-word mass up to n = 4: 8 CTAs per SM (32 registers): Q3 96^3 0.580 -> 0.566 ms, Q2 48^3
-// assembled 0.0641 -> 0.0611 ms; from n = 5 on 32 registers spill, and 6 CTAs stay
-#ifndef FE_DW_MASS_MINB_LOW
-#define FE_DW_MASS_MINB_LOW 8
-#endif
-template <int N, class V, int OP>
-__host__ __device__ constexpr int apply_minb() {
-  return std::is_same<V, dw>::value
-             ? (OP == FE_LAPLACE
-                    ? (N == 3 ? FE_DW_LAPLACE_MINB_N3
-                              : (N < FE_ROLL_MINN ? 3
-                                                  : (N == 8 ? FE_DW_LAPLACE_MINB_N8
-                                                            : (N == 7 ? FE_DW_LAPLACE_MINB_N7 : 4))))
-                    : (N <= 4 ? FE_DW_MASS_MINB_LOW : (N == 6 ? FE_DW_MASS_MINB_N6 : 6)))
-             : 1;
-}
-#ifdef FE_MINB
-#define FE_APPLY_BOUNDS __launch_bounds__(Cfg<N>::THREADS, FE_MINB)
-#else
-#define FE_APPLY_BOUNDS __launch_bounds__(Cfg<N>::THREADS, (apply_minb<N, V, OP>()))
-#endif
 // z-carry bricks: held to a register budget for 3 CTAs per SM (Laplace, as the one-layer brick
 // kernel; left to itself the compiler gives the layer loop 98 registers, 2 CTAs per SM) or 6
 // (mass, whose one-layer kernel needs 32 registers)
@@ -1021,7 +815,7 @@ __host__ __device__ constexpr int apply_minb() {
 #define FE_ZCARRY_MINB_MASS 6
 #endif
 template <int N, class V, int OP, int GEOM, int MODE>
-__global__ void FE_APPLY_BOUNDS k_apply(const __grid_constant__ ApplyArgs<N, V> a) {
+__global__ void __launch_bounds__(Cfg<N>::THREADS) k_apply(const __grid_constant__ ApplyArgs<N, V> a) {
   extern __shared__ __align__(16) unsigned char smraw[];
   if (a.skip && *(volatile const int*)a.skip) return;  // uniform over the grid
   long long cell0;
@@ -1060,5 +854,5 @@ __global__ void __launch_bounds__(Cfg<N>::THREADS,
 
 template <int N, class V>
 inline size_t apply_smem_bytes(int op) {
-  return (size_t)apply_narr<V>(op) * Cfg<N>::TILE * Sm<V>::BYTES;
+  return (size_t)apply_narr(op) * Cfg<N>::TILE * Sm<V>::BYTES;
 }

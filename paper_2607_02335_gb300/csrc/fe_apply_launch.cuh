@@ -4,6 +4,7 @@
 #include <cstdlib>
 #include <cstring>
 
+#include "fe_apply_pair.cuh"
 #include "fe_recompute.cuh"
 
 template <class V>
@@ -16,6 +17,20 @@ template <>
 inline dw fe_cast<dw>(double v) {
   const float h = (float)v;
   return {h, (float)(v - (double)h)};
+}
+template <>
+inline dw2 fe_cast<dw2>(double v) {  // the same value for both cells of a pair
+  const dw x = fe_cast<dw>(v);
+  unsigned h, l;
+  std::memcpy(&h, &x.h, 4);
+  std::memcpy(&l, &x.l, 4);
+  return {h * 0x100000001ull, l * 0x100000001ull};
+}
+template <>
+inline dw2c fe_cast<dw2c>(double v) {
+  const dw2 x = fe_cast<dw2>(v);
+  constexpr unsigned long long sign = 0x8000000080000000ull;
+  return {x.h, x.h ^ sign, x.l ^ sign};
 }
 template <>
 inline bfv fe_cast<bfv>(double v) {  // round to nearest even bf16
@@ -34,15 +49,15 @@ void fill_eo(EO<N, V>& e, const double (&M0)[FE_MAXN][FE_MAXN], bool tr) {
   std::memset(&e, 0, sizeof(e));
   for (int q = 0; q < H; ++q) {
     for (int r = 0; r < H; ++r) {
-      e.A[q][r] = fe_cast<V>(0.5 * (M(q, r) + M(q, N - 1 - r)));
-      e.B[q][r] = fe_cast<V>(0.5 * (M(q, r) - M(q, N - 1 - r)));
+      e.A[q][r] = fe_cast<typename NT<V>::CV>(0.5 * (M(q, r) + M(q, N - 1 - r)));
+      e.B[q][r] = fe_cast<typename NT<V>::CV>(0.5 * (M(q, r) - M(q, N - 1 - r)));
     }
     if (N & 1) {
-      e.cm[q] = fe_cast<V>(M(q, mid));
-      e.cr[q] = fe_cast<V>(M(mid, q));
+      e.cm[q] = fe_cast<typename NT<V>::CV>(M(q, mid));
+      e.cr[q] = fe_cast<typename NT<V>::CV>(M(mid, q));
     }
   }
-  if (N & 1) e.mm = fe_cast<V>(M(mid, mid));
+  if (N & 1) e.mm = fe_cast<typename NT<V>::CV>(M(mid, mid));
 }
 
 // even-odd form of B' (EOB in fe_arith.h) from B = Dh: B'[q][s] = sum_{r > s} Dh[q][r]
@@ -59,43 +74,88 @@ void fill_eob(EOB<N, V>& e, const HostTab& h) {
   std::memset(&e, 0, sizeof(e));
   for (int q = 0; q < E::HO; ++q) {
     for (int s = 0; s < E::HI; ++s) {
-      e.A[q][s] = fe_cast<V>(0.5 * (Bp[q][s] + Bp[q][E::NI - 1 - s]));
-      e.B[q][s] = fe_cast<V>(0.5 * (Bp[q][s] - Bp[q][E::NI - 1 - s]));
+      e.A[q][s] = fe_cast<typename NT<V>::CV>(0.5 * (Bp[q][s] + Bp[q][E::NI - 1 - s]));
+      e.B[q][s] = fe_cast<typename NT<V>::CV>(0.5 * (Bp[q][s] - Bp[q][E::NI - 1 - s]));
     }
-    if (E::NI & 1) e.cm[q] = fe_cast<V>(Bp[q][E::NI / 2]);
+    if (E::NI & 1) e.cm[q] = fe_cast<typename NT<V>::CV>(Bp[q][E::NI / 2]);
   }
   if (N & 1)
-    for (int s = 0; s < E::HI; ++s) e.cr[s] = fe_cast<V>(Bp[N / 2][s]);
+    for (int s = 0; s < E::HI; ++s) e.cr[s] = fe_cast<typename NT<V>::CV>(Bp[N / 2][s]);
 }
 
-template <int N, class V>
-Tab1D<N, V> make_tab(const HostTab& h) {
-  Tab1D<N, V> t;
-  for (int a = 0; a < N; ++a) {
-    t.W_[a] = fe_cast<V>(h.w[a]);
+template <class T, class V, int N>
+void fill_full(T& t, const HostTab& h) {
+  for (int a = 0; a < N; ++a)
     for (int b = 0; b < N; ++b) {
       t.V_[a][b] = fe_cast<V>(h.V[a][b]);
       t.D_[a][b] = fe_cast<V>(h.D[a][b]);
     }
-  }
+}
+template <int N, class V>
+Tab1D<N, V> make_tab(const HostTab& h) {
+  Tab1D<N, V> t;
+  for (int a = 0; a < N; ++a) t.W_[a] = fe_cast<V>(h.w[a]);
   fill_eo<N, V>(t.eV, h.V, false);
   fill_eo<N, V>(t.eVT, h.V, true);
-  fill_eo<N, V>(t.eD, h.D, false);
   fill_eo<N, V>(t.eDT, h.D, true);
-  fill_eob<N, V>(t.eB, h);
+  if constexpr (std::is_same<V, dw2>::value || std::is_same<V, dw>::value) {
+    fill_eob<N, V>(t.eB, h);
+  } else {
+    fill_eo<N, V>(t.eD, h.D, false);
+    fill_full<Tab1D<N, V>, V, N>(t, h);
+  }
   return t;
 }
 
-template <int N, class V, int OP, int GEOM, int MODE = MODE_CELLS>
-static fe_status launch_one(const ApplyArgs<N, V>& a, cudaStream_t st) {
-  using C = Cfg<N>;
-  const size_t smem = apply_smem_bytes<N, V>(OP);
-  auto kern = [] {
+// tile of an arithmetic's kernels
+template <int N, class V>
+struct Shape {
+  static constexpr int CELLS = Cfg<N>::CPB, THREADS = Cfg<N>::THREADS, UPB = Packed<N>::UPB;
+  using B = Brick<N>;
+  static constexpr int BRICK_THREADS = B::BX * B::BY * Cfg<N>::N2;
+  static size_t smem(int op) { return apply_smem_bytes<N, V>(op); }
+  template <int OP, int GEOM, int MODE>
+  static auto kernel() {
     if constexpr (MODE == MODE_BRICKZ)
       return k_apply_zcarry<N, V, OP, GEOM>;
     else
       return k_apply<N, V, OP, GEOM, MODE>;
-  }();
+  }
+};
+template <int N, int SHAPE>
+struct PairShape {
+  using C = PairCfg<N, SHAPE>;
+  static constexpr int CELLS = C::CELLS, THREADS = C::THREADS, UPB = C::UPB;
+  using B = PairBrick<(N <= 4 ? N : 4)>;  // bricks up to n = 4 only
+  static constexpr int BRICK_THREADS = C::THREADS;
+  static size_t smem(int op) { return pair_smem_bytes<N, SHAPE>(op); }
+  template <int OP, int GEOM, int MODE>
+  static auto kernel() {
+    if constexpr (MODE == MODE_BRICKZ)
+      return k_apply_pair_zcarry<N, OP, GEOM>;
+    else
+      return k_apply_pair<N, OP, GEOM, MODE, SHAPE>;
+  }
+};
+template <int N>
+struct Shape<N, dw2> : PairShape<N, TILE_PAIRS> {};
+template <int N>
+struct Shape<N, dw> : PairShape<N, TILE_SINGLE> {};
+
+inline int fe_sm_count() {  // of the current device
+  static int cached[64] = {};
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 1;
+  if (cached[dev] == 0 &&
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
+    cached[dev] = sms;
+  return cached[dev] > 0 ? cached[dev] : 1;
+}
+
+template <int N, class V, int OP, int GEOM, int MODE, class Sh>
+static fe_status launch_shape(const ApplyArgs<N, V>& a, cudaStream_t st) {
+  const size_t smem = Sh::smem(OP);
+  auto kern = Sh::template kernel<OP, GEOM, MODE>();
   static bool attr_done[64] = {};  // one attribute call per instantiation and device
   int dev = 0;
   FE_CUDA(cudaGetDevice(&dev), "cudaGetDevice");
@@ -105,51 +165,63 @@ static fe_status launch_one(const ApplyArgs<N, V>& a, cudaStream_t st) {
     if (dev >= 0 && dev < 64) attr_done[dev] = true;
   }
   long long blocks;
-  int threads = C::THREADS;
+  int threads = Sh::THREADS;
   if constexpr (MODE == MODE_BRICK) {
-    constexpr int BX = Brick<N>::BX, BY = Brick<N>::BY;
+    constexpr int BX = Sh::B::BX, BY = Sh::B::BY;
     blocks = (long long)((a.c.mx + BX - 1) / BX) * ((a.c.my + BY - 1) / BY) * a.c.mz;
-    threads = BX * BY * C::N2;
+    threads = Sh::BRICK_THREADS;
   } else if constexpr (MODE == MODE_BRICKZ) {
-    constexpr int BX = Brick<N>::BX, BY = Brick<N>::BY;
+    constexpr int BX = Sh::B::BX, BY = Sh::B::BY;
     blocks = (long long)((a.c.mx + BX - 1) / BX) * ((a.c.my + BY - 1) / BY) *
              ((a.c.mz + a.zchunk - 1) / a.zchunk);
-    threads = BX * BY * C::N2;
+    threads = Sh::BRICK_THREADS;
   } else if constexpr (MODE == MODE_PACKED) {
-    blocks = (a.c.ncells / 8 + Packed<N>::UPB - 1) / Packed<N>::UPB;
+    blocks = (a.c.ncells / 8 + Sh::UPB - 1) / Sh::UPB;
   } else {
-    blocks = (a.c.ncells - a.c.cell_base + C::CPB - 1) / C::CPB;
+    blocks = (a.c.ncells - a.c.cell_base + Sh::CELLS - 1) / Sh::CELLS;
   }
   if (blocks > 0) kern<<<(unsigned)blocks, threads, smem, st>>>(a);
   return fe_cuda_check(cudaGetLastError(), "apply kernel launch");
+}
+
+// the launch in the arithmetic's tile, or in the pair kernel's small one
+template <int N, class V, int OP, int GEOM, int MODE = MODE_CELLS>
+static fe_status launch_one(const ApplyArgs<N, V>& a, cudaStream_t st) {
+  if constexpr (std::is_same<V, dw2>::value && MODE == MODE_CELLS) {
+    if (pair_shape<N>(a.c.ncells - a.c.cell_base, fe_sm_count()) == TILE_PAIRS_SMALL)
+      return launch_shape<N, V, OP, GEOM, MODE, PairShape<N, TILE_PAIRS_SMALL>>(a, st);
+  }
+  return launch_shape<N, V, OP, GEOM, MODE, Shape<N, V>>(a, st);
 }
 
 // Recompute mode: per chunk of cells, the metric into the L2-sized scratch, then the stored-metric
 // apply on the chunk.
 template <int N, class V, int OP>
 static fe_status launch_recompute(ApplyArgs<N, V> a, const ApplyLaunch& L,
-                                  const typename NT<V>::GV* xyz, typename NT<V>::GV* scratch) {
+                                  const typename RV<V>::GV* xyz, typename NT<V>::GV* scratch) {
   const fe_mesh* m = L.m;
   if (!xyz || !scratch) {
     fe_set_error("apply: recompute-mode buffers missing for this arithmetic");
     return FE_ERR_INVALID;
   }
   using G = GeoCfg<N>;
-  const long long chunk = fe_rc_chunk_cells(N, m->ncells, sizeof(typename NT<V>::GV));
-  RecomputeArgs<N, V> r;
+  using W = typename RV<V>::T;
+  const long long chunk = fe_rc_chunk_cells(N, m->ncells, sizeof(typename NT<W>::GV));
+  RecomputeArgs<N, W> r;
   std::memset(&r, 0, sizeof(r));
   r.xyz = xyz;
-  r.geo = scratch;
+  r.geo = reinterpret_cast<typename NT<W>::GV*>(scratch);
   r.skip = L.skip;
-  r.tab = a.tab;
+  for (int q = 0; q < N; ++q) r.tab.W_[q] = fe_cast<W>(m->tab.w[q]);
+  fill_full<RecomputeTab<N, W>, W, N>(r.tab, m->tab);
   a.c.geo = scratch;
   for (long long c0 = 0; c0 < m->ncells; c0 += chunk) {
     const long long c1 = c0 + chunk < m->ncells ? c0 + chunk : m->ncells;
     r.cell0 = c0;
     r.cell_end = c1;
     const long long gblocks = (c1 - c0 + G::CPB - 1) / G::CPB;
-    k_recompute<N, V, OP>
-        <<<(unsigned)gblocks, G::THREADS, recompute_smem_bytes<N, V>(), L.st>>>(r);
+    k_recompute<N, W, OP>
+        <<<(unsigned)gblocks, G::THREADS, recompute_smem_bytes<N, W>(), L.st>>>(r);
     FE_CUDA(cudaGetLastError(), "recompute kernel launch");
     a.c.cell_base = c0;
     a.c.geo_cell0 = c0;
@@ -166,7 +238,7 @@ static fe_status launch_recompute(ApplyArgs<N, V> a, const ApplyLaunch& L,
 // Layers per CTA of a z-carry launch (< 2: use the one-layer brick kernel).  The CTAs run
 // zchunk layers each, so the grid's last wave decides the tail: the largest zchunk <=
 // FE_ZCARRY_MAXZ whose grid fills at least four waves of resident CTAs, the last one to 97%
-// (Q3 96^3, double-word: 15 layers for the Laplace kernel at 3 CTAs per SM, 9 for mass at 6).
+// (Q3 96^3, double-word: 11 layers for the Laplace kernel at 5 CTAs per SM, 9 for mass at 6).
 template <int N, class V, int OP, int GEOM>
 static fe_status zcarry_slots(int* slots) {
   static int cached[64] = {};
@@ -176,13 +248,13 @@ static fe_status zcarry_slots(int* slots) {
     *slots = cached[dev];
     return FE_OK;
   }
-  auto kern = k_apply_zcarry<N, V, OP, GEOM>;
-  const size_t smem = apply_smem_bytes<N, V>(OP);
+  using Sh = Shape<N, V>;
+  auto kern = Sh::template kernel<OP, GEOM, MODE_BRICKZ>();
+  const size_t smem = Sh::smem(OP);
   FE_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
           "apply smem attribute");
   int per_sm = 0, sms = 0;
-  FE_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-              &per_sm, kern, Brick<N>::BX * Brick<N>::BY * Cfg<N>::N2, smem),
+  FE_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, Sh::BRICK_THREADS, smem),
           "occupancy");
   FE_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "SM count");
   *slots = per_sm * sms;
@@ -207,7 +279,7 @@ static fe_status zcarry_chunk(const fe_mesh* m, int op, bool affine, int* zc) {
     return FE_OK;
   }
   if (slots < 1) return FE_OK;
-  constexpr int BX = Brick<N>::BX, BY = Brick<N>::BY;
+  constexpr int BX = Shape<N, V>::B::BX, BY = Shape<N, V>::B::BY;
   const double per_layer = (double)((m->d.mx + BX - 1) / BX) * ((m->d.my + BY - 1) / BY);
   for (int z = FE_ZCARRY_MAXZ < m->d.mz ? FE_ZCARRY_MAXZ : m->d.mz; z >= 2; --z) {
     const double waves = (double)((m->d.mz + z - 1) / z) * per_layer / slots;
@@ -230,15 +302,29 @@ static fe_status launch_geom(const ApplyArgs<N, V>& a, int op, bool affine, cuda
                           : launch_one<N, V, FE_MASS, GEOM_STORED_K, MODE>(a, st);
 }
 
+// Assembled applies sum the intra-brick interfaces in the kernel up to n = FE_FUSE_MAXN.  Above it
+// the bricks hold fewer cells than the unfused tile (n = 6, 7) or the kernel needs more
+// registers, and the measured assembled time was no better than apply + full DSS.
+#ifndef FE_FUSE_MAXN
+#define FE_FUSE_MAXN 4
+#endif
+// what follows an apply kernel that summed nothing between cells
+static fe_status finish_unfused(const ApplyLaunch& L, int prec) {
+  if (!L.assemble) return FE_OK;
+  if (L.brick_out) {  // the caller runs the passes
+    L.brick_out[0] = L.brick_out[1] = 1;
+    return FE_OK;
+  }
+  return fe_launch_dss(L.m, prec, L.y, L.st);
+}
+
 template <int N, class V>
-static fe_status launch_apply_n(const ApplyLaunch& L, const typename NT<V>::GV* geo,
-                                const typename NT<V>::GV* xyz, typename NT<V>::GV* scratch) {
+static void fill_args(ApplyArgs<N, V>& a, const ApplyLaunch& L, const void* geo) {
   const fe_mesh* m = L.m;
-  ApplyArgs<N, V> a;
   std::memset(&a, 0, sizeof(a));
   a.c.x = static_cast<const typename NT<V>::SV*>(L.x);
   a.c.y = static_cast<typename NT<V>::SV*>(L.y);
-  a.c.geo = geo;
+  a.c.geo = static_cast<const typename NT<V>::GV*>(geo);
   a.c.ncells = m->ncells;
   a.c.mx = m->d.mx;
   a.c.my = m->d.my;
@@ -253,6 +339,27 @@ static fe_status launch_apply_n(const ApplyLaunch& L, const typename NT<V>::GV* 
   a.c.aff[3] = fe_cast<V>(det);
   a.tab = make_tab<N, V>(m->tab);
   a.c.oscale = 1.0f;
+}
+
+template <int N, class V>
+static fe_status launch_apply_n(const ApplyLaunch& L, const typename NT<V>::GV* geo,
+                                const typename RV<V>::GV* xyz, typename NT<V>::GV* scratch) {
+  const fe_mesh* m = L.m;
+  using Sh = Shape<N, V>;
+  const bool affine = m->d.geom_mode == FE_GEOM_AFFINE;
+  const bool fuse = L.assemble && N <= FE_FUSE_MAXN;
+  // single cells where pairs would leave the SMs part-empty (the unfused layouts only)
+  if constexpr (std::is_same<V, dw2>::value) {
+    if (!fuse && !m->packed && m->d.geom_mode != FE_GEOM_RECOMPUTE &&
+        pair_shape<N>(m->ncells, fe_sm_count()) == TILE_SINGLE) {
+      ApplyArgs<N, dw> one;
+      fill_args<N, dw>(one, L, geo);
+      FE_TRY((launch_geom<N, dw, MODE_CELLS>(one, L.op, affine, L.st)));
+      return finish_unfused(L, FE_F64);
+    }
+  }
+  ApplyArgs<N, V> a;
+  fill_args<N, V>(a, L, geo);
   if constexpr (NT<V>::LOWP) {
     if (m->d.geom_mode != FE_GEOM_STORED || !geo) {
       fe_set_error("apply: 16-bit contractions need stored geometry");
@@ -265,35 +372,18 @@ static fe_status launch_apply_n(const ApplyLaunch& L, const typename NT<V>::GV* 
     if (m->d.geom_mode == FE_GEOM_RECOMPUTE) {
       FE_TRY((L.op == FE_LAPLACE ? launch_recompute<N, V, FE_LAPLACE>(a, L, xyz, scratch)
                                  : launch_recompute<N, V, FE_MASS>(a, L, xyz, scratch)));
-      if (L.assemble && L.brick_out) {
-        L.brick_out[0] = L.brick_out[1] = 1;
-        return FE_OK;
-      }
-      return L.assemble ? fe_launch_dss(m, PREC, L.y, L.st) : FE_OK;
+      return finish_unfused(L, PREC);
     }
   }
-  const bool affine = m->d.geom_mode == FE_GEOM_AFFINE;
   if (m->packed) {  // 2^3-packed storage units: unit-internal assembly in the kernel
     if constexpr (N < FE_ROLL_MINN && N <= 4) {
       FE_TRY((launch_geom<N, V, MODE_PACKED>(a, L.op, affine, L.st)));
-      if (!L.assemble) return FE_OK;
-      if (L.brick_out) {
-        L.brick_out[0] = L.brick_out[1] = 1;
-        return FE_OK;
-      }
-      return fe_launch_dss(m, PREC, L.y, L.st);
+      return finish_unfused(L, PREC);
     } else {
       fe_set_error("apply: packed storage units are provided for degrees 1 to 3");
       return FE_ERR_INVALID;
     }
   }
-// Assembled applies sum the intra-brick interfaces in the kernel up to n = FE_FUSE_MAXN.  Above it
-// the bricks hold fewer cells than the unfused tile (n = 6, 7) or the kernel needs more
-// registers, and the measured assembled time was no better than apply + full DSS.
-#ifndef FE_FUSE_MAXN
-#define FE_FUSE_MAXN 4
-#endif
-  const bool fuse = L.assemble && N <= FE_FUSE_MAXN;
   // Fused assembled applies with the DSS passes left to this launcher also sum the z-interfaces
   // in the kernel: a CTA walks zchunk layers of its brick column; only the interfaces between
   // chunks remain for the z-pass.
@@ -304,27 +394,28 @@ static fe_status launch_apply_n(const ApplyLaunch& L, const typename NT<V>::GV* 
       if (zc >= 2) {
         a.zchunk = zc;
         FE_TRY((launch_geom<N, V, MODE_BRICKZ>(a, L.op, affine, L.st)));
-        return fe_launch_dss_strided3(m, PREC, L.y, Brick<N>::BX, Brick<N>::BY, zc, L.st);
+        return fe_launch_dss_strided3(m, PREC, L.y, Sh::B::BX, Sh::B::BY, zc, L.st);
       }
     }
   }
-  if (fuse)
-    FE_TRY((launch_geom<N, V, MODE_BRICK>(a, L.op, affine, L.st)));
-  else
+  if constexpr (N <= FE_FUSE_MAXN) {
+    if (fuse) FE_TRY((launch_geom<N, V, MODE_BRICK>(a, L.op, affine, L.st)));
+  }
+  if (!fuse) {
     FE_TRY((launch_geom<N, V, MODE_CELLS>(a, L.op, affine, L.st)));
-  if (!L.assemble) return FE_OK;
+    return finish_unfused(L, PREC);
+  }
   if (L.brick_out) {  // the caller runs the passes (one launch over many blocks)
-    L.brick_out[0] = fuse ? Brick<N>::BX : 1;
-    L.brick_out[1] = fuse ? Brick<N>::BY : 1;
+    L.brick_out[0] = Sh::B::BX;
+    L.brick_out[1] = Sh::B::BY;
     return FE_OK;
   }
-  return fuse ? fe_launch_dss_strided(m, PREC, L.y, Brick<N>::BX, Brick<N>::BY, L.st)
-              : fe_launch_dss(m, PREC, L.y, L.st);
+  return fe_launch_dss_strided(m, PREC, L.y, Sh::B::BX, Sh::B::BY, L.st);
 }
 
 template <class V>
 static fe_status launch_apply_v(const ApplyLaunch& L, const typename NT<V>::GV* geo,
-                                const typename NT<V>::GV* xyz, typename NT<V>::GV* scratch) {
+                                const typename RV<V>::GV* xyz, typename NT<V>::GV* scratch) {
   switch (L.m->n) {
     case 2: return launch_apply_n<2, V>(L, geo, xyz, scratch);
     case 3: return launch_apply_n<3, V>(L, geo, xyz, scratch);

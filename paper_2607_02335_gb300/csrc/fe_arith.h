@@ -37,11 +37,8 @@ __device__ __forceinline__ dw dw_fast_two_sum(float a, float b) {  // requires |
   float e = __fsub_rn(b, __fsub_rn(s, a));
   return {s, e};
 }
-// unnormalised accumulator acc + c*v, 10 FP32 operations.  s = acc.h + p with p = fl(c.h v.h); of
-// the TwoSum error, acc.h's share t1 = acc.h - (s - bb) is exact (bb = s - acc.h), and p's share
-// p - bb plus the product error c.h v.h - p is c.h v.h - bb, one fma (a small value rounded once,
-// an error of order 2^-24 ulp(s)).  The low parts and cross products go in float.
-// The 12-operation form: exact product error and a full TwoSum, low parts summed in float.
+// unnormalised accumulator acc + c*v: exact product error and a full TwoSum, low parts summed in
+// float (12 operations)
 __device__ __forceinline__ dw dw_mac12(dw acc, dw c, dw v) {
   float p = __fmul_rn(c.h, v.h);
   float e = __fmaf_rn(c.h, v.h, -p);
@@ -50,7 +47,10 @@ __device__ __forceinline__ dw dw_mac12(dw acc, dw c, dw v) {
   dw s = dw_two_sum(acc.h, p);
   return {s.h, __fadd_rn(acc.l, __fadd_rn(s.l, e))};
 }
-#ifndef FE_MAC_V1
+// The same in 10 operations.  s = acc.h + p with p = fl(c.h v.h); of the TwoSum error, acc.h's share
+// t1 = acc.h - (s - bb) is exact (bb = s - acc.h), and p's share p - bb plus the product error c.h v.h
+// - p is c.h v.h - bb, one fma (a small value rounded once, an error of order 2^-24 ulp(s)).  The low
+// parts and cross products go in float.
 __device__ __forceinline__ dw dw_mac(dw acc, dw c, dw v) {
   const float p = __fmul_rn(c.h, v.h);
   const float s = __fadd_rn(acc.h, p);
@@ -60,19 +60,16 @@ __device__ __forceinline__ dw dw_mac(dw acc, dw c, dw v) {
   const float x = __fmaf_rn(c.l, v.h, __fmaf_rn(c.h, v.l, acc.l));
   return {s, __fadd_rn(__fadd_rn(t1, t2), x)};
 }
-#else
-__device__ __forceinline__ dw dw_mac(dw acc, dw c, dw v) { return dw_mac12(acc, c, v); }
-#endif
 // c*v as an unnormalised pair (the first term of a dot product: no TwoSum with a zero accumulator)
 __device__ __forceinline__ dw dw_prod(dw c, dw v) {
-  float p = __fmul_rn(c.h, v.h);
+  const float p = __fmul_rn(c.h, v.h);
   float e = __fmaf_rn(c.h, v.h, -p);
   e = __fmaf_rn(c.h, v.l, e);
   e = __fmaf_rn(c.l, v.h, e);
   return {p, e};
 }
 __device__ __forceinline__ dw dw_add_keep(dw a, dw b) {
-  dw s = dw_two_sum(a.h, b.h);
+  const dw s = dw_two_sum(a.h, b.h);
   return {s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l))};
 }
 __device__ __forceinline__ dw dw_norm(dw a) { return dw_fast_two_sum(a.h, a.l); }
@@ -117,32 +114,6 @@ __device__ __forceinline__ dw dw_from_double(double x) {
   }
   return dw_from_double_slow(x);
 }
-// x * 2^-sh as a double-word: dw_from_double on the scaled exponent (sh from the CTA's largest
-// input, see cta_exp_shift in fe_apply_kernel.cuh).  Zero and subnormal x give 0; values that
-// the scaling leaves outside the exact range take the FP64 path (out of line).
-static __device__ __noinline__ dw dw_from_double_sh_slow(double x, int sh) {
-  const double v = scalbn(x, -sh);
-  const float hi = __double2float_rn(v);
-  return {hi, __double2float_rn(v - (double)hi)};
-}
-__device__ __forceinline__ dw dw_from_double_sh(double x, int sh) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  const unsigned e0 = (unsigned)(b >> 52) & 0x7FFu;
-  const unsigned e = e0 - (unsigned)sh;
-  if (e - 949u <= 201u && e0 - 1u < 2046u) {  // finite, normal, in range after the shift
-    const unsigned sign = (unsigned)(b >> 32) & 0x80000000u;
-    const float hi = __uint_as_float(sign | ((e - 896u) << 23) | (unsigned)((b >> 29) & 0x7FFFFFu));
-    const unsigned m = (unsigned)b & 0x1FFFFFFFu;
-    const float flo = __fsub_rn(__uint_as_float(0x4B000000u | (m & 0x7FFFFFu)), 8388608.0f);
-    const float fhi = __fsub_rn(__uint_as_float(0x4B000000u | (m >> 23)), 8388608.0f);
-    float lo = __fmul_rn(__fmaf_rn(fhi, 8388608.0f, flo), __uint_as_float((e - 948u) << 23));
-    lo = __uint_as_float(__float_as_uint(lo) | sign);
-    return {hi, lo};
-  }
-  if (e0 == 0u) return {0.0f, 0.0f};
-  return dw_from_double_sh_slow(x, sh);
-}
-
 // x * 2^-sh as a double-word without a branch: exact (as dw_from_double) for
 // 2^-74 <= |x| 2^-sh < 2^128; smaller values, zero and subnormals give 0; infinities and NaN give
 // NaN.  The callers choose sh so that no scaled value reaches 2^128.
@@ -220,7 +191,128 @@ __device__ __forceinline__ double dw_to_double_sh(dw a, int sh) {
 }
 
 // ---------------------------------------------------------------------------------------------
-// number traits: value type V, storage type of vectors (SV) and of geometry (GV)
+// packed double-word arithmetic: two values per operand (the two cells of a pair)
+// ---------------------------------------------------------------------------------------------
+// add / sub / mul / fma .f32x2 do the IEEE operation of both halves of a register pair in one
+// instruction.  The FP32 pipe's rate is the same as with scalar instructions (measured: 590 packed
+// against 1150 scalar warp instructions per ns on 152 SMs), but a packed one takes half the issue
+// slots, and the double-word kernels are bound by instruction issue: the other half of the slots
+// carries their loads, addressing and conversions.  Every half gets exactly the operations of the
+// scalar double-word arithmetic.
+typedef unsigned long long f2;
+__device__ __forceinline__ f2 f2_pack(float a, float b) {
+  f2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float2 f2_unpack(f2 v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ f2 f2_add(f2 a, f2 b) {
+  f2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f2 f2_sub(f2 a, f2 b) {
+  f2 r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
+  f2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+// The product is an fma with -0 read from memory the assembler cannot see through: it contracts
+// mul.rn.f32x2 and a following add.rn.f32x2 into one fma in spite of the .rn (measured: a chain of
+// two products 3e-8 off instead of 1e-14), which breaks the error-free sums below.
+static __constant__ f2 c_f2_negzero = 0x8000000080000000ull;
+__device__ __forceinline__ f2 f2_mul(f2 a, f2 b) { return f2_fma(a, b, c_f2_negzero); }
+__device__ __forceinline__ f2 f2_neg(f2 a) { return a ^ 0x8000000080000000ull; }
+
+struct dw2 {
+  f2 h, l;
+};
+// a running dot product with its low part negated (h - nl), and a table coefficient as the
+// products take it: the packed instructions have no operand negation, and with -h and -l of the
+// coefficient in the table every error term of a product comes out negated at no cost (rounding is
+// symmetric)
+struct dw2n {
+  f2 h, nl;
+};
+struct dw2c {
+  f2 h, nh, nl;
+};
+
+__device__ __forceinline__ dw2n dw2_prod(dw2c c, dw2 v) {
+  const f2 p = f2_mul(c.h, v.h);
+  return {p, f2_fma(c.nl, v.h, f2_fma(c.nh, v.l, f2_fma(c.nh, v.h, p)))};
+}
+__device__ __forceinline__ dw2n dw2_mac(dw2n acc, dw2c c, dw2 v) {
+  const f2 p = f2_mul(c.h, v.h);
+  const f2 s = f2_add(acc.h, p);
+  const f2 nbb = f2_sub(acc.h, s);
+  const f2 t1 = f2_sub(acc.h, f2_add(s, nbb));
+  const f2 t2 = f2_fma(c.h, v.h, nbb);
+  const f2 nx = f2_fma(c.nl, v.h, f2_fma(c.nh, v.l, acc.nl));
+  return {s, f2_sub(nx, f2_add(t1, t2))};
+}
+// the same for a run-time factor c
+__device__ __forceinline__ dw2 dw2_prod(dw2 c, dw2 v) {
+  const f2 p = f2_mul(c.h, v.h);
+  return {p, f2_fma(c.l, v.h, f2_fma(c.h, v.l, f2_fma(c.h, v.h, f2_neg(p))))};
+}
+__device__ __forceinline__ dw2 dw2_mac(dw2 acc, dw2 c, dw2 v) {
+  const f2 p = f2_mul(c.h, v.h);
+  const f2 s = f2_add(acc.h, p);
+  const f2 nbb = f2_sub(acc.h, s);
+  const f2 t1 = f2_sub(acc.h, f2_add(s, nbb));
+  const f2 t2 = f2_fma(c.h, v.h, nbb);
+  const f2 x = f2_fma(c.l, v.h, f2_fma(c.h, v.l, acc.l));
+  return {s, f2_add(f2_add(t1, t2), x)};
+}
+__device__ __forceinline__ dw2 dw2_two_sum(f2 a, f2 b) {
+  const f2 s = f2_add(a, b), bb = f2_sub(s, a);
+  return {s, f2_add(f2_sub(a, f2_sub(s, bb)), f2_sub(b, bb))};
+}
+__device__ __forceinline__ dw2 dw2_two_diff(f2 a, f2 b) {
+  const f2 s = f2_sub(a, b), bb = f2_sub(s, a);
+  return {s, f2_sub(f2_sub(a, f2_sub(s, bb)), f2_add(b, bb))};
+}
+__device__ __forceinline__ dw2 dw2_fast_two_sum(f2 a, f2 b) {
+  const f2 s = f2_add(a, b);
+  return {s, f2_sub(b, f2_sub(s, a))};
+}
+__device__ __forceinline__ dw2 dw2_addk(dw2 a, dw2 b) {
+  const dw2 s = dw2_two_sum(a.h, b.h);
+  return {s.h, f2_add(s.l, f2_add(a.l, b.l))};
+}
+__device__ __forceinline__ dw2 dw2_subk(dw2 a, dw2 b) {
+  const dw2 s = dw2_two_diff(a.h, b.h);
+  return {s.h, f2_add(s.l, f2_sub(a.l, b.l))};
+}
+__device__ __forceinline__ dw2 dw2_addk(dw2n a, dw2n b) {
+  const dw2 s = dw2_two_sum(a.h, b.h);
+  return {s.h, f2_sub(s.l, f2_add(a.nl, b.nl))};
+}
+__device__ __forceinline__ dw2 dw2_subk(dw2n a, dw2n b) {
+  const dw2 s = dw2_two_diff(a.h, b.h);
+  return {s.h, f2_sub(s.l, f2_sub(a.nl, b.nl))};
+}
+__device__ __forceinline__ dw2 dw2_add(dw2 a, dw2 b) {
+  const dw2 s = dw2_addk(a, b);
+  return dw2_fast_two_sum(s.h, s.l);
+}
+__device__ __forceinline__ dw2 dw2_mul(dw2 a, dw2 b) {
+  const dw2 p = dw2_prod(a, b);
+  return dw2_fast_two_sum(p.h, p.l);
+}
+
+// ---------------------------------------------------------------------------------------------
+// number traits: value type V, storage type of vectors (SV) and of geometry (GV), coefficient type
+// of the 1D tables (CV)
 // ---------------------------------------------------------------------------------------------
 template <class V>
 struct NT;
@@ -229,6 +321,7 @@ template <>
 struct NT<double> {
   using SV = double;
   using GV = double;
+  using CV = double;
   static constexpr bool LOWP = false;
   __device__ static __forceinline__ double zero() { return 0.0; }
   __device__ static __forceinline__ double mac(double a, double c, double v) { return fma(c, v, a); }
@@ -255,6 +348,7 @@ template <>
 struct NT<float> {
   using SV = float;
   using GV = float;
+  using CV = float;
   static constexpr bool LOWP = false;
   __device__ static __forceinline__ float zero() { return 0.0f; }
   __device__ static __forceinline__ float mac(float a, float c, float v) { return fmaf(c, v, a); }
@@ -293,6 +387,7 @@ template <class W>
 struct NT16 {
   using SV = float;
   using GV = unsigned short;  // bits of the 16-bit metric value
+  using CV = W;
   static constexpr bool LOWP = true;
   __device__ static __forceinline__ float rnd(float x) {
     if constexpr (W::BF)
@@ -325,20 +420,22 @@ struct NT16 {
   }
 };
 
+// scalar double-word values: single cells of the FP64 apply, and the metric formed on the fly
 template <>
 struct NT<dw> {
   using SV = double;
   using GV = float2;
+  using CV = dw;
   static constexpr bool LOWP = false;
   __device__ static __forceinline__ dw zero() { return {0.0f, 0.0f}; }
-  __device__ static __forceinline__ dw mac(dw a, dw c, dw v) { return dw_mac(a, c, v); }
-  // the 12-operation form, for the geometry terms (their error reaches every output)
-  __device__ static __forceinline__ dw mac12(dw a, dw c, dw v) { return dw_mac12(a, c, v); }
   __device__ static __forceinline__ dw prod(dw c, dw v) { return dw_prod(c, v); }
+  __device__ static __forceinline__ dw mac(dw a, dw c, dw v) { return dw_mac(a, c, v); }
   // unnormalised sums (TwoSum of the high parts, low parts added in float): the error stays at
   // the double-word level of the operands, which is all the following products need
   __device__ static __forceinline__ dw addk(dw a, dw b) { return dw_add_keep(a, b); }
   __device__ static __forceinline__ dw subk(dw a, dw b) { return dw_add_keep(a, {-b.h, -b.l}); }
+  // the 12-operation form, for the geometry terms (their error reaches every output)
+  __device__ static __forceinline__ dw mac12(dw a, dw c, dw v) { return dw_mac12(a, c, v); }
   __device__ static __forceinline__ dw fin(dw a) { return dw_norm(a); }
   // intermediate results of the sweeps stay unnormalised: |lo| stays below a few ulp(hi), and the
   // next products use lo only in FP32 cross terms (relative effect ~2^-45)
@@ -352,20 +449,30 @@ struct NT<dw> {
     const dw e = dw_add({1.0f, 0.0f}, dw_mul(a, {-r0, 0.0f}));
     return dw_add({r0, 0.0f}, dw_mul({r0, 0.0f}, e));
   }
-  __device__ static __forceinline__ dw neg(dw a) { return {-a.h, -a.l}; }
-  __device__ static __forceinline__ dw load(const double* p) { return dw_from_double(__ldg(p)); }
-  __device__ static __forceinline__ dw load_stream(const double* p) { return dw_from_double(__ldcs(p)); }
-  // stores of values computed on inputs scaled by 2^-sh (the CTA's exponent shift)
-  __device__ static __forceinline__ void store(double* p, dw v, int sh = 0) {
-    __stcs(p, dw_to_double_sh(v, sh));
-  }
-  // the stored value (binary64) and its store, for sums formed on stored values
-  __device__ static __forceinline__ double to_sv(dw v, int sh = 0) { return dw_to_double_sh(v, sh); }
-  __device__ static __forceinline__ void store_sv(double* p, double v) { __stcs(p, v); }
   __device__ static __forceinline__ dw geo(const float2* p) {
-    float2 g = __ldcs(p);
+    const float2 g = __ldcs(p);
     return {g.x, g.y};
   }
+};
+// pairs of double-word values (one per cell of a pair); loads and stores belong to the kernel
+template <>
+struct NT<dw2> {
+  using SV = double;
+  using GV = float;
+  using CV = dw2c;
+  static constexpr bool LOWP = false;
+  __device__ static __forceinline__ dw2 zero() { return {0ull, 0ull}; }
+  __device__ static __forceinline__ dw2n prod(dw2c c, dw2 v) { return dw2_prod(c, v); }
+  __device__ static __forceinline__ dw2n mac(dw2n a, dw2c c, dw2 v) { return dw2_mac(a, c, v); }
+  __device__ static __forceinline__ dw2 prod(dw2 c, dw2 v) { return dw2_prod(c, v); }
+  __device__ static __forceinline__ dw2 mac(dw2 a, dw2 c, dw2 v) { return dw2_mac(a, c, v); }
+  __device__ static __forceinline__ dw2 addk(dw2 a, dw2 b) { return dw2_addk(a, b); }
+  __device__ static __forceinline__ dw2 subk(dw2 a, dw2 b) { return dw2_subk(a, b); }
+  __device__ static __forceinline__ dw2 addk(dw2n a, dw2n b) { return dw2_addk(a, b); }
+  __device__ static __forceinline__ dw2 subk(dw2n a, dw2n b) { return dw2_subk(a, b); }
+  __device__ static __forceinline__ dw2 keep(dw2n a) { return {a.h, f2_neg(a.nl)}; }
+  __device__ static __forceinline__ dw2 mul(dw2 a, dw2 b) { return dw2_mul(a, b); }
+  __device__ static __forceinline__ dw2 add(dw2 a, dw2 b) { return dw2_add(a, b); }
 };
 template <>
 struct NT<bfv> : NT16<bfv> {};
@@ -384,12 +491,13 @@ struct NT<hfv> : NT16<hfv> {};
 // multiply-adds of the plain product.
 template <int N, class V>
 struct EO {
+  using C = typename NT<V>::CV;
   static constexpr int H = N / 2;
-  V A[H][H];  // (M[q][r] + M[q][n-1-r]) / 2
-  V B[H][H];  // (M[q][r] - M[q][n-1-r]) / 2
-  V cm[H];    // M[q][mid]   (odd n)
-  V cr[H];    // M[mid][r]   (odd n)
-  V mm;       // M[mid][mid] (odd n, sig = +1)
+  C A[H][H];  // (M[q][r] + M[q][n-1-r]) / 2
+  C B[H][H];  // (M[q][r] - M[q][n-1-r]) / 2
+  C cm[H];    // M[q][mid]   (odd n)
+  C cr[H];    // M[mid][r]   (odd n)
+  C mm;       // M[mid][mid] (odd n, sig = +1)
 };
 
 // Even-odd form of the n x (n-1) matrix B' that maps the n-1 differences d_s = x_{s+1} - x_s of a
@@ -402,10 +510,11 @@ template <int N, class V>
 struct EOB {
   static constexpr int NI = N - 1, HI = NI / 2, HO = N / 2;
   static constexpr int HA = HI > 0 ? HI : 1;
-  V A[HO][HA];
-  V B[HO][HA];
-  V cm[HO];  // B'[q][(n-2)/2]   (even n: the middle difference)
-  V cr[HA];  // B'[(n-1)/2][s]   (odd n: the middle output)
+  using C = typename NT<V>::CV;
+  C A[HO][HA];
+  C B[HO][HA];
+  C cm[HO];  // B'[q][(n-2)/2]   (even n: the middle difference)
+  C cr[HA];  // B'[(n-1)/2][s]   (odd n: the middle output)
 };
 
 template <int N, class V>
@@ -414,5 +523,16 @@ struct Tab1D {
   V D_[N][N];  // D[q][r]  = derivative of the Gauss-point Lagrange basis r at s_q (collocation)
   V W_[N];     // Gauss weights on [0,1]
   EO<N, V> eV, eVT, eD, eDT;  // even-odd forms of V, V^T, D, D^T
-  EOB<N, V> eB;               // even-odd form of B' (derivative from nodal differences)
 };
+
+// the tables of the FP64 apply (pairs and single cells): even-odd forms and weights
+template <int N, class V>
+struct TabDW {
+  V W_[N];
+  EO<N, V> eV, eVT, eDT;
+  EOB<N, V> eB;  // even-odd form of B' (derivative from nodal differences)
+};
+template <int N>
+struct Tab1D<N, dw2> : TabDW<N, dw2> {};
+template <int N>
+struct Tab1D<N, dw> : TabDW<N, dw> {};

@@ -42,14 +42,14 @@ struct AllTabs {
   Tab1D<7, V> t7;
   Tab1D<8, V> t8;
 };
-__constant__ AllTabs<dw> c_tabs_dw;
+__constant__ AllTabs<dw2> c_tabs_dw;
 __constant__ AllTabs<float> c_tabs_f32;
 
 template <int N, class V>
 __device__ __forceinline__ const Tab1D<N, V>& tab_of();
 #define FE_TAB_OF(NN)                                                            \
   template <>                                                                    \
-  __device__ __forceinline__ const Tab1D<NN, dw>& tab_of<NN, dw>() {             \
+  __device__ __forceinline__ const Tab1D<NN, dw2>& tab_of<NN, dw2>() {             \
     return c_tabs_dw.t##NN;                                                      \
   }                                                                              \
   template <>                                                                    \
@@ -72,17 +72,17 @@ fe_status ensure_tables(int dev) {
   std::lock_guard<std::mutex> lock(g_tab_mu);
   if (dev < 0 || dev >= 64) return FE_ERR_INVALID;
   if (g_tab_ready[dev]) return FE_OK;
-  AllTabs<dw> tdw;
+  AllTabs<dw2> tdw;
   AllTabs<float> t32;
   HostTab h[8];
   for (int p = 1; p <= 7; ++p) fe_host_tables(p, &h[p]);
-  tdw.t2 = make_tab<2, dw>(h[1]);
-  tdw.t3 = make_tab<3, dw>(h[2]);
-  tdw.t4 = make_tab<4, dw>(h[3]);
-  tdw.t5 = make_tab<5, dw>(h[4]);
-  tdw.t6 = make_tab<6, dw>(h[5]);
-  tdw.t7 = make_tab<7, dw>(h[6]);
-  tdw.t8 = make_tab<8, dw>(h[7]);
+  tdw.t2 = make_tab<2, dw2>(h[1]);
+  tdw.t3 = make_tab<3, dw2>(h[2]);
+  tdw.t4 = make_tab<4, dw2>(h[3]);
+  tdw.t5 = make_tab<5, dw2>(h[4]);
+  tdw.t6 = make_tab<6, dw2>(h[5]);
+  tdw.t7 = make_tab<7, dw2>(h[6]);
+  tdw.t8 = make_tab<8, dw2>(h[7]);
   t32.t2 = make_tab<2, float>(h[1]);
   t32.t3 = make_tab<3, float>(h[2]);
   t32.t4 = make_tab<4, float>(h[3]);
@@ -133,24 +133,29 @@ __device__ __forceinline__ void apply_item(const BProb& P, int prec, int src, lo
   a.mz = P.mz;
   a.dirichlet = P.dirichlet;
   for (int c = 0; c < 4; ++c) {
-    if constexpr (sizeof(V) == sizeof(dw))
-      a.aff[c] = dw_from_double(P.aff[c]);
-    else
+    if constexpr (std::is_same<V, dw2>::value) {
+      const dw v = dw_from_double(P.aff[c]);
+      a.aff[c] = {f2_pack(v.h, v.h), f2_pack(v.l, v.l)};
+    } else
       a.aff[c] = (V)P.aff[c];
   }
-  constexpr int stride = Cfg<N>::TILE + Cfg<N>::CS;
-  if (P.affine)
-    apply_cells<N, V, FE_LAPLACE, GEOM_AFFINE_K>(a, tab_of<N, V>(), cell0, sm, stride);
-  else
-    apply_cells<N, V, FE_LAPLACE, GEOM_STORED_K>(a, tab_of<N, V>(), cell0, sm, stride);
+  if constexpr (std::is_same<V, dw2>::value) {
+    if (P.affine)
+      apply_pairs<N, FE_LAPLACE, GEOM_AFFINE_K, MODE_CELLS>(a, tab_of<N, V>(), cell0, sm);
+    else
+      apply_pairs<N, FE_LAPLACE, GEOM_STORED_K, MODE_CELLS>(a, tab_of<N, V>(), cell0, sm);
+  } else {
+    if (P.affine)
+      apply_cells<N, V, FE_LAPLACE, GEOM_AFFINE_K>(a, tab_of<N, V>(), cell0, sm, Cfg<N>::TILE);
+    else
+      apply_cells<N, V, FE_LAPLACE, GEOM_STORED_K>(a, tab_of<N, V>(), cell0, sm, Cfg<N>::TILE);
+  }
 }
 
-// register budget of the persistent apply: 3 CTAs per SM for the unrolled double-word degrees, 4
-// for the rolled ones (its CTA is wider than the tile and walks many tiles; the one-layer apply's
-// per-degree budgets were measured on the one-layer kernel)
+// register budget of the persistent apply (FP64: that of the one-layer pair kernel)
 template <int N, class V>
 __host__ __device__ constexpr int batch_minb() {
-  return std::is_same<V, dw>::value ? (N < FE_ROLL_MINN ? 3 : 4) : 1;
+  return std::is_same<V, dw2>::value ? pair_minb<N, FE_LAPLACE, MODE_CELLS>() : 1;
 }
 
 // persistent apply over the tiles [lo, hi) of one degree (tiles are grouped by degree), each kernel
@@ -158,7 +163,7 @@ __host__ __device__ constexpr int batch_minb() {
 // The next work item is claimed before the current tile's apply (its atomic round trip overlaps
 // the apply) and published through a double-buffered shared slot.
 template <int N, class V>
-__global__ void __launch_bounds__(BT, (batch_minb<N, V>()))
+__global__ void __launch_bounds__(Shape<N, V>::THREADS, (batch_minb<N, V>()))
     kb_apply_n(const BProb* __restrict__ probs, const Tile* __restrict__ tiles, long long lo,
                long long hi, int slot, int prec, int src, unsigned long long* counter) {
   extern __shared__ __align__(16) unsigned char sm[];
@@ -179,11 +184,6 @@ __global__ void __launch_bounds__(BT, (batch_minb<N, V>()))
     buf ^= 1;
     it = item[buf];
   }
-}
-
-template <int N, class V>
-constexpr size_t tile_bytes() {
-  return (size_t)apply_narr<V>(FE_LAPLACE) * (Cfg<N>::TILE + Cfg<N>::CS) * Sm<V>::BYTES;
 }
 
 // ---- vector kernels over chunks ----------------------------------------------------------------
@@ -672,27 +672,32 @@ unsigned grid_chunks(int n) { return (unsigned)std::max(1, std::min(n, 152 * 8))
 // ---------------------------------------------------------------------------------------------
 fe_status fe_batch_build(FeBatch* B) {
   const int np = (int)B->hp.size();
-  std::vector<Tile> tiles_n[FE_MAXN + 1];
+  std::vector<Tile> tiles_n[2][FE_MAXN + 1];  // [FP64, FP32]
   std::vector<Chunk> vch;
   std::vector<DssRow> dch[3];
   for (int i = 0; i < np; ++i) {
     BProb& P = B->hp[i];
     const int n = P.n;
-    int cpb = 0;
+    int cpb[2] = {0, 0};  // cells per tile
+    auto shape = [&](auto N) {
+      cpb[0] = Shape<decltype(N)::value, dw2>::CELLS;
+      cpb[1] = Shape<decltype(N)::value, float>::CELLS;
+    };
     switch (n) {
-      case 2: cpb = Cfg<2>::CPB; break;
-      case 3: cpb = Cfg<3>::CPB; break;
-      case 4: cpb = Cfg<4>::CPB; break;
-      case 5: cpb = Cfg<5>::CPB; break;
-      case 6: cpb = Cfg<6>::CPB; break;
-      case 7: cpb = Cfg<7>::CPB; break;
-      case 8: cpb = Cfg<8>::CPB; break;
+      case 2: shape(std::integral_constant<int, 2>()); break;
+      case 3: shape(std::integral_constant<int, 3>()); break;
+      case 4: shape(std::integral_constant<int, 4>()); break;
+      case 5: shape(std::integral_constant<int, 5>()); break;
+      case 6: shape(std::integral_constant<int, 6>()); break;
+      case 7: shape(std::integral_constant<int, 7>()); break;
+      case 8: shape(std::integral_constant<int, 8>()); break;
     }
     if (!B->active[i]) {
       P.chunk0 = P.chunk1 = (int)vch.size();
       continue;
     }
-    for (long long c = 0; c < P.ncells; c += cpb) tiles_n[n].push_back({i, 0, c});
+    for (int f = 0; f < 2; ++f)
+      for (long long c = 0; c < P.ncells; c += cpb[f]) tiles_n[f][n].push_back({i, 0, c});
     P.chunk0 = (int)vch.size();
     for (long long e = 0; e < P.ncw; e += CHUNK) vch.push_back({i, 0, e, std::min(P.ncw, e + CHUNK)});
     P.chunk1 = (int)vch.size();
@@ -703,11 +708,12 @@ fe_status fe_batch_build(FeBatch* B) {
   }
   // tiles grouped by degree: one persistent apply launch per degree present
   std::vector<Tile> tiles;
-  for (int nn = 0; nn <= FE_MAXN; ++nn) {
-    B->tile_lo[nn] = (long long)tiles.size();
-    tiles.insert(tiles.end(), tiles_n[nn].begin(), tiles_n[nn].end());
-    B->tile_hi[nn] = (long long)tiles.size();
-  }
+  for (int f = 0; f < 2; ++f)
+    for (int nn = 0; nn <= FE_MAXN; ++nn) {
+      B->tile_lo[f][nn] = (long long)tiles.size();
+      tiles.insert(tiles.end(), tiles_n[f][nn].begin(), tiles_n[f][nn].end());
+      B->tile_hi[f][nn] = (long long)tiles.size();
+    }
   B->ntiles = (long long)tiles.size();
   B->nvch = (int)vch.size();
   for (int a = 0; a < 3; ++a) B->ndch[a] = (int)dch[a].size();
@@ -748,9 +754,11 @@ fe_status fe_batch_build(FeBatch* B) {
 
 template <int N, class V>
 static fe_status launch_apply_degree(FeBatch* B, int slot, int src) {
-  const long long lo = B->tile_lo[N], hi = B->tile_hi[N];
+  constexpr int f = std::is_same<V, dw2>::value ? 0 : 1;
+  const long long lo = B->tile_lo[f][N], hi = B->tile_hi[f][N];
   if (hi <= lo) return FE_OK;
-  const size_t smem = tile_bytes<N, V>();
+  using Sh = Shape<N, V>;
+  const size_t smem = Sh::smem(FE_LAPLACE);
   static int per_sm_dev[64] = {};  // resident CTAs per SM, per device (attribute set once)
   int dev = 0;
   FE_CUDA(cudaGetDevice(&dev), "cudaGetDevice");
@@ -759,21 +767,21 @@ static fe_status launch_apply_degree(FeBatch* B, int slot, int src) {
     FE_CUDA(cudaFuncSetAttribute(kb_apply_n<N, V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)smem),
             "batch apply attribute");
-    FE_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kb_apply_n<N, V>, BT, smem),
+    FE_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kb_apply_n<N, V>, Sh::THREADS, smem),
             "occupancy");
     per_sm = std::max(1, per_sm);
     if (dev >= 0 && dev < 64) per_sm_dev[dev] = per_sm;
   }
   const long long grid = std::min<long long>(hi - lo, 152LL * per_sm);
-  kb_apply_n<N, V><<<(unsigned)grid, BT, smem, B->st>>>(
-      B->d_probs, (const Tile*)B->d_tiles, lo, hi, slot, std::is_same<V, dw>::value ? FE_F64 : FE_F32,
+  kb_apply_n<N, V><<<(unsigned)grid, Sh::THREADS, smem, B->st>>>(
+      B->d_probs, (const Tile*)B->d_tiles, lo, hi, slot, f == 0 ? FE_F64 : FE_F32,
       src, B->d_counter + N);
   return fe_cuda_check(cudaGetLastError(), "batch apply launch");
 }
 
 template <class S>
 static fe_status launch_apply_batched(FeBatch* B, int slot, int src = 0) {
-  using V = typename std::conditional<sizeof(S) == 8, dw, float>::type;
+  using V = typename std::conditional<sizeof(S) == 8, dw2, float>::type;
   FE_CUDA(cudaMemsetAsync(B->d_counter, 0, (FE_MAXN + 1) * sizeof(unsigned long long), B->st),
           "counter reset");
   FE_TRY((launch_apply_degree<2, V>(B, slot, src)));

@@ -10,7 +10,7 @@ struct BProb {
   long long ncells, ncw;
   int mx, my, mz, dirichlet;
   double aff[4];  // affine metric constants detJ/h_x^2, detJ/h_y^2, detJ/h_z^2, detJ
-  const float2* geodw;
+  const float* geodw;
   const float* geo32;
   double *x64, *r64, *z64, *p64, *q64, *w64;
   const double* b64;
@@ -33,7 +33,7 @@ struct FeBatch {
   void* d_tiles = nullptr;
   size_t cap_tiles = 0;
   long long ntiles = 0;
-  long long tile_lo[FE_MAXN + 1] = {}, tile_hi[FE_MAXN + 1] = {};  // tiles of each degree n
+  long long tile_lo[2][FE_MAXN + 1] = {}, tile_hi[2][FE_MAXN + 1] = {};  // tiles of each degree n
   void* d_vch = nullptr;
   size_t cap_vch = 0;
   int nvch = 0;

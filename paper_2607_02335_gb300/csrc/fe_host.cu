@@ -138,7 +138,7 @@ void make_view(const fe_mesh* m, int z0, int z1, fe_mesh* v) {
   v->nbr_lo = m->nbr_lo || z0 > 0;
   v->nbr_hi = m->nbr_hi || z1 < m->d.mz;
   v->geo64 = m->geo64 ? m->geo64 + goff : nullptr;
-  v->geodw = m->geodw ? m->geodw + goff : nullptr;
+  v->geodw = m->geodw ? m->geodw + 2 * goff : nullptr;
   v->geo32 = m->geo32 ? m->geo32 + goff : nullptr;
   for (int k = 0; k < 2; ++k) v->geo16[k] = m->geo16[k] ? m->geo16[k] + goff : nullptr;
   v->xyz64 = nullptr;

@@ -49,9 +49,10 @@ struct fe_mesh {
   int p, n, n3;
   long long ncells, ncw, nu;
   HostTab tab;
-  // stored geometry [cell][FE_GEO_COMPS][n3] (FP64, double-word, FP32 copies)
+  // stored geometry [cell][FE_GEO_COMPS][n3] (FP64 and FP32 copies; the double-word copy holds a
+  // plane of n3 high parts and one of n3 low parts per component)
   double* geo64 = nullptr;
-  float2* geodw = nullptr;
+  float* geodw = nullptr;
   float* geo32 = nullptr;
   unsigned short* geo16[2] = {nullptr, nullptr};  // bf16 / fp16 metric, scaled by gscale[op]
   float gscale[2] = {1.0f, 1.0f};                 // powers of two: Laplace terms, w detJ

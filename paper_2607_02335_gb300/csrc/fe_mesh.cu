@@ -252,6 +252,19 @@ __global__ void k_split_dw(const double* __restrict__ in, float2* __restrict__ o
     out[e] = make_float2(h, __double2float_rn(v - (double)h));
   }
 }
+// the same into planes: each run of n3 values becomes n3 high parts and then n3 low parts (the
+// pair kernel loads the parts of two cells into register pairs, with coalesced 32-bit loads)
+__global__ void k_split_dw_planes(const double* __restrict__ in, float* __restrict__ out, long long n,
+                                  int n3) {
+  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n;
+       e += (long long)gridDim.x * blockDim.x) {
+    const double v = in[e];
+    const float h = __double2float_rn(v);
+    float* o = out + e + e / n3 * n3;
+    o[0] = h;
+    o[n3] = __double2float_rn(v - (double)h);
+  }
+}
 __global__ void k_to_f32(const double* __restrict__ in, float* __restrict__ out, long long n) {
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n;
        e += (long long)gridDim.x * blockDim.x)
@@ -361,8 +374,8 @@ fe_status fe_ensure_geometry(const fe_mesh* cm, int prec, bool native) {
   }
   if (prec == FE_F64 && !native) {
     if (!m->geodw) {
-      FE_TRY(fe_dalloc((void**)&m->geodw, n * sizeof(float2), m->st, "geometry (double-word)"));
-      k_split_dw<<<grid_for(n, 256), 256, 0, m->st>>>(m->geo64, m->geodw, n);
+      FE_TRY(fe_dalloc((void**)&m->geodw, 2 * n * sizeof(float), m->st, "geometry (double-word)"));
+      k_split_dw_planes<<<grid_for(n, 256), 256, 0, m->st>>>(m->geo64, m->geodw, n, m->n3);
       FE_CUDA(cudaStreamSynchronize(m->st), "geometry double-word split");
     }
   } else if (prec == FE_F32) {

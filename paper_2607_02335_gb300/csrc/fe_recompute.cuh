@@ -24,17 +24,42 @@ struct GeoCfg {
 };
 
 template <int N, class V>
+struct RecomputeTab {  // the full matrices of Tab1D
+  V V_[N][N], D_[N][N], W_[N];
+};
+template <int N, class V>
 struct RecomputeArgs {
   const typename NT<V>::GV* xyz;  // [cell][3][N3] offsets from the cell's first node
   typename NT<V>::GV* geo;        // [cell - cell0][7][N3]
   long long cell0, cell_end;
   const int* skip;
-  Tab1D<N, V> tab;
+  RecomputeTab<N, V> tab;
 };
 
-__device__ __forceinline__ void geo_put(float2* p, dw v) { *p = make_float2(v.h, v.l); }
-__device__ __forceinline__ void geo_put(double* p, double v) { *p = v; }
-__device__ __forceinline__ void geo_put(float* p, float v) { *p = v; }
+// component c of point t of one cell's metric; double-word values go to the planes of high and low
+// parts that the pair kernel reads
+template <int N3>
+__device__ __forceinline__ void geo_put(float2* cell, int c, int t, dw v) {
+  float* p = reinterpret_cast<float*>(cell) + c * 2 * N3 + t;
+  p[0] = v.h;
+  p[N3] = v.l;
+}
+template <int N3, class S>
+__device__ __forceinline__ void geo_put(S* cell, int c, int t, S v) {
+  cell[c * N3 + t] = v;
+}
+
+// value type in which the metric of an apply in arithmetic V is formed, and its coordinates' type
+template <class V>
+struct RV {
+  using T = V;
+  using GV = typename NT<V>::GV;
+};
+template <>
+struct RV<dw2> {
+  using T = dw;
+  using GV = float2;
+};
 
 template <int N, class V>
 constexpr size_t recompute_smem_bytes() {
@@ -110,9 +135,9 @@ __global__ void __launch_bounds__(GeoCfg<N>::THREADS)
   const V A20 = dp(J[1][0], J[2][1], J[1][1], J[2][0]);
   const V det = T::add(T::add(T::mul(J[0][0], A00), T::mul(J[0][1], A10)), T::mul(J[0][2], A20));
   const V w3 = T::mul(T::mul(a.tab.W_[i], a.tab.W_[j]), a.tab.W_[k]);
-  typename NT<V>::GV* out = a.geo + (size_t)(cell - a.cell0) * (FE_GEO_COMPS * N3) + t;
+  typename NT<V>::GV* out = a.geo + (size_t)(cell - a.cell0) * (FE_GEO_COMPS * N3);
   if constexpr (OP == FE_MASS) {
-    geo_put(out + 6 * N3, T::mul(w3, det));
+    geo_put<N3>(out, 6, t, T::mul(w3, det));
   } else {
     // G = w detJ J^-1 J^-T = (w / detJ) adj(J) adj(J)^T
     const V A01 = dp(J[0][2], J[2][1], J[0][1], J[2][2]);
@@ -125,11 +150,11 @@ __global__ void __launch_bounds__(GeoCfg<N>::THREADS)
     auto row = [&](V p0, V p1, V p2, V q0, V q1, V q2) {
       return T::mul(sc, T::add(T::add(T::mul(p0, q0), T::mul(p1, q1)), T::mul(p2, q2)));
     };
-    geo_put(out + 0 * N3, row(A00, A01, A02, A00, A01, A02));
-    geo_put(out + 1 * N3, row(A10, A11, A12, A10, A11, A12));
-    geo_put(out + 2 * N3, row(A20, A21, A22, A20, A21, A22));
-    geo_put(out + 3 * N3, row(A00, A01, A02, A10, A11, A12));
-    geo_put(out + 4 * N3, row(A00, A01, A02, A20, A21, A22));
-    geo_put(out + 5 * N3, row(A10, A11, A12, A20, A21, A22));
+    geo_put<N3>(out, 0, t, row(A00, A01, A02, A00, A01, A02));
+    geo_put<N3>(out, 1, t, row(A10, A11, A12, A10, A11, A12));
+    geo_put<N3>(out, 2, t, row(A20, A21, A22, A20, A21, A22));
+    geo_put<N3>(out, 3, t, row(A00, A01, A02, A10, A11, A12));
+    geo_put<N3>(out, 4, t, row(A00, A01, A02, A20, A21, A22));
+    geo_put<N3>(out, 5, t, row(A10, A11, A12, A20, A21, A22));
   }
 }
