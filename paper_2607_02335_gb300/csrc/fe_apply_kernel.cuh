@@ -28,6 +28,7 @@
 #include <type_traits>
 
 #include "fe_internal.h"
+#include "fe_reduce.cuh"
 
 template <int N>
 struct Cfg {
@@ -219,6 +220,7 @@ struct ApplyArgs {
   CellArgs<N, V> c;
   const int* skip;  // optional device flag: the whole launch returns at once when *skip != 0
   int zchunk;       // MODE_BRICKZ: z-layers per CTA
+  CgApply cg;       // cg.sc: the fused CG iteration (MODE_CELLS, Laplace)
   Tab1D<N, V> tab;
 };
 
@@ -533,11 +535,12 @@ __device__ __forceinline__ void apply_cells_rolled(const CellArgs<N, V>& a, cons
 }
 
 // The cells cell0 .. cell0 + CPB - 1 (those below ncells), applied by the CTA's CPB*n^2 threads.
-template <int N, class V, int OP, int GEOM, int MODE = MODE_CELLS>
+template <int N, class V, int OP, int GEOM, int MODE = MODE_CELLS, bool CG = false>
 __device__ __forceinline__ void apply_cells(const CellArgs<N, V>& a, const Tab1D<N, V>& tab,
                                             long long cell0, unsigned char* smraw,
                                             int tile_stride,
-                                            ZCarry<typename NT<V>::SV>* zc = nullptr) {
+                                            ZCarry<typename NT<V>::SV>* zc = nullptr,
+                                            const CgApply* cg = nullptr) {
   static_assert(MODE != MODE_PACKED || N < FE_ROLL_MINN, "packed units: unrolled degrees only");
   static_assert(MODE != MODE_BRICKZ || (N < FE_ROLL_MINN && !NT<V>::LOWP),
                 "z-carry bricks: unrolled degrees, FP64 / FP32 values");
@@ -589,10 +592,24 @@ __device__ __forceinline__ void apply_cells(const CellArgs<N, V>& a, const Tab1D
     }
   };
   V u[N], w[N];
+  if constexpr (CG) {  // fused CG iteration (FP32): p := z + beta p on the way in
+    const float beta = (float)cg->sc->beta;
+    const float* z = static_cast<const float*>(cg->z);
+    float* p = const_cast<float*>(a.x);
 #pragma unroll
-  for (int k = 0; k < N; ++k) {
-    V v = active ? T::load_stream(a.x + xaddr(k)) : T::zero();
-    u[k] = masked(k) ? T::zero() : v;
+    for (int k = 0; k < N; ++k) w[k] = active ? p[xaddr(k)] : 0.0f, u[k] = active ? z[xaddr(k)] : 0.0f;
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      u[k] = u[k] + beta * w[k];
+      if (active) p[xaddr(k)] = u[k];
+      if (masked(k)) u[k] = 0.0f;
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      V v = active ? T::load_stream(a.x + xaddr(k)) : T::zero();
+      u[k] = masked(k) ? T::zero() : v;
+    }
   }
   // low degrees: issue the metric loads now so that their latency hides behind the sweeps
 #ifndef FE_PREFETCH_MAXN
@@ -794,6 +811,7 @@ __device__ __forceinline__ void apply_cells(const CellArgs<N, V>& a, const Tab1D
     }
     return;
   }
+  Acc<float> qp;
   if (active) {
 #pragma unroll
     for (int k = 0; k < N; ++k) {
@@ -801,21 +819,22 @@ __device__ __forceinline__ void apply_cells(const CellArgs<N, V>& a, const Tab1D
       if (masked(k)) v = T::zero();
       if constexpr (T::LOWP) v.v *= a.oscale;
       T::store(a.y + gbase + k * N2 + lt, v);
+      if constexpr (CG) qp.add_prod(v, *(volatile const float*)(a.x + gbase + k * N2 + lt));
     }
   }
+  if constexpr (CG) cg_finish_apply(*cg, qp);
 }
 
-// z-carry bricks: held to a register budget for 3 CTAs per SM (Laplace, as the one-layer brick
-// kernel; left to itself the compiler gives the layer loop 98 registers, 2 CTAs per SM) or 6
-// (mass, whose one-layer kernel needs 32 registers)
-#ifndef FE_ZCARRY_MINB_LAPLACE
-#define FE_ZCARRY_MINB_LAPLACE 3
-#endif
-#ifndef FE_ZCARRY_MINB_MASS
-#define FE_ZCARRY_MINB_MASS 6
-#endif
-template <int N, class V, int OP, int GEOM, int MODE>
-__global__ void __launch_bounds__(Cfg<N>::THREADS) k_apply(const __grid_constant__ ApplyArgs<N, V> a) {
+// Z-carry bricks: register budgets of 3 (FP64 Laplace), 4 (FP32 Laplace: 64 registers; at 3 the
+// compiler takes 69, and a Q3 64^3 assembled apply 152 us instead of 142) or 6 (mass) CTAs per SM.
+template <class V, int OP>
+__host__ __device__ constexpr int zcarry_minb() {
+  return OP == FE_MASS ? 6 : std::is_same<V, float>::value ? 4 : 3;
+}
+// (one CTA per SM asked for: left to itself the compiler holds the FP32 kernels to 32-40 registers for
+// occupancy, and Q7 32^3 Laplace takes 123 us instead of 115)
+template <int N, class V, int OP, int GEOM, int MODE, bool CG>
+__global__ void __launch_bounds__(Cfg<N>::THREADS, 1) k_apply(const __grid_constant__ ApplyArgs<N, V> a) {
   extern __shared__ __align__(16) unsigned char smraw[];
   if (a.skip && *(volatile const int*)a.skip) return;  // uniform over the grid
   long long cell0;
@@ -825,14 +844,14 @@ __global__ void __launch_bounds__(Cfg<N>::THREADS) k_apply(const __grid_constant
     cell0 = (long long)blockIdx.x * Packed<N>::UPB;
   else
     cell0 = a.c.cell_base + (long long)blockIdx.x * Cfg<N>::CPB;
-  apply_cells<N, V, OP, GEOM, MODE>(a.c, a.tab, cell0, smraw, Cfg<N>::TILE);
+  apply_cells<N, V, OP, GEOM, MODE, CG>(a.c, a.tab, cell0, smraw, Cfg<N>::TILE, nullptr, &a.cg);
 }
 
 // MODE_BRICKZ: blockIdx.x = chunk * (bricks per layer) + brick column; the CTA applies the layers
 // [z0, z1) of its column one after the other
 template <int N, class V, int OP, int GEOM>
 __global__ void __launch_bounds__(Cfg<N>::THREADS,
-                                  OP == FE_LAPLACE ? FE_ZCARRY_MINB_LAPLACE : FE_ZCARRY_MINB_MASS)
+                                  (zcarry_minb<V, OP>()))
     k_apply_zcarry(const __grid_constant__ ApplyArgs<N, V> a) {
   extern __shared__ __align__(16) unsigned char smraw[];
   if (a.skip && *(volatile const int*)a.skip) return;  // uniform over the grid

@@ -114,12 +114,12 @@ struct Shape {
   using B = Brick<N>;
   static constexpr int BRICK_THREADS = B::BX * B::BY * Cfg<N>::N2;
   static size_t smem(int op) { return apply_smem_bytes<N, V>(op); }
-  template <int OP, int GEOM, int MODE>
+  template <int OP, int GEOM, int MODE, bool CG = false>
   static auto kernel() {
     if constexpr (MODE == MODE_BRICKZ)
       return k_apply_zcarry<N, V, OP, GEOM>;
     else
-      return k_apply<N, V, OP, GEOM, MODE>;
+      return k_apply<N, V, OP, GEOM, MODE, CG>;
   }
 };
 template <int N, int SHAPE>
@@ -129,12 +129,12 @@ struct PairShape {
   using B = PairBrick<(N <= 4 ? N : 4)>;  // bricks up to n = 4 only
   static constexpr int BRICK_THREADS = C::THREADS;
   static size_t smem(int op) { return pair_smem_bytes<N, SHAPE>(op); }
-  template <int OP, int GEOM, int MODE>
+  template <int OP, int GEOM, int MODE, bool CG = false>
   static auto kernel() {
     if constexpr (MODE == MODE_BRICKZ)
       return k_apply_pair_zcarry<N, OP, GEOM>;
     else
-      return k_apply_pair<N, OP, GEOM, MODE, SHAPE>;
+      return k_apply_pair<N, OP, GEOM, MODE, SHAPE, CG>;
   }
 };
 template <int N>
@@ -152,10 +152,16 @@ inline int fe_sm_count() {  // of the current device
   return cached[dev] > 0 ? cached[dev] : 1;
 }
 
-template <int N, class V, int OP, int GEOM, int MODE, class Sh>
+template <int N, class V, int OP, int GEOM, int MODE, class Sh, bool CG = false>
 static fe_status launch_shape(const ApplyArgs<N, V>& a, cudaStream_t st) {
+  // the fused CG iteration is an instantiation of its own: its loads and sums take registers
+  if constexpr (!CG && OP == FE_LAPLACE && MODE == MODE_CELLS &&
+                (std::is_same<V, float>::value || std::is_same<V, dw>::value ||
+                 std::is_same<V, dw2>::value)) {
+    if (a.cg.sc) return launch_shape<N, V, OP, GEOM, MODE, Sh, true>(a, st);
+  }
   const size_t smem = Sh::smem(OP);
-  auto kern = Sh::template kernel<OP, GEOM, MODE>();
+  auto kern = Sh::template kernel<OP, GEOM, MODE, CG>();
   static bool attr_done[64] = {};  // one attribute call per instantiation and device
   int dev = 0;
   FE_CUDA(cudaGetDevice(&dev), "cudaGetDevice");
@@ -331,6 +337,7 @@ static void fill_args(ApplyArgs<N, V>& a, const ApplyLaunch& L, const void* geo)
   a.c.mz = m->d.mz;
   a.c.dirichlet = fe_dir_mask(m);
   a.skip = L.skip;
+  if (L.cg) a.cg = *L.cg;
   const double hx = 1.0 / m->d.mx, hy = 1.0 / m->d.my, hz = 1.0 / fe_mz_global(m),
                det = hx * hy * hz;
   a.c.aff[0] = fe_cast<V>(det / (hx * hx));

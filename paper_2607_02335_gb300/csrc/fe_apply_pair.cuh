@@ -376,11 +376,11 @@ __device__ __forceinline__ void pair_sweep(const Sm<V>& s, int base, int st, con
 }
 
 // The tile at cell0, applied by the CTA's PairCfg<N>::THREADS threads.
-template <int N, int OP, int GEOM, int MODE, int SHAPE = TILE_PAIRS>
+template <int N, int OP, int GEOM, int MODE, int SHAPE = TILE_PAIRS, bool CG = false>
 __device__ __forceinline__ void apply_pairs(const CellArgs<N, typename PairCfg<N, SHAPE>::V>& a,
                                             const Tab1D<N, typename PairCfg<N, SHAPE>::V>& tab,
                                             long long cell0, unsigned char* smraw,
-                                            ZCarry2* zc = nullptr) {
+                                            ZCarry2* zc = nullptr, const CgApply* cg = nullptr) {
   static_assert(SHAPE != TILE_SINGLE || MODE == MODE_CELLS, "single cells: consecutive cells only");
   using C = PairCfg<N, SHAPE>;
   using V = typename C::V;
@@ -447,9 +447,21 @@ __device__ __forceinline__ void apply_pairs(const CellArgs<N, typename PairCfg<N
 #pragma unroll
   for (int c = 0; c < W; ++c)
 #pragma unroll
-    for (int k = 0; k < N; ++k) {
+    for (int k = 0; k < N; ++k)
       xr[c][k] = act[c] && !masked(c, k) ? __ldcs(a.x + xaddr(c, k)) : 0.0;
-    }
+  if constexpr (CG) {  // fused CG iteration: p := z + beta p on the way in (0 at masked nodes)
+    const double beta = cg->sc->beta;
+    const double* z = static_cast<const double*>(cg->z);
+    double* p = const_cast<double*>(a.x);
+#pragma unroll
+    for (int c = 0; c < W; ++c)
+#pragma unroll
+      for (int k = 0; k < N; ++k)
+        if (act[c] && !masked(c, k)) {
+          xr[c][k] = z[xaddr(c, k)] + beta * xr[c][k];
+          p[xaddr(c, k)] = xr[c][k];
+        }
+  }
 
   // metric of component comp at point k of the z-lines: planes of high and of low parts per cell; a
   // cell that does not exist reads the tile's first one (its values multiply zeros)
@@ -730,19 +742,26 @@ __device__ __forceinline__ void apply_pairs(const CellArgs<N, typename PairCfg<N
     }
     return;
   }
+  Acc<double> qp;
 #pragma unroll 1
   for (int k = 0; k < N; ++k) {
     const V v = s0.get(bz + k * PS);
 #pragma unroll
-    for (int c = 0; c < W; ++c)
-      if (act[c]) __stcs(a.y + cell[c] * N3 + lt + k * N2, out(v, c, k));
+    for (int c = 0; c < W; ++c) {
+      if (!act[c]) continue;
+      const long long e = cell[c] * N3 + lt + k * N2;
+      const double q = out(v, c, k);
+      __stcs(a.y + e, q);
+      if constexpr (CG) qp.add_prod(q, *(volatile const double*)(a.x + e));
+    }
   }
+  if constexpr (CG) cg_finish_apply(*cg, qp);
 }
 
-template <int N, int OP, int GEOM, int MODE, int SHAPE>
+template <int N, int OP, int GEOM, int MODE, int SHAPE, bool CG>
 __global__ void __launch_bounds__(PairCfg<N, SHAPE>::THREADS,
                                   (SHAPE == TILE_PAIRS
-                                       ? pair_minb<N, OP, MODE>()
+                                       ? (CG && N <= 4 ? 4 : pair_minb<N, OP, MODE>())
                                        : 512 / ((PairCfg<N, SHAPE>::THREADS + 31) / 32 * 32)))
     k_apply_pair(const __grid_constant__ ApplyArgs<N, typename PairCfg<N, SHAPE>::V> a) {
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -754,7 +773,7 @@ __global__ void __launch_bounds__(PairCfg<N, SHAPE>::THREADS,
     cell0 = (long long)blockIdx.x * PairCfg<N>::UPB;
   else
     cell0 = a.c.cell_base + (long long)blockIdx.x * PairCfg<N, SHAPE>::CELLS;
-  apply_pairs<N, OP, GEOM, MODE, SHAPE>(a.c, a.tab, cell0, smraw);
+  apply_pairs<N, OP, GEOM, MODE, SHAPE, CG>(a.c, a.tab, cell0, smraw, nullptr, &a.cg);
 }
 
 // Tile shape of a launch on consecutive cells.  A lone warp on a scheduler runs the packed
@@ -763,11 +782,12 @@ __global__ void __launch_bounds__(PairCfg<N, SHAPE>::THREADS,
 // single against pairs: n = 8 16.2 against 18.7 us, n = 6 12.1 against 13.2, n = 4 7.0 against 7.3;
 // 12^3 cells, 37 warps per SM, n = 7: 32.5 against 29.1).  Above, the small pair tile where the busiest
 // of the SMs has fewer warps to work through with it, in a launch of at most four ordinary CTAs per SM.
+inline bool pair_single(long long cells, int n, int sms) { return cells * n * n <= 16LL * 32 * sms; }
 template <int N>
 inline int pair_shape(long long cells, int sms) {
   using L = PairCfg<N>;
   using S = PairCfg<N, TILE_PAIRS_SMALL>;
-  if (cells * L::N2 <= 16LL * 32 * sms) return TILE_SINGLE;
+  if (pair_single(cells, N, sms)) return TILE_SINGLE;
   const long long pairs = (cells + 1) / 2;
   auto busiest = [&](int np, int threads) {
     return ((pairs + np - 1) / np + sms - 1) / sms * ((threads + 31) / 32);

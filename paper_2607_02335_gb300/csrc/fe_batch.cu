@@ -587,7 +587,9 @@ __global__ void __launch_bounds__(BT)
   const double rz = (mode == FIN_INIT_R || mode == FIN_ITER) ? sum_chunks(partials, P.chunk0, P.chunk1, 1, sh) : 0.0;
   const double qz = (mode == FIN_ITER && flexible) ? sum_chunks(partials, P.chunk0, P.chunk1, 2, sh) : 0.0;
   if (threadIdx.x != 0) return;
-  fin_scalars(sc, rn2, rz, qz, rtol, mode, flexible);
+  const double rel = mode == FIN_INIT_B ? 0.0 : fin_rel(sc, rn2);
+  const double beta = mode == FIN_ITER ? fin_new_beta(sc, rz, qz, flexible) : 0.0;
+  fin_scalars(sc, rn2, rz, rel, beta, rtol, mode);
 }
 
 // reset the inner scalars for a new inner solve (done mirrors the outer state)

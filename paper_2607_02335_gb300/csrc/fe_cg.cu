@@ -6,10 +6,11 @@
 // one dual and one primal vector (Lemma "Duality Pairing Identity"), so the iterates equal those
 // of CG on the assembled system (Theorem "Equivalence of Communication-Free FCG").
 //
-// One iteration is a fixed launch sequence captured once into a CUDA graph:
-//   q = A p;  <q,p> -> alpha;  u += alpha p, r -= alpha q;  w = S r;
-//   z = D^{-1} w (0 on Dirichlet nodes) with sum w^2/mult, <r,z> (and <q,z> for FCG) -> beta;
-//   p = z + beta p.
+// One iteration is a fixed launch sequence, captured into a CUDA graph of GRAPH_ITERS iterations:
+//   p = z + beta p, q = A p, <q,p> -> alpha (one kernel where the operator takes it, CgApply);
+//   u += alpha p, r -= alpha q;
+//   w = S r, z = D^{-1} w (0 on Dirichlet nodes) with sum w^2/mult, <r,z> (and <q,z> for FCG) -> beta.
+// The scalars of a pairing are finished by the last CTA of its kernel.
 // alpha, beta, the residual and the stop flag stay in device memory; every kernel returns at once
 // when the flag is set, so the host replays the graph several times between two reads of the flag.
 // Convergence (unspecified in the paper): ||G^T r||_2 / ||G^T b||_2 <= rtol over free nodes, with
@@ -179,14 +180,6 @@ __global__ void k_update_ur<float, float>(float* __restrict__ u, float* __restri
   for (; e < n; e += stride) step(e, u[e], p[e], q[e], r[e]);
 }
 
-// p = z + c p (host scalar): the search direction kept across a reliable update
-__global__ void k_keep_direction(float* __restrict__ p, const float* __restrict__ z, float c,
-                                 long long n) {
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n;
-       e += (long long)gridDim.x * blockDim.x)
-    p[e] = fmaf(c, p[e], z[e]);
-}
-
 // p = z + beta p (stream_u elements' loads in flight per thread, on a resident grid)
 template <class S>
 __global__ void k_update_p(S* __restrict__ p, const S* __restrict__ z, const CgScal* __restrict__ sc,
@@ -206,53 +199,61 @@ __global__ void k_update_p(S* __restrict__ p, const S* __restrict__ z, const CgS
   for (; e < n; e += stride) p[e] = z[e] + b * p[e];
 }
 
-template <class S>
-__device__ __forceinline__ dw prod_dw(S a, S b);
-template <>
-__device__ __forceinline__ dw prod_dw<double>(double a, double b) {
-  return dw_mul(dw_from_double(a), dw_from_double(b));
-}
-template <>
-__device__ __forceinline__ dw prod_dw<float>(float a, float b) {
-  const float p = __fmul_rn(a, b);
-  return {p, __fmaf_rn(a, b, -p)};
-}
-
-// A thread's running sum of products in a pairing: float vectors in double-word (exact products);
-// double vectors in binary64 FMAs on the FP64 pipe, one per product, which costs less than
-// converting both factors to double-word (the conversions were the kernels' issue bound)
-template <class S>
-struct Acc;
-template <>
-struct Acc<float> {
-  dw v = {0.0f, 0.0f};
-  __device__ __forceinline__ void add_prod(float a, float b) { v = dw_add(v, prod_dw<float>(a, b)); }
-  __device__ __forceinline__ dw value() const { return v; }
-};
-template <>
-struct Acc<double> {
-  double v = 0.0;
-  __device__ __forceinline__ void add_prod(double a, double b) { v = fma(a, b, v); }
-  __device__ __forceinline__ dw value() const { return dw_from_double(v); }
-};
 // double-word for both: the preconditioner kernel already spends its FP64-pipe share on z = w /
 // diag (measured: binary64 FMAs for <r,z> there made it slower, 165 -> 202 us at Q3 64^3)
 template <class S>
 struct AccDw {
   dw v = {0.0f, 0.0f};
-  __device__ __forceinline__ void add_prod(S a, S b) { v = dw_add(v, prod_dw<S>(a, b)); }
+  __device__ __forceinline__ void add_prod(S a, S b) { v = dw_add(v, prod_dw(a, b)); }
   __device__ __forceinline__ dw value() const { return v; }
 };
 
-// partial of <q, p>  (slot 0)
+// residual norm, convergence test and beta
+struct FinBeta {
+  double rtol;  // negative: sc->rtol
+  int mode, flexible;
+  double* hist;
+};
+// by one CTA; the two divisions and the square root, long on the FP64 pipe, in two warps
+__device__ void fin_beta(const double* partials, int nparts, CgScal* sc, const FinBeta& f, double* sh) {
+  __shared__ double rel;
+  double v[3] = {0.0, 0.0, 0.0};
+  if (f.mode == FIN_ITER && f.flexible) {
+    sum_slots<3>(partials, nparts, RED_BLOCKS, v, sh);
+  } else if (f.mode == FIN_INIT_R || f.mode == FIN_ITER) {
+    double t[2];
+    sum_slots<2>(partials, nparts, RED_BLOCKS, t, sh);
+    v[0] = t[0], v[1] = t[1];
+  } else {
+    double t[1];
+    sum_slots<1>(partials, nparts, RED_BLOCKS, t, sh);
+    v[0] = t[0];
+  }
+  if (threadIdx.x == 0) sh[0] = v[0];
+  __syncthreads();
+  if (threadIdx.x == 32 && f.mode != FIN_INIT_B) rel = fin_rel(sc, sh[0]);
+  const double beta =
+      threadIdx.x == 0 && f.mode == FIN_ITER ? fin_new_beta(sc, v[1], v[2], f.flexible) : 0.0;
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  const int k = sc->iter;
+  if (f.mode == FIN_INIT_R) sc->beta = 0.0;  // the first direction is z
+  fin_scalars(sc, v[0], v[1], rel, beta, f.rtol < 0.0 ? sc->rtol : f.rtol, f.mode);
+  if (f.hist && f.mode == FIN_ITER) {
+    f.hist[3 * k + 2] = sc->relres;
+    if (!sc->done) f.hist[3 * k + 1] = sc->beta;
+  }
+}
+
+// <q, p> (slot 0) and alpha
 template <class S>
 __global__ void __launch_bounds__(RED_THREADS)
-    k_qp(const S* __restrict__ q, const S* __restrict__ p, double* __restrict__ partials,
-         const CgScal* __restrict__ sc, long long n) {
+    k_qp(const S* __restrict__ q, const S* __restrict__ p, double* partials, unsigned* count,
+         CgScal* sc, long long n, double* hist) {
   if (*(volatile const int*)&sc->done) return;
-  __shared__ dw sh[32];
+  __shared__ double sh[SUM_THREADS];
   Acc<S> acc;
-  constexpr long long STRIDE = (long long)RED_BLOCKS * RED_THREADS;
+  const long long STRIDE = (long long)gridDim.x * RED_THREADS;
   constexpr int QU = stream_u<S>();
   long long e = (long long)blockIdx.x * RED_THREADS + threadIdx.x;
   // QU elements' loads in flight before their products join the accumulator, in the same order
@@ -267,26 +268,34 @@ __global__ void __launch_bounds__(RED_THREADS)
     for (int u = 0; u < QU; ++u) acc.add_prod(qv[u], pv[u]);
   }
   for (; e < n; e += STRIDE) acc.add_prod(q[e], p[e]);
-  const dw accv = block_reduce_dw(acc.value(), sh);
-  if (threadIdx.x == 0) partials[blockIdx.x] = dw_to_double(accv);
+  const double v = block_sum_f64(acc.value(), sh);
+  if (threadIdx.x == 0) partials[blockIdx.x] = v;
+  if (last_cta(count)) fin_alpha(partials, (int)gridDim.x, sc, hist, sh);
 }
 
 // z = w * invdiag (when z != null); partials: slot 0 sum w^2 invmult, slot 1 <r,z>, slot 2 <q,z>
 // With `redistribute` the dual residual is replaced by its assembled value split evenly over the
 // copies, r = (S r) / mult (0 on Dirichlet nodes): the same G^T r and the same pairings with
-// continuous vectors, without the cancelling per-copy parts that FP32 cannot hold.
-template <class S>
+// continuous vectors, without the cancelling per-copy parts that FP32 cannot hold.  N > 0: w is not
+// assembled yet, and every entry gathers its node's copies (dss_gather, n = N).
+template <class S, int N>
 __global__ void __launch_bounds__(RED_THREADS)
     k_precond(const S* __restrict__ w, S* __restrict__ r, const S* __restrict__ q,
               const S* __restrict__ invdiag, const float* __restrict__ invmult, S* __restrict__ z,
-              double* __restrict__ partials, const CgScal* __restrict__ sc, long long n,
-              int check_done, int redistribute) {
+              double* partials, unsigned* count, CgScal* sc, long long n, int check_done, int redistribute,
+              const DssGrid grid, const FinBeta fin) {
   if (check_done && *(volatile const int*)&sc->done) return;
-  __shared__ dw sh[32];
+  auto assembled = [&](long long f) {
+    if constexpr (N > 0)
+      return dss_gather<S, N>(w, (int)f, grid);
+    else
+      return w[f];
+  };
+  __shared__ double sh[SUM_THREADS];
   dw a0 = {0.0f, 0.0f};
   AccDw<S> a1, a2;
   auto body = [&](long long e, S we, float im, S idg, S rv, S qv) {
-    const dw w2 = prod_dw<S>(we, we);
+    const dw w2 = prod_dw(we, we);
     a0 = dw_add(a0, {w2.h * im, w2.l * im});  // im: a power of two or zero, exact scaling
     if (z) {
       const S ze = we * idg;
@@ -302,7 +311,7 @@ __global__ void __launch_bounds__(RED_THREADS)
       if (q) a2.add_prod(qv, ze);
     }
   };
-  constexpr long long STRIDE = (long long)RED_BLOCKS * RED_THREADS;
+  const long long STRIDE = (long long)gridDim.x * RED_THREADS;
   long long e = (long long)blockIdx.x * RED_THREADS + threadIdx.x;
   // RED_U elements' loads in flight before they join the accumulators, in the same order
   for (; e + (RED_U - 1) * STRIDE < n; e += RED_U * STRIDE) {
@@ -311,7 +320,7 @@ __global__ void __launch_bounds__(RED_THREADS)
 #pragma unroll
     for (int u = 0; u < RED_U; ++u) {
       const long long f = e + u * STRIDE;
-      wv[u] = w[f];
+      wv[u] = assembled(f);
       im[u] = invmult[f];
       idg[u] = z ? invdiag[f] : S(0);
       rv[u] = (z && !redistribute) ? r[f] : S(0);
@@ -321,62 +330,19 @@ __global__ void __launch_bounds__(RED_THREADS)
     for (int u = 0; u < RED_U; ++u) body(e + u * STRIDE, wv[u], im[u], idg[u], rv[u], qv[u]);
   }
   for (; e < n; e += STRIDE)
-    body(e, w[e], invmult[e], z ? invdiag[e] : S(0), (z && !redistribute) ? r[e] : S(0),
+    body(e, assembled(e), invmult[e], z ? invdiag[e] : S(0), (z && !redistribute) ? r[e] : S(0),
          (z && q) ? q[e] : S(0));
-  a0 = block_reduce_dw(a0, sh);
-  if (threadIdx.x == 0) partials[0 * RED_BLOCKS + blockIdx.x] = dw_to_double(a0);
+  const double v0 = block_sum_f64(dw_to_double(a0), sh);
+  if (threadIdx.x == 0) partials[0 * RED_BLOCKS + blockIdx.x] = v0;
   if (z) {
-    const dw v1 = block_reduce_dw(a1.value(), sh);
-    if (threadIdx.x == 0) partials[1 * RED_BLOCKS + blockIdx.x] = dw_to_double(v1);
+    const double v1 = block_sum_f64(dw_to_double(a1.value()), sh);
+    if (threadIdx.x == 0) partials[1 * RED_BLOCKS + blockIdx.x] = v1;
     if (q) {
-      const dw v2 = block_reduce_dw(a2.value(), sh);
-      if (threadIdx.x == 0) partials[2 * RED_BLOCKS + blockIdx.x] = dw_to_double(v2);
+      const double v2 = block_sum_f64(dw_to_double(a2.value()), sh);
+      if (threadIdx.x == 0) partials[2 * RED_BLOCKS + blockIdx.x] = v2;
     }
   }
-}
-
-__device__ double sum_slot(const double* partials, int slot, dw* sh) {
-  dw acc = {0.0f, 0.0f};
-  for (int b = threadIdx.x; b < RED_BLOCKS; b += RED_THREADS)
-    acc = dw_add(acc, dw_from_double(partials[slot * RED_BLOCKS + b]));
-  acc = block_reduce_dw(acc, sh);
-  return dw_to_double(acc);  // valid in thread 0
-}
-
-// alpha = <r,z>/<q,p>
-__global__ void __launch_bounds__(RED_THREADS)
-    k_fin_alpha(const double* __restrict__ partials, CgScal* __restrict__ sc, double* hist) {
-  if (*(volatile const int*)&sc->done) return;
-  __shared__ dw sh[32];
-  const double qp = sum_slot(partials, 0, sh);
-  if (threadIdx.x == 0) {
-    sc->qp = qp;
-    if (!(qp > 0.0) || !isfinite(qp) || !isfinite(sc->rz)) {
-      sc->status = FE_ERR_BREAKDOWN;
-      sc->done = 1;
-    } else {
-      sc->alpha = sc->rz / qp;
-      if (hist) hist[3 * sc->iter + 0] = sc->alpha;
-    }
-  }
-}
-
-// residual norm, convergence test and beta
-__global__ void __launch_bounds__(RED_THREADS)
-    k_fin_beta(const double* __restrict__ partials, CgScal* __restrict__ sc, double rtol, int mode,
-               int flexible, double* hist) {
-  if ((mode == FIN_ITER || mode == FIN_OUTER) && *(volatile const int*)&sc->done) return;
-  __shared__ dw sh[32];
-  const double rn2 = sum_slot(partials, 0, sh);
-  const double rz = (mode == FIN_INIT_R || mode == FIN_ITER) ? sum_slot(partials, 1, sh) : 0.0;
-  const double qz = (mode == FIN_ITER && flexible) ? sum_slot(partials, 2, sh) : 0.0;
-  if (threadIdx.x != 0) return;
-  const int k = sc->iter;
-  fin_scalars(sc, rn2, rz, qz, rtol < 0.0 ? sc->rtol : rtol, mode, flexible);
-  if (hist && mode == FIN_ITER) {
-    hist[3 * k + 2] = sc->relres;
-    if (!sc->done) hist[3 * k + 1] = sc->beta;
-  }
+  if (last_cta(count)) fin_beta(partials, (int)gridDim.x, sc, fin, sh);
 }
 
 // z = d / s (FP64 primal correction from the FP32 inner solve)
@@ -396,8 +362,8 @@ __global__ void __launch_bounds__(RED_THREADS)
   for (long long e = (long long)blockIdx.x * RED_THREADS + threadIdx.x; e < n;
        e += (long long)RED_BLOCKS * RED_THREADS) {
     const double ze = z[e];
-    a1 = dw_add(a1, prod_dw<double>(r[e], ze));
-    if (q) a2 = dw_add(a2, prod_dw<double>(q[e], ze));
+    a1 = dw_add(a1, prod_dw(r[e], ze));
+    if (q) a2 = dw_add(a2, prod_dw(q[e], ze));
   }
   a1 = block_reduce_dw(a1, sh);
   if (threadIdx.x == 0) partials[1 * RED_BLOCKS + blockIdx.x] = dw_to_double(a1);
@@ -410,18 +376,25 @@ __global__ void __launch_bounds__(RED_THREADS)
 // outer FCG scalars: init rz = <r,z>; iteration beta = -<q,z>/<q,p>, rz = <r,z>
 __global__ void __launch_bounds__(RED_THREADS)
     k_fin_fcg(const double* __restrict__ partials, CgScal* __restrict__ sc, int init) {
-  __shared__ dw sh[32];
-  const double rz = sum_slot(partials, 1, sh);
-  const double qz = init ? 0.0 : sum_slot(partials, 2, sh);
+  __shared__ double sh[SUM_THREADS];
+  double v[2];
+  sum_slots<2>(partials + RED_BLOCKS, RED_BLOCKS, RED_BLOCKS, v, sh);
   if (threadIdx.x != 0) return;
-  if (!init) sc->beta = -qz / sc->qp;
-  sc->rz = rz;
+  if (!init) sc->beta = -v[1] / sc->qp;
+  sc->rz = v[0];
 }
 
 unsigned grid_for(long long n) {
   long long b = (n + 255) / 256;
   if (b > 152LL * 16) b = 152LL * 16;
   return (unsigned)(b < 1 ? 1 : b);
+}
+
+// CTAs of the vector kernels of an iteration: four elements per thread at least, at most the resident
+// grid (the reductions' order depends on n only)
+unsigned red_grid(long long n) {
+  const long long b = (n + 4 * RED_THREADS - 1) / (4 * RED_THREADS);
+  return (unsigned)(b < 1 ? 1 : b > RED_BLOCKS ? RED_BLOCKS : b);
 }
 
 // ---- workspace -------------------------------------------------------------------------------
@@ -433,7 +406,7 @@ static void free_work(CgWork* w, cudaStream_t st) {
     if (w->g64[f]) cudaGraphExecDestroy(w->g64[f]);
     if (w->g32[f]) cudaGraphExecDestroy(w->g32[f]);
   }
-  void* bufs[] = {w->x, w->r, w->z, w->p, w->q, w->w, w->bs, w->invdiag64, w->partials, w->hist,
+  void* bufs[] = {w->x, w->r, w->z, w->p, w->q, w->w, w->bs, w->invdiag64, w->partials, w->count, w->hist,
                   w->r32, w->z32, w->p32, w->q32, w->w32, w->d32, w->invdiag32, w->invmult, w->sc};
   for (void* b : bufs) fe_dfree(b, st);
   cudaFreeHost(w->hsc);
@@ -466,8 +439,11 @@ fe_status fe_cg_get_work(const fe_mesh* cm, bool mixed, CgWork** out) {
     for (double** v : d) FE_TRY(fe_dalloc((void**)v, n * sizeof(double), w->st, "cg vector"));
     FE_TRY(fe_dalloc((void**)&w->invdiag32, n * sizeof(float), w->st, "cg vector"));
     FE_TRY(fe_dalloc((void**)&w->invmult, n * sizeof(float), w->st, "cg vector"));
-    FE_TRY(fe_dalloc((void**)&w->partials, (size_t)RED_BLOCKS * RED_SLOTS * sizeof(double), w->st,
+    FE_TRY(fe_dalloc((void**)&w->partials,
+                     ((size_t)RED_BLOCKS * RED_SLOTS + m->ncells / 2 + 1) * sizeof(double), w->st,
                      "cg partials"));
+    FE_TRY(fe_dalloc((void**)&w->count, sizeof(unsigned), w->st, "cg counter"));
+    FE_CUDA(cudaMemsetAsync(w->count, 0, sizeof(unsigned), w->st), "cg counter");
     FE_TRY(fe_dalloc((void**)&w->sc, 2 * sizeof(CgScal), w->st, "cg scalars"));
     FE_CUDA(cudaMallocHost(&w->hsc, 2 * sizeof(CgScal)), "cudaMallocHost cg scalars");
     FE_TRY(fe_launch_invmult(m, w->invmult, w->st));
@@ -497,29 +473,72 @@ fe_status launch_inner_apply(const ApplyLaunch& L, const CgWork* w) {
   return w->inner_prec == FE_F32 ? fe_launch_apply_f32(L) : fe_launch_apply_lowp(L, w->inner_prec);
 }
 
+// Whether S r is gathered inside the preconditioner kernel instead of summed by three passes first:
+// on small vectors the passes are three launches of little work, on larger ones their whole-sector
+// traffic is cheaper than the gather's.  Gathered against passes, per iteration: FP32 Q5 12^3 (0.4
+// million entries) 47 against 53 us, Q3 24^3 (0.9) 51 against 54, Q3 32^3 (2.1) 74 against 72; FP64 Q5
+// 12^3 58 against 63, Q1 40^3 (0.5) 73 against 64, Q3 24^3 92 against 79.
+template <class S>
+bool gather_dss(const fe_mesh* m, long long n, DssGrid* g) {
+  return fe_dss_grid(m, g) && n <= (sizeof(S) == 4 ? 1ll << 20 : 400000ll);
+}
+
+// w = S wv, z = D^{-1} w, the pairings and the scalars of `fin` (k_precond)
+template <class S>
+fe_status launch_precond(const fe_mesh* m, CgWork* w, S* wv, S* r, const S* q, const S* invdiag, S* z,
+                         CgScal* sc, int check_done, int redistribute, const FinBeta& fin) {
+  DssGrid g;
+  void (*kernel)(const S*, S*, const S*, const S*, const float*, S*, double*, unsigned*, CgScal*,
+                 long long, int, int, const DssGrid, const FinBeta) = k_precond<S, 0>;
+  if (gather_dss<S>(m, w->n, &g)) {
+    switch (m->n) {
+      case 2: kernel = k_precond<S, 2>; break;
+      case 3: kernel = k_precond<S, 3>; break;
+      case 4: kernel = k_precond<S, 4>; break;
+      case 5: kernel = k_precond<S, 5>; break;
+      case 6: kernel = k_precond<S, 6>; break;
+      case 7: kernel = k_precond<S, 7>; break;
+      case 8: kernel = k_precond<S, 8>; break;
+    }
+  } else {
+    FE_TRY(fe_launch_dss(m, sizeof(S) == 8 ? FE_F64 : FE_F32, wv, w->st));
+  }
+  kernel<<<red_grid(w->n), RED_THREADS, 0, w->st>>>(wv, r, q, invdiag, w->invmult, z, w->partials,
+                                                    w->count, sc, w->n, check_done, redistribute, g,
+                                                    fin);
+  return fe_cuda_check(cudaGetLastError(), "preconditioner launch");
+}
+
 // one PCG iteration on vectors of type S, solution of type U, scalars sc
 template <class S, class U>
 fe_status enqueue_iteration(const fe_mesh* m, CgWork* w, int op, bool flexible, U* u, S* r, S* z,
                             S* p, S* q, S* wv, const S* invdiag, CgScal* sc, double* hist) {
   const long long n = w->n;
   ApplyLaunch L{m, op, p, q, w->st, &sc->done};
+  // FP32 iterations redistribute: r = (S r)/mult is formed by the preconditioner
+  const int redistribute = sizeof(S) == 4 ? 1 : 0;
+  const unsigned grid = red_grid(n);
+  const CgApply cg{z, sc, w->partials + (size_t)RED_BLOCKS * RED_SLOTS, w->count, hist};
+  const bool fused = sizeof(S) == 8 ? fe_apply_fuses_cg(m, FE_F64)
+                                    : w->inner_prec == FE_F32 && fe_apply_fuses_cg(m, FE_F32);
+  if (fused)
+    L.cg = &cg;
+  else
+    k_update_p<S><<<grid, RED_THREADS, 0, w->st>>>(p, z, sc, n);
   if (sizeof(S) == 8)
     FE_TRY(fe_launch_apply_f64dw(L));
   else
     FE_TRY(launch_inner_apply(L, w));
-  // FP32 iterations redistribute: r = (S r)/mult is formed by the preconditioner
-  const int redistribute = sizeof(S) == 4 ? 1 : 0;
-  k_qp<S><<<RED_BLOCKS, RED_THREADS, 0, w->st>>>(q, p, w->partials, sc, n);
-  k_fin_alpha<<<1, RED_THREADS, 0, w->st>>>(w->partials, sc, hist);
-  k_update_ur<S, U><<<RED_BLOCKS, RED_THREADS, 0, w->st>>>(u, r, wv, p, q, sc, n, !redistribute);
-  FE_TRY(fe_launch_dss(m, sizeof(S) == 8 ? FE_F64 : FE_F32, wv, w->st));
-  k_precond<S><<<RED_BLOCKS, RED_THREADS, 0, w->st>>>(wv, r, flexible ? q : nullptr, invdiag,
-                                                      w->invmult, z, w->partials, sc, n, 1,
-                                                      redistribute);
-  k_fin_beta<<<1, RED_THREADS, 0, w->st>>>(w->partials, sc, -1.0, FIN_ITER, flexible ? 1 : 0, hist);
-  k_update_p<S><<<RED_BLOCKS, RED_THREADS, 0, w->st>>>(p, z, sc, n);
-  return fe_cuda_check(cudaGetLastError(), "cg iteration launch");
+  if (!fused)
+    k_qp<S><<<grid, RED_THREADS, 0, w->st>>>(q, p, w->partials, w->count, sc, n, hist);
+  k_update_ur<S, U><<<grid, RED_THREADS, 0, w->st>>>(u, r, wv, p, q, sc, n, !redistribute);
+  FE_CUDA(cudaGetLastError(), "cg iteration launch");
+  return launch_precond<S>(m, w, wv, r, flexible ? q : nullptr, invdiag, z, sc, 1, redistribute,
+                           {-1.0, FIN_ITER, flexible ? 1 : 0, hist});
 }
+
+// iterations per graph: between the graphs of a run the GPU waits for the launch
+constexpr int GRAPH_ITERS = 4;
 
 // the iteration graph; its stopping tolerance is read from sc->rtol at every replay
 template <class S, class U>
@@ -532,7 +551,9 @@ fe_status build_graph(const fe_mesh* m, CgWork* w, int op, bool flexible, U* u, 
     FE_TRY(sizeof(S) == 8 ? fe_launch_apply_f64dw(L) : launch_inner_apply(L, w));
   }
   FE_CUDA(cudaStreamBeginCapture(w->st, cudaStreamCaptureModeThreadLocal), "begin capture");
-  fe_status s = enqueue_iteration<S, U>(m, w, op, flexible, u, r, z, p, q, wv, invdiag, sc, hist);
+  fe_status s = FE_OK;
+  for (int k = 0; k < GRAPH_ITERS && s == FE_OK; ++k)
+    s = enqueue_iteration<S, U>(m, w, op, flexible, u, r, z, p, q, wv, invdiag, sc, hist);
   cudaError_t e = cudaStreamEndCapture(w->st, &g);
   if (s != FE_OK) {
     if (g) cudaGraphDestroy(g);
@@ -546,9 +567,9 @@ fe_status build_graph(const fe_mesh* m, CgWork* w, int op, bool flexible, U* u, 
 
 // run graph replays until the flag is set; returns the host copy of the scalars
 fe_status run_until_done(CgWork* w, cudaGraphExec_t exec, int slot, CgScal* out) {
-  const int batch = 8;
+  const int batch = 8;  // iterations between two looks at the flag
   for (;;) {
-    for (int b = 0; b < batch; ++b) FE_CUDA(cudaGraphLaunch(exec, w->st), "graph launch");
+    for (int b = 0; b < batch; b += GRAPH_ITERS) FE_CUDA(cudaGraphLaunch(exec, w->st), "graph launch");
     FE_CUDA(cudaMemcpyAsync(&w->hsc[slot], &w->sc[slot], sizeof(CgScal), cudaMemcpyDeviceToHost,
                             w->st),
             "scalar readback");
@@ -585,21 +606,20 @@ template <class S>
 fe_status residual_norm(const fe_mesh* m, CgWork* w, const S* v, S* wv, CgScal* sc, int mode) {
   FE_CUDA(cudaMemcpyAsync(wv, v, w->n * sizeof(S), cudaMemcpyDeviceToDevice, w->st), "cg copy");
   FE_TRY(fe_launch_dss(m, sizeof(S) == 8 ? FE_F64 : FE_F32, wv, w->st));
-  k_precond<S><<<RED_BLOCKS, RED_THREADS, 0, w->st>>>(wv, nullptr, nullptr, nullptr, w->invmult,
-                                                      nullptr, w->partials, sc, w->n, 0, 0);
-  k_fin_beta<<<1, RED_THREADS, 0, w->st>>>(w->partials, sc, 0.0, mode, 0, nullptr);
+  k_precond<S, 0><<<red_grid(w->n), RED_THREADS, 0, w->st>>>(
+      wv, nullptr, nullptr, nullptr, w->invmult, nullptr, w->partials, w->count, sc, w->n, 0, 0,
+      DssGrid(), {0.0, mode, 0, nullptr});
   return fe_cuda_check(cudaGetLastError(), "residual norm launch");
 }
 
-// initial preconditioned residual: w = S r, z = D^{-1} w, <r,z>, relres; p = z
+// initial preconditioned residual: w = S r, z = D^{-1} w, <r,z>, relres; p = z (and beta = 0, so the
+// first iteration's z + beta p is z)
 template <class S>
 fe_status init_direction(const fe_mesh* m, CgWork* w, S* r, S* z, S* p, S* wv, const S* invdiag,
                          CgScal* sc, double rtol) {
   FE_CUDA(cudaMemcpyAsync(wv, r, w->n * sizeof(S), cudaMemcpyDeviceToDevice, w->st), "cg copy");
-  FE_TRY(fe_launch_dss(m, sizeof(S) == 8 ? FE_F64 : FE_F32, wv, w->st));
-  k_precond<S><<<RED_BLOCKS, RED_THREADS, 0, w->st>>>(wv, r, nullptr, invdiag, w->invmult, z,
-                                                      w->partials, sc, w->n, 0, sizeof(S) == 4 ? 1 : 0);
-  k_fin_beta<<<1, RED_THREADS, 0, w->st>>>(w->partials, sc, rtol, FIN_INIT_R, 0, nullptr);
+  FE_TRY(launch_precond<S>(m, w, wv, r, nullptr, invdiag, z, sc, 0, sizeof(S) == 4 ? 1 : 0,
+                           {rtol, FIN_INIT_R, 0, nullptr}));
   FE_CUDA(cudaMemcpyAsync(p, z, w->n * sizeof(S), cudaMemcpyDeviceToDevice, w->st), "cg copy");
   return fe_cuda_check(cudaGetLastError(), "init launch");
 }
@@ -665,8 +685,8 @@ fe_status solve_fcg_outer(const fe_mesh* m, CgWork* w, int op, const double* b, 
   while (total < opts->maxit) {
     ApplyLaunch L{m, op, w->p, w->q, w->st, nullptr};
     FE_TRY(fe_launch_apply_f64dw(L));
-    k_qp<double><<<RED_BLOCKS, RED_THREADS, 0, w->st>>>(w->q, w->p, w->partials, &w->sc[0], n);
-    k_fin_alpha<<<1, RED_THREADS, 0, w->st>>>(w->partials, &w->sc[0], nullptr);
+    k_qp<double><<<red_grid(n), RED_THREADS, 0, w->st>>>(w->q, w->p, w->partials, w->count,
+                                                         &w->sc[0], n, nullptr);
     k_update_ur<double, double><<<RED_BLOCKS, RED_THREADS, 0, w->st>>>(
         w->x, w->r, w->w, w->p, w->q, &w->sc[0], n, 1);
     FE_TRY(residual_norm<double>(m, w, w->r, w->w, &w->sc[0], FIN_NORM));
@@ -751,16 +771,15 @@ fe_status solve_reliable(const fe_mesh* m, CgWork* w, int op, const double* b, d
       // z = P r', <r', z>; p = z + beta p in the new scale (p and rz_old were in units of s_old)
       FE_CUDA(cudaMemcpyAsync(w->w32, w->r32, n * sizeof(float), cudaMemcpyDeviceToDevice, w->st),
               "cg copy");
-      FE_TRY(fe_launch_dss(m, FE_F32, w->w32, w->st));
-      k_precond<float><<<RED_BLOCKS, RED_THREADS, 0, w->st>>>(w->w32, w->r32, nullptr, w->invdiag32,
-                                                              w->invmult, w->z32, w->partials,
-                                                              &w->sc[1], n, 0, 1);
-      k_fin_beta<<<1, RED_THREADS, 0, w->st>>>(w->partials, &w->sc[1], irtol, FIN_INIT_R, 0, nullptr);
+      FE_TRY(launch_precond<float>(m, w, w->w32, w->r32, nullptr, w->invdiag32, w->z32, &w->sc[1], 0, 1,
+                                   {irtol, FIN_INIT_R, 0, nullptr}));
       FE_TRY(read_scal(w, 1, &h));
       const double ratio = s / s_old;
       const double beta = h.rz / (rz_old * ratio * ratio);
-      k_keep_direction<<<grid_for(n), 256, 0, w->st>>>(w->p32, w->z32, (float)(beta * ratio), n);
-      FE_CUDA(cudaGetLastError(), "keep direction launch");
+      w->hsc[1].beta = beta * ratio;  // the run's first iteration forms z + (beta ratio) p
+      FE_CUDA(cudaMemcpyAsync(&w->sc[1].beta, &w->hsc[1].beta, sizeof(double), cudaMemcpyHostToDevice,
+                              w->st),
+              "keep direction");
     }
     if (!h.done) {
       if (!w->g32[0])

@@ -20,14 +20,20 @@ struct CgScal {
 // beta.  FIN_NORM: residual only.  FIN_OUTER: residual, outer count, convergence.
 enum { FIN_INIT_B = 0, FIN_INIT_R = 1, FIN_ITER = 2, FIN_NORM = 3, FIN_OUTER = 4 };
 
-__device__ __forceinline__ void fin_scalars(CgScal* sc, double rn2, double rz, double qz, double rtol,
-                                            int mode, int flexible) {
+// relative residual and beta of the new values
+__device__ __forceinline__ double fin_rel(const CgScal* sc, double rn2) {
+  return sc->bnorm2 > 0.0 ? sqrt(rn2 / sc->bnorm2) : 0.0;
+}
+__device__ __forceinline__ double fin_new_beta(const CgScal* sc, double rz, double qz, int flexible) {
+  return flexible ? -qz / sc->qp : rz / sc->rz;
+}
+__device__ __forceinline__ void fin_scalars(CgScal* sc, double rn2, double rz, double rel, double beta,
+                                            double rtol, int mode) {
   if (mode == FIN_INIT_B) {
     sc->bnorm2 = rn2;
     return;
   }
   sc->rnorm2 = rn2;
-  const double rel = sc->bnorm2 > 0.0 ? sqrt(rn2 / sc->bnorm2) : 0.0;
   sc->relres = rel;
   if (mode == FIN_NORM) return;
   if (mode == FIN_OUTER) {
@@ -77,7 +83,7 @@ __device__ __forceinline__ void fin_scalars(CgScal* sc, double rn2, double rz, d
     sc->done = 1;
     return;
   }
-  sc->beta = flexible ? -qz / sc->qp : rz / sc->rz;
+  sc->beta = beta;
   sc->rz = rz;
 }
 
@@ -91,7 +97,8 @@ struct CgWork {
   double* invdiag64 = nullptr;
   float* invdiag32 = nullptr;
   float* invmult = nullptr;
-  double* partials = nullptr;
+  double* partials = nullptr;  // RED_SLOTS slots of RED_BLOCKS, then one per CTA of a fused apply
+  unsigned* count = nullptr;   // arrivals of the grid reductions, 0 between launches
   CgScal* sc = nullptr;   // [0] outer / FP64 solve, [1] inner FP32 solve
   CgScal* hsc = nullptr;  // pinned host mirror
   double* hist = nullptr;

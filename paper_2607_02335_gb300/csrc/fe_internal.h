@@ -137,6 +137,14 @@ void fe_mesh_release_async(fe_mesh* m, cudaStream_t st);
 // diagonal exist (the server keeps only what its solves read)
 void fe_mesh_drop_geo64(fe_mesh* m, cudaStream_t st);
 
+struct CgScal;
+struct CgApply {
+  const void* z;     // z of p := z + beta p, in the arithmetic of the vectors
+  CgScal* sc;        // beta in, alpha out
+  double* partials;  // one per CTA: at least n_cells / 2 + 1
+  unsigned* count;   // 0 between launches
+  double* hist;      // alpha history or null
+};
 // apply (fe_apply.cu / fe_apply_*.cu)
 struct ApplyLaunch {
   const fe_mesh* m;
@@ -148,7 +156,12 @@ struct ApplyLaunch {
   bool assemble = false;      // FE_ASSEMBLE: the launcher also runs the DSS on y
   int* brick_out = nullptr;   // assembled launches with this set leave the DSS passes to the
                               // caller and report the brick (bx, by) the kernel summed inside
+  // one CG iteration's neighbours of the operator, fused into a Laplace apply that assembles nothing
+  // (fe_apply_fuses_cg): x is p, first updated to z + beta p in place; <q,p> and alpha at the end
+  const CgApply* cg = nullptr;
 };
+// whether a CG iteration's FE_F64 or FE_F32 apply on this mesh is the fused one (fe_apply_dw.cu)
+bool fe_apply_fuses_cg(const fe_mesh* m, int prec);
 // fe_apply with its checks; an assembled call with brick_out set leaves the DSS passes to the
 // caller as ApplyLaunch::brick_out does (fe_api.cu)
 fe_status fe_apply_impl(const fe_mesh* m, fe_op op, fe_prec prec, const void* x, void* y,

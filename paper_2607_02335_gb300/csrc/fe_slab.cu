@@ -250,12 +250,14 @@ __global__ void k_fin(const double* __restrict__ red_all, int size, int nslots, 
   const double rho = dw_to_double(acc[0]), gamma = dw_to_double(acc[1]),
                delta = dw_to_double(acc[2]);
   if (mode == FIN_INIT_B) {
-    fin_scalars(sc, rho, 0.0, 0.0, rtol, FIN_INIT_B, 0);
+    fin_scalars(sc, rho, 0.0, 0.0, 0.0, rtol, FIN_INIT_B);
     return;
   }
   const int k = sc->iter;
   const double alpha_used = sc->alpha;
-  fin_scalars(sc, rho, gamma, 0.0, rtol, mode, 0);  // FIN_ITER: beta = gamma / gamma_old
+  // FIN_ITER: beta = gamma / gamma_old
+  fin_scalars(sc, rho, gamma, fin_rel(sc, rho),
+              mode == FIN_ITER ? fin_new_beta(sc, gamma, 0.0, 0) : 0.0, rtol, mode);
   if (mode == FIN_ITER && hist) {
     hist[3 * k + 0] = alpha_used;
     hist[3 * k + 2] = sc->relres;
