@@ -488,7 +488,7 @@ __device__ __forceinline__ void apply_pairs(const CellArgs<N, typename PairCfg<N
   // the metric of the next point (the first one's is loaded before the last V sweep)
   constexpr bool AHEAD = OP == FE_LAPLACE && STORED && TU.ahead != 0;
   V next[AHEAD ? 6 : 1];
-  ExpShift es;
+  ExpShift es = {};
   // v[c][r], a line's values per cell -> out[r]
   auto to_lanes = [&](const auto& v, auto& out) {
     constexpr int M = sizeof(out) / sizeof(out[0]);

@@ -214,52 +214,144 @@ __device__ __forceinline__ float* vec<float>(const BProb& P, int which) {
   }
 }
 
+// 16-byte pieces of a chunk.  A thread issues the loads of all its pieces (of every vector of the
+// kernel) before the first store or sum: one memory round trip per chunk in FP32, two in FP64, where
+// single elements four at a time took four (16-problem FP32 batch: <q,p> 10 us, the u/r update 13, the
+// preconditioner 13, the p update 8 per launch).
+template <class S, int UN = 4>
+struct Vec {
+  static constexpr int W = 16 / sizeof(S), U = UN;
+  S v[U][W];
+  __device__ __forceinline__ void load(int u, const S* p) {
+    using T = typename std::conditional<sizeof(S) == 8, double2, float4>::type;
+    *reinterpret_cast<T*>(v[u]) = *reinterpret_cast<const T*>(p);
+  }
+  __device__ __forceinline__ void store(int u, S* p) const {
+    using T = typename std::conditional<sizeof(S) == 8, double2, float4>::type;
+    *reinterpret_cast<T*>(p) = *reinterpret_cast<const T*>(v[u]);
+  }
+};
+// the float companion (1/mult) of a Vec<S>'s pieces
 template <class S>
-__device__ __forceinline__ dw prod2(S a, S b);
-template <>
-__device__ __forceinline__ dw prod2<double>(double a, double b) {
-  return dw_mul(dw_from_double(a), dw_from_double(b));
+__device__ __forceinline__ void load_mult(float (&o)[Vec<S>::W], const float* p) {
+  if constexpr (sizeof(S) == 4)
+    *reinterpret_cast<float4*>(o) = *reinterpret_cast<const float4*>(p);
+  else
+    *reinterpret_cast<float2*>(o) = *reinterpret_cast<const float2*>(p);
 }
-template <>
-__device__ __forceinline__ dw prod2<float>(float a, float b) {
-  const float p = __fmul_rn(a, b);
-  return {p, __fmaf_rn(a, b, -p)};
+// pieces(v0) for every group of U pieces of the chunk [lo, hi) (piece v starts at element lo + v W), then
+// single(e) for the elements after the last whole piece
+template <class V, class F, class G>
+__device__ __forceinline__ void over_chunk(long long lo, long long hi, F pieces, G single) {
+  constexpr int W = V::W, U = V::U;
+  const int n = (int)(hi - lo), nv = n / W;
+  for (int v0 = threadIdx.x; v0 < nv; v0 += U * BT) pieces(v0, nv);
+  const int t = nv * W + threadIdx.x;
+  if (t < n) single(lo + t);
 }
 
-// partials[chunk*4 + 0] = sum q p
+// ---- per-problem scalars, finished by the CTA that writes the last of the problem's partials ----------
+template <int NS>
+__device__ __forceinline__ void sum_chunks(const BProb& P, const double* partials, double (&v)[NS],
+                                           double* sh) {
+#pragma unroll
+  for (int s = 0; s < NS; ++s) v[s] = 0.0;
+  for (int c = P.chunk0 + threadIdx.x; c < P.chunk1; c += BT)
+#pragma unroll
+    for (int s = 0; s < NS; ++s) v[s] += __ldcg(partials + (size_t)c * 4 + s);
+  block_sums_f64<NS>(v, sh);
+}
+
+__device__ __forceinline__ void batch_fin_alpha(const BProb& P, int slot, const double* partials,
+                                                double* sh) {
+  CgScal* sc = &P.sc[slot];
+  double qp[1];
+  sum_chunks<1>(P, partials, qp, sh);
+  if (threadIdx.x != 0) return;
+  sc->qp = qp[0];
+  if (!(qp[0] > 0.0) || !isfinite(qp[0]) || !isfinite(sc->rz)) {
+    sc->status = FE_ERR_BREAKDOWN;
+    sc->done = 1;
+  } else {
+    sc->alpha = sc->rz / qp[0];
+  }
+}
+
+// mode: FIN_INIT_B, FIN_INIT_R, FIN_ITER, FIN_NORM, FIN_OUTER (fe_cgcore.h); tolerances and the
+// FCG switch are per problem (slot 0: the outer or FP64 solve, slot 1: the inner FP32 solve).  The
+// divisions and the square root, long on the FP64 pipe, in two warps.
+__device__ __forceinline__ void batch_fin_beta(const BProb& P, int slot, int mode,
+                                               const double* partials, double* sh) {
+  CgScal* sc = &P.sc[slot];
+  const int flexible = slot == 0 ? P.flexible : 0;
+  const double rtol = slot == 0 ? P.rtol : sc->rtol;
+  double v[3] = {0.0, 0.0, 0.0};
+  if (mode == FIN_ITER && flexible) {
+    sum_chunks<3>(P, partials, v, sh);
+  } else {
+    double t[2];  // slot 1 is stale, and not used, in the modes without <r,z>
+    sum_chunks<2>(P, partials, t, sh);
+    v[0] = t[0], v[1] = t[1];
+  }
+  if (threadIdx.x == 0) sh[0] = v[0];
+  __syncthreads();
+  if (threadIdx.x == 32 && mode != FIN_INIT_B) sh[1] = fin_rel(sc, sh[0]);
+  const double beta = threadIdx.x == 0 && mode == FIN_ITER ? fin_new_beta(sc, v[1], v[2], flexible) : 0.0;
+  __syncthreads();
+  if (threadIdx.x == 0) fin_scalars(sc, v[0], v[1], sh[1], beta, rtol, mode);
+  __syncthreads();  // sh is used again by the CTA's next chunk
+}
+
+// called by every thread once the chunk's partials are written (by thread 0); true in the CTA whose
+// chunk is the last of its problem's.  A problem's chunks all arrive or, when it is done, none.
+__device__ __forceinline__ bool last_chunk(const BProb& P, unsigned* arrive) {
+  __shared__ int last;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(arrive, 1u) == (unsigned)(P.chunk1 - P.chunk0 - 1);
+    if (last) *arrive = 0u;
+  }
+  __syncthreads();
+  const bool mine = last != 0;
+  __syncthreads();
+  if (mine) __threadfence();
+  return mine;
+}
+
+// <q, p> and alpha of every problem (partials[chunk*4 + 0])
 template <class S>
 __global__ void __launch_bounds__(BT)
     kb_qp(const BProb* __restrict__ probs, const Chunk* __restrict__ chunks, int nchunks, int slot,
-          double* __restrict__ partials) {
-  __shared__ dw sh[32];
+          double* partials, unsigned* arrive) {
+  using V = Vec<S>;
+  __shared__ double sh[SUM_MAX * SUM_THREADS];
   for (int c = blockIdx.x; c < nchunks; c += gridDim.x) {
     const Chunk C = chunks[c];
     const BProb& P = probs[C.prob];
     if (*(volatile const int*)&P.sc[slot].done) continue;
     const S* q = vec<S>(P, 4);
     const S* p = vec<S>(P, 3);
-    // float: double-word sums of exact products; double: binary64 FMAs (one FP64-pipe operation
-    // per product costs less than converting both factors to double-word)
-    dw acc = {0.0f, 0.0f};
-    double acc64 = 0.0;
-    auto add = [&](S a, S b) {
-      if constexpr (sizeof(S) == 8)
-        acc64 = fma(a, b, acc64);
-      else
-        acc = dw_add(acc, prod2<S>(a, b));
-    };
-    long long e = C.lo + threadIdx.x;
-    for (; e + (RED_U - 1) * BT < C.hi; e += RED_U * BT) {  // loads first, same order
-      S qv[RED_U], pv[RED_U];
+    Acc<S> acc;
+    over_chunk<V>(
+        C.lo, C.hi,
+        [&](int v0, int nv) {
+          V qv, pv;
 #pragma unroll
-      for (int u = 0; u < RED_U; ++u) qv[u] = q[e + u * BT], pv[u] = p[e + u * BT];
+          for (int u = 0; u < V::U; ++u) {
+            const int v = v0 + u * BT;
+            if (v < nv) qv.load(u, q + C.lo + v * V::W), pv.load(u, p + C.lo + v * V::W);
+          }
 #pragma unroll
-      for (int u = 0; u < RED_U; ++u) add(qv[u], pv[u]);
-    }
-    for (; e < C.hi; e += BT) add(q[e], p[e]);
-    if constexpr (sizeof(S) == 8) acc = dw_from_double(acc64);
-    acc = block_reduce_dw(acc, sh);
-    if (threadIdx.x == 0) partials[(size_t)c * 4 + 0] = dw_to_double(acc);
+          for (int u = 0; u < V::U; ++u)
+            if (v0 + u * BT < nv)
+#pragma unroll
+              for (int w = 0; w < V::W; ++w) acc.add_prod(qv.v[u][w], pv.v[u][w]);
+        },
+        [&](long long e) { acc.add_prod(q[e], p[e]); });
+    double v[1] = {acc.value()};
+    block_sums_f64<1>(v, sh);
+    if (threadIdx.x == 0) partials[(size_t)c * 4 + 0] = v[0];
+    if (arrive && last_chunk(P, arrive + C.prob)) batch_fin_alpha(P, slot, partials, sh);
   }
 }
 
@@ -269,107 +361,109 @@ template <class S>
 __global__ void __launch_bounds__(BT)
     kb_update_ur(const BProb* __restrict__ probs, const Chunk* __restrict__ chunks, int nchunks,
                  int slot, int keep_r) {
+  using V = Vec<S, sizeof(S) == 4 ? 4 : 2>;
   for (int c = blockIdx.x; c < nchunks; c += gridDim.x) {
     const Chunk C = chunks[c];
     const BProb& P = probs[C.prob];
     if (*(volatile const int*)&P.sc[slot].done) continue;
-    const double a = P.sc[slot].alpha;
+    const S a = (S)P.sc[slot].alpha;
     S* u = vec<S>(P, 0);
     S* r = vec<S>(P, 1);
     const S* p = vec<S>(P, 3);
     const S* q = vec<S>(P, 4);
     S* w = vec<S>(P, 5);
-    // FP32 state: FP32 arithmetic (the FP64 pipe is slow).  RED_U elements' loads are issued
-    // before their stores (the vectors are distinct arrays)
-    auto step = [&](long long e, S ue, S pe, S qe, S rq) {
-      S re;
-      if constexpr (sizeof(S) == 4) {
-        const float af = (float)a;
-        u[e] = fmaf(af, pe, ue);
-        re = fmaf(-af, qe, rq);
-      } else {
-        u[e] = fma(a, pe, ue);
-        re = fma(-a, qe, rq);
-      }
-      if (keep_r) r[e] = re;
-      w[e] = re;
+    auto fma_ = [](S x, S y, S z) {
+      if constexpr (sizeof(S) == 4)
+        return fmaf(x, y, z);
+      else
+        return fma(x, y, z);
     };
-    long long e = C.lo + threadIdx.x;
-    for (; e + (RED_U - 1) * BT < C.hi; e += RED_U * BT) {
-      S uv[RED_U], pv[RED_U], qv[RED_U], rv[RED_U];
+    over_chunk<V>(
+        C.lo, C.hi,
+        [&](int v0, int nv) {
+          V uv, pv, qv, rv;
 #pragma unroll
-      for (int k = 0; k < RED_U; ++k) {
-        const long long f = e + k * BT;
-        uv[k] = u[f], pv[k] = p[f], qv[k] = q[f], rv[k] = r[f];
-      }
+          for (int k = 0; k < V::U; ++k) {
+            const int v = v0 + k * BT;
+            const long long e = C.lo + (long long)v * V::W;
+            if (v < nv) uv.load(k, u + e), pv.load(k, p + e), qv.load(k, q + e), rv.load(k, r + e);
+          }
 #pragma unroll
-      for (int k = 0; k < RED_U; ++k) step(e + k * BT, uv[k], pv[k], qv[k], rv[k]);
-    }
-    for (; e < C.hi; e += BT) step(e, u[e], p[e], q[e], r[e]);
+          for (int k = 0; k < V::U; ++k) {
+            const int v = v0 + k * BT;
+            if (v >= nv) continue;
+            const long long e = C.lo + (long long)v * V::W;
+#pragma unroll
+            for (int t = 0; t < V::W; ++t) {
+              uv.v[k][t] = fma_(a, pv.v[k][t], uv.v[k][t]);
+              rv.v[k][t] = fma_(-a, qv.v[k][t], rv.v[k][t]);
+            }
+            uv.store(k, u + e);
+            if (keep_r) rv.store(k, r + e);
+            rv.store(k, w + e);
+          }
+        },
+        [&](long long e) {
+          u[e] = fma_(a, p[e], u[e]);
+          const S re = fma_(-a, q[e], r[e]);
+          if (keep_r) r[e] = re;
+          w[e] = re;
+        });
   }
 }
 
-// structured DSS pass of one axis over rows of interfaces of every problem, one warp per row:
+// structured DSS pass of one axis over rows of interfaces of every problem, DSS_TEAM threads per row
+// (one warp per row left a row of 12 cells six round trips long: 12 us a pass in the 16-problem batch):
 // x-pass row (cz, cy) with items (interface, face node), y-pass row (cz, interface) and z-pass row
 // (interface, cy) with items (cx, face node); node counts are compile-time, so the index
 // arithmetic inside a row is multiplications and shifts.  Pairs of one pass are disjoint.
+constexpr int DSS_TEAM = 128;
 template <class S, int N>
 __device__ __forceinline__ void dss_row(S* __restrict__ v, int axis, int row, int mx, int my,
                                         int lane) {
   constexpr int P = N - 1, N2 = N * N, N3 = N2 * N;
-  long long first, rstep;
-  int items, lstep, locL0, locR0, sa, sb;
+  long long first, rstep;  // left cell of the row's first item; right cell - left cell
+  int items, locL0, locR0, sa, sb;
   if (axis == 0) {
     first = (long long)row * mx;
     items = (mx - 1) * N2;
-    lstep = 1;
     rstep = 1;
     locL0 = P, locR0 = 0, sa = N, sb = N2;
   } else if (axis == 1) {
     const int cz = row / (my - 1), u = row - cz * (my - 1);
     first = ((long long)cz * my + u) * mx;
     items = mx * N2;
-    lstep = 1;
     rstep = mx;
     locL0 = P * N, locR0 = 0, sa = 1, sb = N2;
   } else {
     const int u = row / my, cy = row - u * my;
     first = ((long long)u * my + cy) * mx;
     items = mx * N2;
-    lstep = 1;
     rstep = (long long)mx * my;
     locL0 = P * N2, locR0 = 0, sa = 1, sb = N;
   }
-  // RED_U pairs' loads in flight before their stores (pairs of a pass are disjoint)
-  auto addr = [&](int it, S*& pl, S*& pr) {
-    const int g = it / N2, f = it - g * N2, fb = f / N, fa = f - fb * N;
-    const long long L = first + (long long)g * lstep;
-    const int off = fa * sa + fb * sb;
-    pl = v + L * N3 + locL0 + off;
-    pr = v + (L + rstep) * N3 + locR0 + off;
-  };
-  int it = lane;
-  for (; it + (RED_U - 1) * 32 < items; it += RED_U * 32) {
-    S *pl[RED_U], *pr[RED_U], l[RED_U], r[RED_U];
+  S* const left = v + first * N3 + locL0;
+  S* const right = v + (first + rstep) * N3 + locR0;
+  // DU pairs' loads in flight before their stores (pairs of a pass are disjoint)
+  constexpr int DU = 4;
+  for (int it = lane; it < items; it += DU * DSS_TEAM) {
+    int off[DU];
+    S l[DU], r[DU];
 #pragma unroll
-    for (int k = 0; k < RED_U; ++k) {
-      addr(it + k * 32, pl[k], pr[k]);
-      l[k] = *pl[k];
-      r[k] = *pr[k];
+    for (int k = 0; k < DU; ++k) {
+      const int t = min(it + k * DSS_TEAM, items - 1);  // past the end: read again, not stored
+      const int g = t / N2, f = t - g * N2, fb = f / N, fa = f - fb * N;
+      off[k] = g * N3 + fa * sa + fb * sb;
+      l[k] = left[off[k]];
+      r[k] = right[off[k]];
     }
 #pragma unroll
-    for (int k = 0; k < RED_U; ++k) {
-      const S sum = l[k] + r[k];
-      *pl[k] = sum;
-      *pr[k] = sum;
-    }
-  }
-  for (; it < items; it += 32) {
-    S *pl, *pr;
-    addr(it, pl, pr);
-    const S sum = *pl + *pr;
-    *pl = sum;
-    *pr = sum;
+    for (int k = 0; k < DU; ++k)
+      if (it + k * DSS_TEAM < items) {
+        const S sum = l[k] + r[k];
+        left[off[k]] = sum;
+        right[off[k]] = sum;
+      }
   }
 }
 
@@ -377,12 +471,12 @@ template <class S>
 __global__ void __launch_bounds__(BT)
     kb_dss(const BProb* __restrict__ probs, const DssRow* __restrict__ rows, int nrows, int slot,
            int axis) {
-  const int lane = threadIdx.x & 31;
-  const int warps = gridDim.x * (BT / 32);
-  for (int w = blockIdx.x * (BT / 32) + (threadIdx.x >> 5); w < nrows; w += warps) {
+  constexpr int TEAMS = BT / DSS_TEAM;
+  const int lane = threadIdx.x % DSS_TEAM;
+  for (int w = blockIdx.x * TEAMS + threadIdx.x / DSS_TEAM; w < nrows; w += gridDim.x * TEAMS) {
     const DssRow R = rows[w];
     const BProb& P = probs[R.prob];
-    if (*(volatile const int*)&P.sc[slot].done) continue;  // uniform over the warp
+    if (*(volatile const int*)&P.sc[slot].done) continue;  // uniform over the team
     S* v = vec<S>(P, 5);
     switch (P.n) {
       case 2: dss_row<S, 2>(v, axis, R.row, P.mx, P.my, lane); break;
@@ -396,13 +490,14 @@ __global__ void __launch_bounds__(BT)
   }
 }
 
-// z = w * invdiag (mode & 1), r = w * invmult (mode & 2, redistribute); partials slot 0 sum w^2/mult,
-// slot 1 <r,z>, slot 2 <q,z> (mode & 4)
+// z = w * invdiag (pmode & 1), r = w * invmult (pmode & 2, redistribute); partials slot 0 sum
+// w^2/mult, slot 1 <r,z>, slot 2 <q,z> (pmode & 4); then the problem's scalars (batch_fin_beta, mode)
 template <class S>
 __global__ void __launch_bounds__(BT)
     kb_precond(const BProb* __restrict__ probs, const Chunk* __restrict__ chunks, int nchunks,
-               int slot, int mode, double* __restrict__ partials) {
-  __shared__ dw sh[32];
+               int slot, int pmode, int mode, double* partials, unsigned* arrive) {
+  using V = Vec<S, 2>;
+  __shared__ double sh[SUM_MAX * SUM_THREADS];
   for (int c = blockIdx.x; c < nchunks; c += gridDim.x) {
     const Chunk C = chunks[c];
     const BProb& P = probs[C.prob];
@@ -412,53 +507,66 @@ __global__ void __launch_bounds__(BT)
     S* z = vec<S>(P, 2);
     const S* q = vec<S>(P, 4);
     const S* idg = (sizeof(S) == 8) ? (const S*)P.invdiag64 : (const S*)P.invdiag32;
-    dw a0 = {0.0f, 0.0f}, a1 = {0.0f, 0.0f}, a2 = {0.0f, 0.0f};
-    auto body = [&](long long e, S we, float im, S dg, S rv, S qv) {
-      const dw w2 = prod2<S>(we, we);
-      a0 = dw_add(a0, {w2.h * im, w2.l * im});
-      if (mode & 1) {
-        const S ze = we * dg;
-        z[e] = ze;
-        S re;
-        if (mode & 2) {
-          re = we * (S)im;
-          r[e] = re;
-        } else {
-          re = rv;
-        }
-        a1 = dw_add(a1, prod2<S>(re, ze));
-        if (mode & 4) a2 = dw_add(a2, prod2<S>(qv, ze));
-      }
+    const float* im = P.invmult;
+    const bool dir = pmode & 1, redist = pmode & 2, flex = pmode & 4;
+    Sum2 a0, a1, a2;
+    auto body = [&](S we, float ime, S dg, S& re, S qe) -> S {  // returns z, updates r
+      const dw w2 = prod_dw(we, we);
+      a0.add({w2.h * ime, w2.l * ime});
+      if (!dir) return S(0);
+      const S ze = we * dg;
+      if (redist) re = we * (S)ime;
+      a1.add(prod_dw(re, ze));
+      if (flex) a2.add(prod_dw(qe, ze));
+      return ze;
     };
-    long long e = C.lo + threadIdx.x;
-    for (; e + (RED_U - 1) * BT < C.hi; e += RED_U * BT) {  // loads first, same order
-      S wv[RED_U], dv[RED_U], rv[RED_U], qv[RED_U];
-      float im[RED_U];
+    over_chunk<V>(
+        C.lo, C.hi,
+        [&](int v0, int nv) {
+          V wv, dv, rv, qv;
+          float mv[V::U][V::W];
 #pragma unroll
-      for (int u = 0; u < RED_U; ++u) {
-        const long long f = e + u * BT;
-        wv[u] = w[f];
-        im[u] = P.invmult[f];
-        dv[u] = (mode & 1) ? idg[f] : S(0);
-        rv[u] = ((mode & 1) && !(mode & 2)) ? r[f] : S(0);
-        qv[u] = ((mode & 1) && (mode & 4)) ? q[f] : S(0);
-      }
+          for (int k = 0; k < V::U; ++k) {
+            const int v = v0 + k * BT;
+            const long long e = C.lo + (long long)v * V::W;
+            if (v >= nv) continue;
+            wv.load(k, w + e);
+            load_mult<S>(mv[k], im + e);
+            if (dir) dv.load(k, idg + e);
+            if (dir && !redist) rv.load(k, r + e);
+            if (dir && flex) qv.load(k, q + e);
+          }
 #pragma unroll
-      for (int u = 0; u < RED_U; ++u) body(e + u * BT, wv[u], im[u], dv[u], rv[u], qv[u]);
+          for (int k = 0; k < V::U; ++k) {
+            const int v = v0 + k * BT;
+            const long long e = C.lo + (long long)v * V::W;
+            if (v >= nv) continue;
+#pragma unroll
+            for (int t = 0; t < V::W; ++t)
+              wv.v[k][t] = body(wv.v[k][t], mv[k][t], dv.v[k][t], rv.v[k][t], qv.v[k][t]);
+            if (dir) wv.store(k, z + e);
+            if (dir && redist) rv.store(k, r + e);
+          }
+        },
+        [&](long long e) {
+          S re = dir && !redist ? r[e] : S(0);
+          const S ze = body(w[e], im[e], dir ? idg[e] : S(0), re, dir && flex ? q[e] : S(0));
+          if (dir) z[e] = ze;
+          if (dir && redist) r[e] = re;
+        });
+    // slots 1 and 2 only where they are formed
+    if (flex) {
+      double v[3] = {a0.value(), a1.value(), a2.value()};
+      block_sums_f64<3>(v, sh);
+      if (threadIdx.x == 0)
+        for (int k = 0; k < 3; ++k) partials[(size_t)c * 4 + k] = v[k];
+    } else {
+      double v[2] = {a0.value(), a1.value()};
+      block_sums_f64<2>(v, sh);
+      if (threadIdx.x == 0)
+        for (int k = 0; k < (dir ? 2 : 1); ++k) partials[(size_t)c * 4 + k] = v[k];
     }
-    for (; e < C.hi; e += BT)
-      body(e, w[e], P.invmult[e], (mode & 1) ? idg[e] : S(0),
-           ((mode & 1) && !(mode & 2)) ? r[e] : S(0), ((mode & 1) && (mode & 4)) ? q[e] : S(0));
-    a0 = block_reduce_dw(a0, sh);
-    if (threadIdx.x == 0) partials[(size_t)c * 4 + 0] = dw_to_double(a0);
-    if (mode & 1) {
-      a1 = block_reduce_dw(a1, sh);
-      if (threadIdx.x == 0) partials[(size_t)c * 4 + 1] = dw_to_double(a1);
-      if (mode & 4) {
-        a2 = block_reduce_dw(a2, sh);
-        if (threadIdx.x == 0) partials[(size_t)c * 4 + 2] = dw_to_double(a2);
-      }
-    }
+    if (arrive && last_chunk(P, arrive + C.prob)) batch_fin_beta(P, slot, mode, partials, sh);
   }
 }
 
@@ -467,6 +575,7 @@ template <class S>
 __global__ void __launch_bounds__(BT)
     kb_update_p(const BProb* __restrict__ probs, const Chunk* __restrict__ chunks, int nchunks,
                 int slot) {
+  using V = Vec<S>;
   for (int c = blockIdx.x; c < nchunks; c += gridDim.x) {
     const Chunk C = chunks[c];
     const BProb& P = probs[C.prob];
@@ -474,15 +583,26 @@ __global__ void __launch_bounds__(BT)
     const S b = (S)P.sc[slot].beta;
     S* p = vec<S>(P, 3);
     const S* z = vec<S>(P, 2);
-    long long e = C.lo + threadIdx.x;
-    for (; e + (RED_U - 1) * BT < C.hi; e += RED_U * BT) {  // loads before stores
-      S zv[RED_U], pv[RED_U];
+    over_chunk<V>(
+        C.lo, C.hi,
+        [&](int v0, int nv) {
+          V zv, pv;
 #pragma unroll
-      for (int k = 0; k < RED_U; ++k) zv[k] = z[e + k * BT], pv[k] = p[e + k * BT];
+          for (int k = 0; k < V::U; ++k) {
+            const int v = v0 + k * BT;
+            const long long e = C.lo + (long long)v * V::W;
+            if (v < nv) zv.load(k, z + e), pv.load(k, p + e);
+          }
 #pragma unroll
-      for (int k = 0; k < RED_U; ++k) p[e + k * BT] = zv[k] + b * pv[k];
-    }
-    for (; e < C.hi; e += BT) p[e] = z[e] + b * p[e];
+          for (int k = 0; k < V::U; ++k) {
+            const int v = v0 + k * BT;
+            if (v >= nv) continue;
+#pragma unroll
+            for (int t = 0; t < V::W; ++t) pv.v[k][t] = zv.v[k][t] + b * pv.v[k][t];
+            pv.store(k, p + C.lo + (long long)v * V::W);
+          }
+        },
+        [&](long long e) { p[e] = z[e] + b * p[e]; });
   }
 }
 
@@ -547,49 +667,23 @@ __global__ void __launch_bounds__(BT)
   }
 }
 
-// ---- per-problem finishing kernels (one CTA per problem) --------------------------------------
-__device__ double sum_chunks(const double* partials, int c0, int c1, int slot, dw* sh) {
-  dw acc = {0.0f, 0.0f};
-  for (int c = c0 + threadIdx.x; c < c1; c += BT)
-    acc = dw_add(acc, dw_from_double(partials[(size_t)c * 4 + slot]));
-  acc = block_reduce_dw(acc, sh);
-  return dw_to_double(acc);
-}
-
+// ---- per-problem kernels -----------------------------------------------------------------------
+// the scalars of large batches, and FIN_OUTER from the partials of a preceding FIN_NORM: one CTA per
+// problem
 __global__ void __launch_bounds__(BT)
-    kb_fin_alpha(BProb* __restrict__ probs, int slot, const double* __restrict__ partials) {
-  __shared__ dw sh[32];
-  BProb& P = probs[blockIdx.x];
-  CgScal* sc = &P.sc[slot];
-  if (*(volatile int*)&sc->done) return;
-  const double qp = sum_chunks(partials, P.chunk0, P.chunk1, 0, sh);
-  if (threadIdx.x != 0) return;
-  sc->qp = qp;
-  if (!(qp > 0.0) || !isfinite(qp) || !isfinite(sc->rz)) {
-    sc->status = FE_ERR_BREAKDOWN;
-    sc->done = 1;
-  } else {
-    sc->alpha = sc->rz / qp;
-  }
+    kb_fin_alpha(const BProb* __restrict__ probs, int slot, const double* __restrict__ partials) {
+  __shared__ double sh[SUM_MAX * SUM_THREADS];
+  const BProb& P = probs[blockIdx.x];
+  if (*(volatile const int*)&P.sc[slot].done) return;
+  batch_fin_alpha(P, slot, partials, sh);
 }
-
-// mode: FIN_INIT_B, FIN_INIT_R, FIN_ITER, FIN_NORM, FIN_OUTER (fe_cgcore.h); tolerances and the
-// FCG switch are per problem (slot 0: the outer or FP64 solve, slot 1: the inner FP32 solve)
 __global__ void __launch_bounds__(BT)
-    kb_fin_beta(BProb* __restrict__ probs, int slot, int mode, const double* __restrict__ partials) {
-  __shared__ dw sh[32];
-  BProb& P = probs[blockIdx.x];
-  CgScal* sc = &P.sc[slot];
-  if (*(volatile int*)&sc->done) return;
-  const int flexible = slot == 0 ? P.flexible : 0;
-  const double rtol = slot == 0 ? P.rtol : sc->rtol;
-  const double rn2 = sum_chunks(partials, P.chunk0, P.chunk1, 0, sh);
-  const double rz = (mode == FIN_INIT_R || mode == FIN_ITER) ? sum_chunks(partials, P.chunk0, P.chunk1, 1, sh) : 0.0;
-  const double qz = (mode == FIN_ITER && flexible) ? sum_chunks(partials, P.chunk0, P.chunk1, 2, sh) : 0.0;
-  if (threadIdx.x != 0) return;
-  const double rel = mode == FIN_INIT_B ? 0.0 : fin_rel(sc, rn2);
-  const double beta = mode == FIN_ITER ? fin_new_beta(sc, rz, qz, flexible) : 0.0;
-  fin_scalars(sc, rn2, rz, rel, beta, rtol, mode);
+    kb_fin_beta(const BProb* __restrict__ probs, int slot, int mode,
+                const double* __restrict__ partials) {
+  __shared__ double sh[SUM_MAX * SUM_THREADS];
+  const BProb& P = probs[blockIdx.x];
+  if (*(volatile const int*)&P.sc[slot].done) return;
+  batch_fin_beta(P, slot, mode, partials, sh);
 }
 
 // reset the inner scalars for a new inner solve (done mirrors the outer state)
@@ -742,6 +836,13 @@ fe_status fe_batch_build(FeBatch* B) {
     FE_TRY(fe_dalloc((void**)&B->d_partials, pbytes + pbytes / 2, B->st, "batch partials"));
     B->cap_partials = pbytes + pbytes / 2;
   }
+  if (B->cap_arrive < (size_t)np) {
+    fe_dfree(B->d_arrive, B->st);
+    B->d_arrive = nullptr;
+    FE_TRY(fe_dalloc((void**)&B->d_arrive, 2 * (size_t)np * sizeof(unsigned), B->st, "batch arrivals"));
+    B->cap_arrive = 2 * (size_t)np;
+    FE_CUDA(cudaMemsetAsync(B->d_arrive, 0, B->cap_arrive * sizeof(unsigned), B->st), "batch arrivals");
+  }
   if (!B->d_counter)
     FE_TRY(fe_dalloc((void**)&B->d_counter, 64 * sizeof(unsigned long long), B->st, "counter"));
   FE_TRY(up((void**)&B->d_sc, &B->cap_sc, nullptr, 0));
@@ -755,7 +856,7 @@ fe_status fe_batch_build(FeBatch* B) {
 }
 
 template <int N, class V>
-static fe_status launch_apply_degree(FeBatch* B, int slot, int src) {
+static fe_status launch_apply_degree(FeBatch* B, int slot, int src, cudaStream_t st) {
   constexpr int f = std::is_same<V, dw2>::value ? 0 : 1;
   const long long lo = B->tile_lo[f][N], hi = B->tile_hi[f][N];
   if (hi <= lo) return FE_OK;
@@ -775,50 +876,95 @@ static fe_status launch_apply_degree(FeBatch* B, int slot, int src) {
     if (dev >= 0 && dev < 64) per_sm_dev[dev] = per_sm;
   }
   const long long grid = std::min<long long>(hi - lo, 152LL * per_sm);
-  kb_apply_n<N, V><<<(unsigned)grid, Sh::THREADS, smem, B->st>>>(
+  kb_apply_n<N, V><<<(unsigned)grid, Sh::THREADS, smem, st>>>(
       B->d_probs, (const Tile*)B->d_tiles, lo, hi, slot, f == 0 ? FE_F64 : FE_F32,
       src, B->d_counter + N);
   return fe_cuda_check(cudaGetLastError(), "batch apply launch");
 }
 
+template <class V>
+static fe_status launch_apply_degree(FeBatch* B, int n, int slot, int src, cudaStream_t st) {
+  switch (n) {
+    case 2: return launch_apply_degree<2, V>(B, slot, src, st);
+    case 3: return launch_apply_degree<3, V>(B, slot, src, st);
+    case 4: return launch_apply_degree<4, V>(B, slot, src, st);
+    case 5: return launch_apply_degree<5, V>(B, slot, src, st);
+    case 6: return launch_apply_degree<6, V>(B, slot, src, st);
+    case 7: return launch_apply_degree<7, V>(B, slot, src, st);
+    default: return launch_apply_degree<8, V>(B, slot, src, st);
+  }
+}
+
+// The applies of the degrees present, side by side on forked streams: in a small batch each alone leaves
+// most of the SMs idle (16 problems of degrees 2, 3, 5 and 7: 7, 7, 15 and 24 us one after the other).
 template <class S>
 static fe_status launch_apply_batched(FeBatch* B, int slot, int src = 0) {
   using V = typename std::conditional<sizeof(S) == 8, dw2, float>::type;
+  constexpr int f = sizeof(S) == 8 ? 0 : 1;
   FE_CUDA(cudaMemsetAsync(B->d_counter, 0, (FE_MAXN + 1) * sizeof(unsigned long long), B->st),
           "counter reset");
-  FE_TRY((launch_apply_degree<2, V>(B, slot, src)));
-  FE_TRY((launch_apply_degree<3, V>(B, slot, src)));
-  FE_TRY((launch_apply_degree<4, V>(B, slot, src)));
-  FE_TRY((launch_apply_degree<5, V>(B, slot, src)));
-  FE_TRY((launch_apply_degree<6, V>(B, slot, src)));
-  FE_TRY((launch_apply_degree<7, V>(B, slot, src)));
-  return launch_apply_degree<8, V>(B, slot, src);
+  int deg[FE_MAXN], nd = 0;
+  for (int n = FE_MAXN; n >= 2; --n)  // the largest degree on the batch's own stream
+    if (B->tile_hi[f][n] > B->tile_lo[f][n]) deg[nd++] = n;
+  const int forks = std::min(nd - 1, FeBatch::FORKS);
+  if (forks > 0) {
+    for (int k = 0; k <= forks; ++k) {
+      if (k < forks && !B->fork_st[k])
+        FE_CUDA(cudaStreamCreateWithFlags(&B->fork_st[k], cudaStreamNonBlocking), "batch fork");
+      if (!B->fork_ev[k])
+        FE_CUDA(cudaEventCreateWithFlags(&B->fork_ev[k], cudaEventDisableTiming), "batch fork");
+    }
+    FE_CUDA(cudaEventRecord(B->fork_ev[forks], B->st), "batch fork");
+    for (int k = 0; k < forks; ++k)
+      FE_CUDA(cudaStreamWaitEvent(B->fork_st[k], B->fork_ev[forks], 0), "batch fork");
+  }
+  for (int k = 0; k < nd; ++k)
+    FE_TRY((launch_apply_degree<V>(B, deg[k], slot, src,
+                                   k == 0 ? B->st : B->fork_st[(k - 1) % FeBatch::FORKS])));
+  for (int k = 0; k < forks; ++k) {
+    FE_CUDA(cudaEventRecord(B->fork_ev[k], B->fork_st[k]), "batch join");
+    FE_CUDA(cudaStreamWaitEvent(B->st, B->fork_ev[k], 0), "batch join");
+  }
+  return FE_OK;
 }
 
 template <class S>
 static fe_status launch_dss_batched(FeBatch* B, int slot) {
   for (int axis = 2; axis >= 0; --axis)
     if (B->ndch[axis] > 0)
-      kb_dss<S><<<grid_chunks((B->ndch[axis] + BT / 32 - 1) / (BT / 32)), BT, 0, B->st>>>(
+      kb_dss<S><<<grid_chunks((B->ndch[axis] * DSS_TEAM + BT - 1) / BT), BT, 0, B->st>>>(
           B->d_probs, (const DssRow*)B->d_dch[axis], B->ndch[axis], slot, axis);
   return fe_cuda_check(cudaGetLastError(), "batch dss launch");
+}
+
+// Arrival counters of the kernels that finish the scalars themselves: for batches whose chunks are all
+// resident at once.  In larger ones a CTA waits at the end of each chunk for its arrival (about the
+// time of the chunk's own traffic), and kernels of their own do it (64 problems of 135 million entries:
+// 3865 ms with arrivals, 3731 without).
+static unsigned* arrivals(const FeBatch* B) { return B->nvch <= 152 * 8 ? B->d_arrive : nullptr; }
+template <class S>
+static void launch_precond_batched(FeBatch* B, int slot, int pmode, int mode) {
+  unsigned* arrive = arrivals(B);
+  kb_precond<S><<<grid_chunks(B->nvch), BT, 0, B->st>>>(B->d_probs, (const Chunk*)B->d_vch, B->nvch, slot,
+                                                        pmode, mode, B->d_partials, arrive);
+  if (!arrive)
+    kb_fin_beta<<<(unsigned)B->hp.size(), BT, 0, B->st>>>(B->d_probs, slot, mode, B->d_partials);
 }
 
 // one PCG iteration of every active problem on vectors of type S, scalars `slot`
 template <class S>
 fe_status fe_batch_iteration(FeBatch* B, int slot, int redistribute) {
   const int flexible = slot == 0 ? B->any_flexible : 0;
-  const int np = (int)B->hp.size();
   const unsigned g = grid_chunks(B->nvch);
   const Chunk* ch = (const Chunk*)B->d_vch;
   FE_TRY(launch_apply_batched<S>(B, slot));
-  kb_qp<S><<<g, BT, 0, B->st>>>(B->d_probs, ch, B->nvch, slot, B->d_partials);
-  kb_fin_alpha<<<np, BT, 0, B->st>>>(B->d_probs, slot, B->d_partials);
+  unsigned* arrive = arrivals(B);
+  kb_qp<S><<<g, BT, 0, B->st>>>(B->d_probs, ch, B->nvch, slot, B->d_partials, arrive);
+  if (!arrive)
+    kb_fin_alpha<<<(unsigned)B->hp.size(), BT, 0, B->st>>>(B->d_probs, slot, B->d_partials);
   kb_update_ur<S><<<g, BT, 0, B->st>>>(B->d_probs, ch, B->nvch, slot, !redistribute);
   FE_TRY(launch_dss_batched<S>(B, slot));
-  kb_precond<S><<<g, BT, 0, B->st>>>(B->d_probs, ch, B->nvch, slot,
-                                     1 | (redistribute ? 2 : 0) | (flexible ? 4 : 0), B->d_partials);
-  kb_fin_beta<<<np, BT, 0, B->st>>>(B->d_probs, slot, FIN_ITER, B->d_partials);
+  launch_precond_batched<S>(B, slot, 1 | (redistribute ? 2 : 0) | (flexible ? 4 : 0), FIN_ITER);
   kb_update_p<S><<<g, BT, 0, B->st>>>(B->d_probs, ch, B->nvch, slot);
   return fe_cuda_check(cudaGetLastError(), "batch iteration launch");
 }
@@ -834,8 +980,7 @@ fe_status fe_batch_norm(FeBatch* B, int slot, int src, int mode, int redistribut
   kb_copy<S><<<g, BT, 0, B->st>>>(B->d_probs, ch, B->nvch, slot, 5, src);
   FE_TRY(launch_dss_batched<S>(B, slot));
   const int pm = (mode == FIN_INIT_R) ? (1 | (redistribute ? 2 : 0)) : 0;
-  kb_precond<S><<<g, BT, 0, B->st>>>(B->d_probs, ch, B->nvch, slot, pm, B->d_partials);
-  kb_fin_beta<<<np, BT, 0, B->st>>>(B->d_probs, slot, mode, B->d_partials);
+  launch_precond_batched<S>(B, slot, pm, mode);
   if (mode == FIN_INIT_R) kb_copy<S><<<g, BT, 0, B->st>>>(B->d_probs, ch, B->nvch, slot, 3, 2);
   return fe_cuda_check(cudaGetLastError(), "batch norm launch");
 }
@@ -862,8 +1007,7 @@ fe_status fe_batch_inner_start(FeBatch* B) {
   FE_TRY(fe_batch_norm<float>(B, 1, 1, FIN_INIT_B, 0));
   kb_copy<float><<<g, BT, 0, B->st>>>(B->d_probs, ch, B->nvch, 1, 5, 1);
   FE_TRY(launch_dss_batched<float>(B, 1));
-  kb_precond<float><<<g, BT, 0, B->st>>>(B->d_probs, ch, B->nvch, 1, 1 | 2, B->d_partials);
-  kb_fin_beta<<<np, BT, 0, B->st>>>(B->d_probs, 1, FIN_INIT_R, B->d_partials);
+  launch_precond_batched<float>(B, 1, 1 | 2, FIN_INIT_R);
   kb_keep_direction<<<g, BT, 0, B->st>>>(B->d_probs, ch, B->nvch);
   return fe_cuda_check(cudaGetLastError(), "batch run start");
 }
@@ -897,6 +1041,11 @@ FeBatch::~FeBatch() {
   for (int a = 0; a < 3; ++a) fe_dfree(d_dch[a], st);
   fe_dfree(d_partials, st);
   fe_dfree(d_counter, st);
+  fe_dfree(d_arrive, st);
+  for (cudaEvent_t e : fork_ev)
+    if (e) cudaEventDestroy(e);
+  for (cudaStream_t f : fork_st)
+    if (f) cudaStreamDestroy(f);
   fe_dfree(d_sc, st);
   if (st) cudaStreamSynchronize(st);
   cudaFreeHost(hsc);

@@ -43,6 +43,12 @@ struct FeBatch {
   double* d_partials = nullptr;
   size_t cap_partials = 0;
   unsigned long long* d_counter = nullptr;
+  unsigned* d_arrive = nullptr;  // per problem: chunks whose partials are written, 0 between launches
+  size_t cap_arrive = 0;
+  // the persistent applies of different degrees run side by side: streams forked from and joined to st
+  static constexpr int FORKS = 3;
+  cudaStream_t fork_st[FORKS] = {};
+  cudaEvent_t fork_ev[FORKS + 1] = {};
   CgScal* d_sc = nullptr;  // gathered scalar records for one readback
   size_t cap_sc = 0;
   cudaStream_t st = nullptr;

@@ -203,9 +203,9 @@ __global__ void k_update_p(S* __restrict__ p, const S* __restrict__ z, const CgS
 // diag (measured: binary64 FMAs for <r,z> there made it slower, 165 -> 202 us at Q3 64^3)
 template <class S>
 struct AccDw {
-  dw v = {0.0f, 0.0f};
-  __device__ __forceinline__ void add_prod(S a, S b) { v = dw_add(v, prod_dw(a, b)); }
-  __device__ __forceinline__ dw value() const { return v; }
+  Sum2 v;
+  __device__ __forceinline__ void add_prod(S a, S b) { v.add(prod_dw(a, b)); }
+  __device__ __forceinline__ double value() const { return v.value(); }
 };
 
 // residual norm, convergence test and beta
@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(RED_THREADS)
     k_qp(const S* __restrict__ q, const S* __restrict__ p, double* partials, unsigned* count,
          CgScal* sc, long long n, double* hist) {
   if (*(volatile const int*)&sc->done) return;
-  __shared__ double sh[SUM_THREADS];
+  __shared__ double sh[SUM_MAX * SUM_THREADS];
   Acc<S> acc;
   const long long STRIDE = (long long)gridDim.x * RED_THREADS;
   constexpr int QU = stream_u<S>();
@@ -268,8 +268,9 @@ __global__ void __launch_bounds__(RED_THREADS)
     for (int u = 0; u < QU; ++u) acc.add_prod(qv[u], pv[u]);
   }
   for (; e < n; e += STRIDE) acc.add_prod(q[e], p[e]);
-  const double v = block_sum_f64(acc.value(), sh);
-  if (threadIdx.x == 0) partials[blockIdx.x] = v;
+  double v[1] = {acc.value()};
+  block_sums_f64<1>(v, sh);
+  if (threadIdx.x == 0) partials[blockIdx.x] = v[0];
   if (last_cta(count)) fin_alpha(partials, (int)gridDim.x, sc, hist, sh);
 }
 
@@ -291,12 +292,12 @@ __global__ void __launch_bounds__(RED_THREADS)
     else
       return w[f];
   };
-  __shared__ double sh[SUM_THREADS];
-  dw a0 = {0.0f, 0.0f};
+  __shared__ double sh[SUM_MAX * SUM_THREADS];
+  Sum2 a0;
   AccDw<S> a1, a2;
   auto body = [&](long long e, S we, float im, S idg, S rv, S qv) {
     const dw w2 = prod_dw(we, we);
-    a0 = dw_add(a0, {w2.h * im, w2.l * im});  // im: a power of two or zero, exact scaling
+    a0.add({w2.h * im, w2.l * im});  // im: a power of two or zero, exact scaling
     if (z) {
       const S ze = we * idg;
       z[e] = ze;
@@ -332,15 +333,17 @@ __global__ void __launch_bounds__(RED_THREADS)
   for (; e < n; e += STRIDE)
     body(e, assembled(e), invmult[e], z ? invdiag[e] : S(0), (z && !redistribute) ? r[e] : S(0),
          (z && q) ? q[e] : S(0));
-  const double v0 = block_sum_f64(dw_to_double(a0), sh);
-  if (threadIdx.x == 0) partials[0 * RED_BLOCKS + blockIdx.x] = v0;
-  if (z) {
-    const double v1 = block_sum_f64(dw_to_double(a1.value()), sh);
-    if (threadIdx.x == 0) partials[1 * RED_BLOCKS + blockIdx.x] = v1;
-    if (q) {
-      const double v2 = block_sum_f64(dw_to_double(a2.value()), sh);
-      if (threadIdx.x == 0) partials[2 * RED_BLOCKS + blockIdx.x] = v2;
-    }
+  // slots 1 and 2 only where they are formed
+  if (q) {
+    double v[3] = {a0.value(), a1.value(), a2.value()};
+    block_sums_f64<3>(v, sh);
+    if (threadIdx.x == 0)
+      for (int k = 0; k < 3; ++k) partials[k * RED_BLOCKS + blockIdx.x] = v[k];
+  } else {
+    double v[2] = {a0.value(), a1.value()};
+    block_sums_f64<2>(v, sh);
+    if (threadIdx.x == 0)
+      for (int k = 0; k < (z ? 2 : 1); ++k) partials[k * RED_BLOCKS + blockIdx.x] = v[k];
   }
   if (last_cta(count)) fin_beta(partials, (int)gridDim.x, sc, fin, sh);
 }
@@ -376,7 +379,7 @@ __global__ void __launch_bounds__(RED_THREADS)
 // outer FCG scalars: init rz = <r,z>; iteration beta = -<q,z>/<q,p>, rz = <r,z>
 __global__ void __launch_bounds__(RED_THREADS)
     k_fin_fcg(const double* __restrict__ partials, CgScal* __restrict__ sc, int init) {
-  __shared__ double sh[SUM_THREADS];
+  __shared__ double sh[SUM_MAX * SUM_THREADS];
   double v[2];
   sum_slots<2>(partials + RED_BLOCKS, RED_BLOCKS, RED_BLOCKS, v, sh);
   if (threadIdx.x != 0) return;

@@ -52,24 +52,30 @@ __device__ __forceinline__ double block_reduce_f64(double v, double* sh /* [32] 
   return v;
 }
 
-// The same for CTAs of any size up to 256, summed by one warp: an SM takes 19 cycles for a warp's
-// binary64 addition, and a tree in every warp has 80 of them per CTA where this has 13.
-constexpr int SUM_THREADS = 256;
-__device__ __forceinline__ double block_sum_f64(double v, double* sh /* [SUM_THREADS] */) {
-  sh[threadIdx.x] = v;
+// The same for NS values and CTAs of any size up to 256, summed by one warp: an SM takes 19 cycles for a
+// warp's binary64 addition, and a tree in every warp has 80 of them per CTA and value where this has 13.
+constexpr int SUM_THREADS = 256, SUM_MAX = 3;
+template <int NS>
+__device__ __forceinline__ void block_sums_f64(double (&v)[NS], double* sh /* [NS * SUM_THREADS] */) {
+  static_assert(NS <= SUM_MAX, "shared memory of the callers");
+#pragma unroll
+  for (int s = 0; s < NS; ++s) sh[s * SUM_THREADS + threadIdx.x] = v[s];
   __syncthreads();
   if (threadIdx.x < 32) {
     const int n = blockDim.x, lanes = min(32, n);
-    for (int t = threadIdx.x + 32; t < n; t += 32) v += sh[t];
+    for (int t = threadIdx.x + 32; t < n; t += 32)
+#pragma unroll
+      for (int s = 0; s < NS; ++s) v[s] += sh[s * SUM_THREADS + t];
     const unsigned mask = lanes == 32 ? 0xffffffffu : (1u << lanes) - 1u;
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      const double t = __shfl_down_sync(mask, v, off);
-      if ((int)threadIdx.x + off < lanes) v += t;
-    }
+    for (int off = 16; off > 0; off >>= 1)
+#pragma unroll
+      for (int s = 0; s < NS; ++s) {
+        const double t = __shfl_down_sync(mask, v[s], off);
+        if ((int)threadIdx.x + off < lanes) v[s] += t;
+      }
   }
   __syncthreads();
-  return v;
 }
 
 // True in the last CTA of the grid to arrive, which then sees everything the others wrote before they
@@ -99,7 +105,8 @@ __device__ __forceinline__ void sum_slots(const double* partials, int nparts, in
 #pragma unroll
     for (int s = 0; s < NS; ++s) acc[s] += __ldcg(partials + (size_t)s * stride + b);
 #pragma unroll
-  for (int s = 0; s < NS; ++s) out[s] = block_sum_f64(acc[s], sh);
+  for (int s = 0; s < NS; ++s) out[s] = acc[s];
+  block_sums_f64<NS>(out, sh);
 }
 
 // alpha = <r,z>/<q,p> from the partials of <q,p>, by one CTA
@@ -119,6 +126,20 @@ __device__ __forceinline__ void fin_alpha(const double* partials, int nparts, Cg
   }
 }
 
+// A thread's running sum of double-word terms, compensated (Dot2 of Ogita, Rump and Oishi, "Accurate sum
+// and dot product", SIAM J. Sci. Comput. 2005: the accuracy of a sum in twice the working precision):
+// the TwoSum error and the term's low part go to a second float.  8 operations a term where a
+// normalised double-word sum takes 20.
+struct Sum2 {
+  float h = 0.0f, l = 0.0f;
+  __device__ __forceinline__ void add(dw t) {
+    const dw s = dw_two_sum(h, t.h);
+    h = s.h;
+    l = __fadd_rn(l, __fadd_rn(s.l, t.l));
+  }
+  __device__ __forceinline__ double value() const { return dw_to_double({h, l}); }
+};
+
 // A thread's running sum of products in a pairing: float vectors in double-word (exact products);
 // double vectors in binary64 FMAs on the FP64 pipe, one per product, which costs less than
 // converting both factors to double-word
@@ -133,9 +154,9 @@ template <class S>
 struct Acc;
 template <>
 struct Acc<float> {
-  dw v = {0.0f, 0.0f};
-  __device__ __forceinline__ void add_prod(float a, float b) { v = dw_add(v, prod_dw(a, b)); }
-  __device__ __forceinline__ double value() const { return dw_to_double(v); }
+  Sum2 v;
+  __device__ __forceinline__ void add_prod(float a, float b) { v.add(prod_dw(a, b)); }
+  __device__ __forceinline__ double value() const { return v.value(); }
 };
 template <>
 struct Acc<double> {
@@ -148,7 +169,8 @@ struct Acc<double> {
 template <class S>
 __device__ __forceinline__ void cg_finish_apply(const CgApply& cg, const Acc<S>& acc) {
   __shared__ double sh[SUM_THREADS];
-  const double v = block_sum_f64(acc.value(), sh);
-  if (threadIdx.x == 0) cg.partials[blockIdx.x] = v;
+  double v[1] = {acc.value()};
+  block_sums_f64<1>(v, sh);
+  if (threadIdx.x == 0) cg.partials[blockIdx.x] = v[0];
   if (last_cta(cg.count)) fin_alpha(cg.partials, (int)gridDim.x, cg.sc, cg.hist, sh);
 }
