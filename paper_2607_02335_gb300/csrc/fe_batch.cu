@@ -295,7 +295,7 @@ __device__ __forceinline__ void batch_fin_beta(const BProb& P, int slot, int mod
   }
   if (threadIdx.x == 0) sh[0] = v[0];
   __syncthreads();
-  if (threadIdx.x == 32 && mode != FIN_INIT_B) sh[1] = fin_rel(sc, sh[0]);
+  if (threadIdx.x == 32 && mode != FIN_INIT_B) sh[1] = fin_rel(sc, sh[0], mode);
   const double beta = threadIdx.x == 0 && mode == FIN_ITER ? fin_new_beta(sc, v[1], v[2], flexible) : 0.0;
   __syncthreads();
   if (threadIdx.x == 0) fin_scalars(sc, v[0], v[1], sh[1], beta, rtol, mode);
@@ -621,49 +621,106 @@ __global__ void __launch_bounds__(BT)
   }
 }
 
-// inner start: r32 = s (S r64) / mult with s = 1/sqrt(rnorm2) (w64 holds S r64), d32 = 0
+// a value formed by one thread for its CTA (divisions and square roots in every thread would queue on the
+// FP64 pipe: 35 us for the run start of a 16-problem batch)
+template <class F>
+__device__ __forceinline__ double by_one_thread(double* sh, F f) {
+  __syncthreads();  // the previous chunk's value has been read
+  if (threadIdx.x == 0) *sh = f();
+  __syncthreads();
+  return *sh;
+}
+
+// start of an FP32 run (k_start_run of fe_cg.cu): w64 holds S r64, s = 1/sqrt(rnorm2); r32 = s w / mult,
+// z32 = D^{-1} (s w), d32 = 0, and the run's initial scalars (FIN_START)
 __global__ void __launch_bounds__(BT)
-    kb_to_inner(const BProb* __restrict__ probs, const Chunk* __restrict__ chunks, int nchunks) {
+    kb_start_run(const BProb* __restrict__ probs, const Chunk* __restrict__ chunks, int nchunks,
+                 double* partials, unsigned* arrive) {
+  __shared__ double sh[SUM_MAX * SUM_THREADS];
+  __shared__ double scale;
   for (int c = blockIdx.x; c < nchunks; c += gridDim.x) {
     const Chunk C = chunks[c];
     const BProb& P = probs[C.prob];
     if (*(volatile const int*)&P.sc[0].done) continue;
-    const double s = 1.0 / sqrt(P.sc[0].rnorm2);
-    for (long long e = C.lo + threadIdx.x; e < C.hi; e += BT) {
-      P.r32[e] = (float)(s * P.w64[e] * (double)P.invmult[e]);
-      P.d32[e] = 0.0f;
+    const double s = by_one_thread(&scale, [&] { return 1.0 / sqrt(P.sc[0].rnorm2); });
+    Sum2 a0;
+    Acc<float> a1;
+    for (long long e = C.lo + threadIdx.x; e < C.hi; e += RED_U * BT) {
+      double wv[RED_U];
+      float im[RED_U], dg[RED_U];
+#pragma unroll
+      for (int u = 0; u < RED_U; ++u) {
+        const long long f = e + u * BT;
+        if (f < C.hi) wv[u] = P.w64[f], im[u] = P.invmult[f], dg[u] = P.invdiag32[f];
+      }
+#pragma unroll
+      for (int u = 0; u < RED_U; ++u) {
+        const long long f = e + u * BT;
+        if (f >= C.hi) continue;
+        const float we = (float)(s * wv[u]), ze = we * dg[u], re = we * im[u];
+        P.r32[f] = re;
+        P.z32[f] = ze;
+        P.d32[f] = 0.0f;
+        const dw w2 = prod_dw(we, we);
+        a0.add({w2.h * im[u], w2.l * im[u]});
+        a1.add_prod(re, ze);
+      }
     }
+    double v[2] = {a0.value(), a1.value()};
+    block_sums_f64<2>(v, sh);
+    if (threadIdx.x == 0)
+      for (int k = 0; k < 2; ++k) partials[(size_t)c * 4 + k] = v[k];
+    if (arrive && last_chunk(P, arrive + C.prob)) batch_fin_beta(P, 1, FIN_START, partials, sh);
   }
 }
 
 // reliable update: x64 += d32 / s (s = 1/||G^T r|| of the run's residual)
 __global__ void __launch_bounds__(BT)
     kb_correct(const BProb* __restrict__ probs, const Chunk* __restrict__ chunks, int nchunks) {
+  __shared__ double scale;
   for (int c = blockIdx.x; c < nchunks; c += gridDim.x) {
     const Chunk C = chunks[c];
     const BProb& P = probs[C.prob];
     if (*(volatile const int*)&P.sc[0].done) continue;
-    const double inv_s = sqrt(P.sc[0].rnorm2);
-    for (long long e = C.lo + threadIdx.x; e < C.hi; e += BT) P.x64[e] += inv_s * (double)P.d32[e];
+    const double inv_s = by_one_thread(&scale, [&] { return sqrt(P.sc[0].rnorm2); });
+    for (long long e = C.lo + threadIdx.x; e < C.hi; e += RED_U * BT) {
+      double xv[RED_U];
+      float dv[RED_U];
+#pragma unroll
+      for (int u = 0; u < RED_U; ++u)
+        if (e + u * BT < C.hi) xv[u] = P.x64[e + u * BT], dv[u] = P.d32[e + u * BT];
+#pragma unroll
+      for (int u = 0; u < RED_U; ++u)
+        if (e + u * BT < C.hi) P.x64[e + u * BT] = xv[u] + inv_s * (double)dv[u];
+    }
   }
 }
 
-// start of a run: p32 = z32 (a problem's first run) or p32 = z32 + c p32, the direction of the
-// previous run kept in the new scale: c = beta (s/s_old) with beta = <r', z'> / (rz_old
-// (s/s_old)^2), rz_old = <r_{k-1}, z_{k-1}> in the old scale (sc[0].rz_new), s_old in sc[0].qz
+// search direction at the start of an FP32 run: z for a problem's first run (sc[0].pad), else the
+// previous run's direction kept across the reliable update, p = z + beta p in the new scale with
+// beta = <r',z'> / <r_{k-1},z_{k-1}> (saved by kb_save_run in sc[0].rz_new, the scale in sc[0].qz)
 __global__ void __launch_bounds__(BT)
     kb_keep_direction(const BProb* __restrict__ probs, const Chunk* __restrict__ chunks, int nchunks) {
+  __shared__ double scale;
   for (int c = blockIdx.x; c < nchunks; c += gridDim.x) {
     const Chunk C = chunks[c];
     const BProb& P = probs[C.prob];
     if (*(volatile const int*)&P.sc[0].done) continue;
-    if (P.sc[0].pad) {  // first run: p = z (the buffer's old contents are not read)
-      for (long long e = C.lo + threadIdx.x; e < C.hi; e += BT) P.p32[e] = P.z32[e];
-      continue;
+    const bool first = P.sc[0].pad != 0;  // the buffer's old contents are not read
+    const float cf = (float)by_one_thread(&scale, [&] {
+      if (first) return 0.0;
+      const double ratio = (1.0 / sqrt(P.sc[0].rnorm2)) / P.sc[0].qz;
+      return P.sc[1].rz / (P.sc[0].rz_new * ratio);
+    });
+    for (long long e = C.lo + threadIdx.x; e < C.hi; e += RED_U * BT) {
+      float zv[RED_U], pv[RED_U];
+#pragma unroll
+      for (int u = 0; u < RED_U; ++u)
+        if (e + u * BT < C.hi) zv[u] = P.z32[e + u * BT], pv[u] = first ? 0.0f : P.p32[e + u * BT];
+#pragma unroll
+      for (int u = 0; u < RED_U; ++u)
+        if (e + u * BT < C.hi) P.p32[e + u * BT] = fmaf(cf, pv[u], zv[u]);
     }
-    const double ratio = (1.0 / sqrt(P.sc[0].rnorm2)) / P.sc[0].qz;
-    const float cf = (float)(P.sc[1].rz / (P.sc[0].rz_new * ratio));
-    for (long long e = C.lo + threadIdx.x; e < C.hi; e += BT) P.p32[e] = fmaf(cf, P.p32[e], P.z32[e]);
   }
 }
 
@@ -727,14 +784,22 @@ __global__ void kb_count_inner(BProb* __restrict__ probs, int nprob) {
   if (!probs[i].sc[0].done) in->stall_total += in->iter;
 }
 
-// r = b - q
+// r = b - q, also into w (whose sums over the interfaces follow)
 __global__ void __launch_bounds__(BT)
     kb_residual(const BProb* __restrict__ probs, const Chunk* __restrict__ chunks, int nchunks) {
   for (int c = blockIdx.x; c < nchunks; c += gridDim.x) {
     const Chunk C = chunks[c];
     const BProb& P = probs[C.prob];
     if (*(volatile const int*)&P.sc[0].done) continue;
-    for (long long e = C.lo + threadIdx.x; e < C.hi; e += BT) P.r64[e] = P.b64[e] - P.q64[e];
+    for (long long e = C.lo + threadIdx.x; e < C.hi; e += RED_U * BT) {
+      double bv[RED_U], qv[RED_U];
+#pragma unroll
+      for (int u = 0; u < RED_U; ++u)
+        if (e + u * BT < C.hi) bv[u] = P.b64[e + u * BT], qv[u] = P.q64[e + u * BT];
+#pragma unroll
+      for (int u = 0; u < RED_U; ++u)
+        if (e + u * BT < C.hi) P.r64[e + u * BT] = P.w64[e + u * BT] = bv[u] - qv[u];
+    }
   }
 }
 
@@ -971,21 +1036,17 @@ fe_status fe_batch_iteration(FeBatch* B, int slot, int redistribute) {
 template fe_status fe_batch_iteration<double>(FeBatch*, int, int);
 template fe_status fe_batch_iteration<float>(FeBatch*, int, int);
 
-// w = S(src) and the norm (and, with init_dir, z = D^{-1} w, p = z, <r,z>) of every active problem
-template <class S>
-fe_status fe_batch_norm(FeBatch* B, int slot, int src, int mode, int redistribute) {
-  const int np = (int)B->hp.size();
+// w = S(src) (src < 0: of what w holds) and the norm (FIN_INIT_R: also z = D^{-1} w, p = z, <r,z>) of
+// every active problem, in FP64
+fe_status fe_batch_norm(FeBatch* B, int src, int mode) {
   const unsigned g = grid_chunks(B->nvch);
   const Chunk* ch = (const Chunk*)B->d_vch;
-  kb_copy<S><<<g, BT, 0, B->st>>>(B->d_probs, ch, B->nvch, slot, 5, src);
-  FE_TRY(launch_dss_batched<S>(B, slot));
-  const int pm = (mode == FIN_INIT_R) ? (1 | (redistribute ? 2 : 0)) : 0;
-  launch_precond_batched<S>(B, slot, pm, mode);
-  if (mode == FIN_INIT_R) kb_copy<S><<<g, BT, 0, B->st>>>(B->d_probs, ch, B->nvch, slot, 3, 2);
+  if (src >= 0) kb_copy<double><<<g, BT, 0, B->st>>>(B->d_probs, ch, B->nvch, 0, 5, src);
+  FE_TRY(launch_dss_batched<double>(B, 0));
+  launch_precond_batched<double>(B, 0, mode == FIN_INIT_R ? 1 : 0, mode);
+  if (mode == FIN_INIT_R) kb_copy<double><<<g, BT, 0, B->st>>>(B->d_probs, ch, B->nvch, 0, 3, 2);
   return fe_cuda_check(cudaGetLastError(), "batch norm launch");
 }
-template fe_status fe_batch_norm<double>(FeBatch*, int, int, int, int);
-template fe_status fe_batch_norm<float>(FeBatch*, int, int, int, int);
 
 fe_status fe_batch_read(FeBatch* B) {
   const int np = (int)B->hp.size();
@@ -1003,11 +1064,9 @@ fe_status fe_batch_inner_start(FeBatch* B) {
   const unsigned g = grid_chunks(B->nvch);
   const Chunk* ch = (const Chunk*)B->d_vch;
   kb_reset_inner<<<(np + 127) / 128, 128, 0, B->st>>>(B->d_probs, np);
-  kb_to_inner<<<g, BT, 0, B->st>>>(B->d_probs, ch, B->nvch);
-  FE_TRY(fe_batch_norm<float>(B, 1, 1, FIN_INIT_B, 0));
-  kb_copy<float><<<g, BT, 0, B->st>>>(B->d_probs, ch, B->nvch, 1, 5, 1);
-  FE_TRY(launch_dss_batched<float>(B, 1));
-  launch_precond_batched<float>(B, 1, 1 | 2, FIN_INIT_R);
+  unsigned* arrive = arrivals(B);
+  kb_start_run<<<g, BT, 0, B->st>>>(B->d_probs, ch, B->nvch, B->d_partials, arrive);
+  if (!arrive) kb_fin_beta<<<np, BT, 0, B->st>>>(B->d_probs, 1, FIN_START, B->d_partials);
   kb_keep_direction<<<g, BT, 0, B->st>>>(B->d_probs, ch, B->nvch);
   return fe_cuda_check(cudaGetLastError(), "batch run start");
 }
@@ -1022,7 +1081,7 @@ fe_status fe_batch_inner_finish(FeBatch* B) {
   kb_correct<<<g, BT, 0, B->st>>>(B->d_probs, ch, B->nvch);
   FE_TRY(launch_apply_batched<double>(B, 0, 1));  // q = A x
   kb_residual<<<g, BT, 0, B->st>>>(B->d_probs, ch, B->nvch);
-  FE_TRY(fe_batch_norm<double>(B, 0, 1, FIN_NORM, 0));
+  FE_TRY(fe_batch_norm(B, -1, FIN_NORM));
   kb_fin_beta<<<np, BT, 0, B->st>>>(B->d_probs, 0, FIN_OUTER, B->d_partials);
   return fe_cuda_check(cudaGetLastError(), "batch reliable update");
 }
@@ -1100,7 +1159,7 @@ fe_status fe_batch_setup(FeBatch* B) {
   const unsigned g = grid_chunks(B->nvch);
   const Chunk* ch = (const Chunk*)B->d_vch;
   kb_init_scal<<<(np + 127) / 128, 128, 0, B->st>>>(B->d_probs, np);
-  FE_TRY(fe_batch_norm<double>(B, 0, 6, FIN_INIT_B, 0));  // ||G^T b||
+  FE_TRY(fe_batch_norm(B, 6, FIN_INIT_B));  // ||G^T b||
   FE_TRY(launch_apply_batched<double>(B, 0, 1));               // q = A x
   kb_residual<<<g, BT, 0, B->st>>>(B->d_probs, ch, B->nvch);
   return fe_cuda_check(cudaGetLastError(), "batch setup");
@@ -1114,8 +1173,8 @@ bool fe_batch_all_done(FeBatch* B, int slot) {
 
 fe_status fe_batch_start(FeBatch* B, bool mixed) {
   FE_TRY(fe_batch_setup(B));
-  if (!mixed) return fe_batch_norm<double>(B, 0, 1, FIN_INIT_R, 0);
-  FE_TRY(fe_batch_norm<double>(B, 0, 1, FIN_NORM, 0));
+  if (!mixed) return fe_batch_norm(B, -1, FIN_INIT_R);
+  FE_TRY(fe_batch_norm(B, -1, FIN_NORM));
   const int np = (int)B->hp.size();
   kb_fin_beta<<<np, BT, 0, B->st>>>(B->d_probs, 0, FIN_OUTER, B->d_partials);  // converged at x0?
   return fe_cuda_check(cudaGetLastError(), "batch start");

@@ -66,8 +66,7 @@ fe_status fe_batch_setup(FeBatch* B);  // fresh scalars, ||G^T b||, r = b - A x
 bool fe_batch_all_done(FeBatch* B, int slot);
 template <class S>
 fe_status fe_batch_iteration(FeBatch* B, int slot, int redistribute);
-template <class S>
-fe_status fe_batch_norm(FeBatch* B, int slot, int src, int mode, int redistribute);
+fe_status fe_batch_norm(FeBatch* B, int src, int mode);
 // mixed solves: start of an FP32 run, and its end with the FP64 reliable update
 fe_status fe_batch_inner_start(FeBatch* B);
 fe_status fe_batch_inner_finish(FeBatch* B);

@@ -88,21 +88,6 @@ __global__ void k_scale_vec(const double* src, double* dst, double s, long long 
     dst[e] = s * src[e];
 }
 
-// Inner right-hand side r32 = s * (S r) / mult, d32 = 0.  The dual residual r is unassembled: the
-// copies of a node hold partial integrals that cancel when summed, so near convergence single
-// copies are orders of magnitude larger than G^T r.  Rounding them to FP32 would destroy the
-// assembled value; the residual is therefore assembled in FP64 first (w = S r) and its value is
-// split evenly over the copies.  G^T r32 = s G^T r, and every pairing with a continuous vector is
-// unchanged (Lemma "Duality Pairing Identity").
-__global__ void k_to_inner(const double* __restrict__ w, const float* __restrict__ invmult,
-                           float* __restrict__ r32, float* __restrict__ d32, double s, long long n) {
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n;
-       e += (long long)gridDim.x * blockDim.x) {
-    r32[e] = (float)(s * w[e] * (double)invmult[e]);
-    d32[e] = 0.0f;
-  }
-}
-
 // x += d / s
 __global__ void k_correct(double* __restrict__ x, const float* __restrict__ d, double inv_s,
                           long long n) {
@@ -213,6 +198,7 @@ struct FinBeta {
   double rtol;  // negative: sc->rtol
   int mode, flexible;
   double* hist;
+  double keep = 0.0;  // FIN_START: beta / <r,z>
 };
 // by one CTA; the two divisions and the square root, long on the FP64 pipe, in two warps
 __device__ void fin_beta(const double* partials, int nparts, CgScal* sc, const FinBeta& f, double* sh) {
@@ -220,7 +206,7 @@ __device__ void fin_beta(const double* partials, int nparts, CgScal* sc, const F
   double v[3] = {0.0, 0.0, 0.0};
   if (f.mode == FIN_ITER && f.flexible) {
     sum_slots<3>(partials, nparts, RED_BLOCKS, v, sh);
-  } else if (f.mode == FIN_INIT_R || f.mode == FIN_ITER) {
+  } else if (f.mode == FIN_INIT_R || f.mode == FIN_ITER || f.mode == FIN_START) {
     double t[2];
     sum_slots<2>(partials, nparts, RED_BLOCKS, t, sh);
     v[0] = t[0], v[1] = t[1];
@@ -231,13 +217,15 @@ __device__ void fin_beta(const double* partials, int nparts, CgScal* sc, const F
   }
   if (threadIdx.x == 0) sh[0] = v[0];
   __syncthreads();
-  if (threadIdx.x == 32 && f.mode != FIN_INIT_B) rel = fin_rel(sc, sh[0]);
+  if (threadIdx.x == 32 && f.mode != FIN_INIT_B) rel = fin_rel(sc, sh[0], f.mode);
   const double beta =
       threadIdx.x == 0 && f.mode == FIN_ITER ? fin_new_beta(sc, v[1], v[2], f.flexible) : 0.0;
   __syncthreads();
   if (threadIdx.x != 0) return;
   const int k = sc->iter;
-  if (f.mode == FIN_INIT_R) sc->beta = 0.0;  // the first direction is z
+  // the direction the first iteration forms, z + beta p: p was z (beta = 0), or a kept direction
+  if (f.mode == FIN_INIT_R) sc->beta = 0.0;
+  if (f.mode == FIN_START) sc->beta = f.keep * v[1];
   fin_scalars(sc, v[0], v[1], rel, beta, f.rtol < 0.0 ? sc->rtol : f.rtol, f.mode);
   if (f.hist && f.mode == FIN_ITER) {
     f.hist[3 * k + 2] = sc->relres;
@@ -345,6 +333,54 @@ __global__ void __launch_bounds__(RED_THREADS)
     if (threadIdx.x == 0)
       for (int k = 0; k < (z ? 2 : 1); ++k) partials[k * RED_BLOCKS + blockIdx.x] = v[k];
   }
+  if (last_cta(count)) fin_beta(partials, (int)gridDim.x, sc, fin, sh);
+}
+
+// Start of an FP32 run on A d = s S(r)/mult, from w = S r in FP64 (assembled: every copy of a node holds
+// its value): r32 = s w / mult, z32 = D^{-1} (s w), d32 = 0, and the pairings sum (s w)^2/mult and
+// <r32, z32>; p = z where p is given.  The dual residual r is unassembled: the copies of a node hold
+// partial integrals that cancel when summed, so near convergence single copies are orders of magnitude
+// larger than G^T r.  Rounding them to FP32 would destroy the assembled value; the residual is therefore
+// assembled in FP64 first and its value is split evenly over the copies.  G^T r32 = s G^T r, and every
+// pairing with a continuous vector is unchanged (Lemma "Duality Pairing Identity").  S r32 is s w
+// rounded (exactly where mult is a power of two), so nothing is summed again: the separate passes (right-
+// hand side, copy, interface sums, norm, copy, interface sums, preconditioner, two readings of the
+// scalars by the host) made an outer step at Q3 32^3 0.15 ms longer than this one kernel (20 us) does.
+__global__ void __launch_bounds__(RED_THREADS)
+    k_start_run(const double* __restrict__ w, const float* __restrict__ invmult,
+                const float* __restrict__ invdiag, double s, float* __restrict__ r,
+                float* __restrict__ z, float* __restrict__ d, float* __restrict__ p, double* partials,
+                unsigned* count, CgScal* sc, long long n, const FinBeta fin) {
+  __shared__ double sh[SUM_MAX * SUM_THREADS];
+  Sum2 a0;
+  Acc<float> a1;
+  const long long STRIDE = (long long)gridDim.x * RED_THREADS;
+  for (long long e = (long long)blockIdx.x * RED_THREADS + threadIdx.x; e < n; e += RED_U * STRIDE) {
+    double wv[RED_U];
+    float im[RED_U], dg[RED_U];
+#pragma unroll
+    for (int u = 0; u < RED_U; ++u) {
+      const long long f = e + u * STRIDE;
+      if (f < n) wv[u] = w[f], im[u] = invmult[f], dg[u] = invdiag[f];
+    }
+#pragma unroll
+    for (int u = 0; u < RED_U; ++u) {
+      const long long f = e + u * STRIDE;
+      if (f >= n) continue;
+      const float we = (float)(s * wv[u]), ze = we * dg[u], re = we * im[u];
+      r[f] = re;
+      z[f] = ze;
+      d[f] = 0.0f;
+      if (p) p[f] = ze;
+      const dw w2 = prod_dw(we, we);
+      a0.add({w2.h * im[u], w2.l * im[u]});
+      a1.add_prod(re, ze);
+    }
+  }
+  double v[2] = {a0.value(), a1.value()};
+  block_sums_f64<2>(v, sh);
+  if (threadIdx.x == 0)
+    for (int k = 0; k < 2; ++k) partials[k * RED_BLOCKS + blockIdx.x] = v[k];
   if (last_cta(count)) fin_beta(partials, (int)gridDim.x, sc, fin, sh);
 }
 
@@ -604,10 +640,11 @@ fe_status read_scal(CgWork* w, int slot, CgScal* out) {
   return FE_OK;
 }
 
-// ||G^T v||^2 / bnorm into slot's scalars: w = S v, precond kernel without z
+// ||G^T v||^2 / bnorm into slot's scalars: w = S v (v null: v is in w already), precond kernel without z
 template <class S>
 fe_status residual_norm(const fe_mesh* m, CgWork* w, const S* v, S* wv, CgScal* sc, int mode) {
-  FE_CUDA(cudaMemcpyAsync(wv, v, w->n * sizeof(S), cudaMemcpyDeviceToDevice, w->st), "cg copy");
+  if (v)
+    FE_CUDA(cudaMemcpyAsync(wv, v, w->n * sizeof(S), cudaMemcpyDeviceToDevice, w->st), "cg copy");
   FE_TRY(fe_launch_dss(m, sizeof(S) == 8 ? FE_F64 : FE_F32, wv, w->st));
   k_precond<S, 0><<<red_grid(w->n), RED_THREADS, 0, w->st>>>(
       wv, nullptr, nullptr, nullptr, w->invmult, nullptr, w->partials, w->count, sc, w->n, 0, 0,
@@ -627,24 +664,26 @@ fe_status init_direction(const fe_mesh* m, CgWork* w, S* r, S* z, S* p, S* wv, c
   return fe_cuda_check(cudaGetLastError(), "init launch");
 }
 
+// start of an FP32 run (k_start_run); first: the direction is z, else z + keep <r,z> p
+fe_status launch_start_run(CgWork* w, double s, bool first, double keep) {
+  k_start_run<<<red_grid(w->n), RED_THREADS, 0, w->st>>>(
+      w->w, w->invmult, w->invdiag32, s, w->r32, w->z32, w->d32, first ? w->p32 : nullptr, w->partials,
+      w->count, &w->sc[1], w->n, {-1.0, FIN_START, 0, nullptr, first ? 0.0 : keep});
+  return fe_cuda_check(cudaGetLastError(), "run start launch");
+}
+
 // Inner FP32 PCG on A d = s S(r)/mult with s = 1/||G^T r|| (w must hold S r in FP64, rnorm2
 // its squared norm).  Returns the inner iteration count in *iters and the scale s.
 fe_status inner_solve(const fe_mesh* m, CgWork* w, int op, int flex, double rnorm2, double irtol,
                       int maxit, int* iters, double* s_out) {
-  const long long n = w->n;
   const double s = 1.0 / sqrt(rnorm2);
-  k_to_inner<<<grid_for(n), 256, 0, w->st>>>(w->w, w->invmult, w->r32, w->d32, s, n);
   FE_TRY(set_scal(w, 1, maxit, 20, irtol));
-  FE_TRY(residual_norm<float>(m, w, w->r32, w->w32, &w->sc[1], FIN_INIT_B));
-  FE_TRY(init_direction<float>(m, w, w->r32, w->z32, w->p32, w->w32, w->invdiag32, &w->sc[1], irtol));
+  FE_TRY(launch_start_run(w, s, true, 0.0));
   CgScal h;
-  FE_TRY(read_scal(w, 1, &h));
-  if (!h.done) {
-    if (!w->g32[flex])
-      FE_TRY((build_graph<float, float>(m, w, op, flex, w->d32, w->r32, w->z32, w->p32, w->q32,
-                                        w->w32, w->invdiag32, &w->sc[1], nullptr, &w->g32[flex])));
-    FE_TRY(run_until_done(w, w->g32[flex], 1, &h));
-  }
+  if (!w->g32[flex])
+    FE_TRY((build_graph<float, float>(m, w, op, flex, w->d32, w->r32, w->z32, w->p32, w->q32, w->w32,
+                                      w->invdiag32, &w->sc[1], nullptr, &w->g32[flex])));
+  FE_TRY(run_until_done(w, w->g32[flex], 1, &h));
   *iters = h.iter;
   *s_out = s;
   if (h.status == FE_ERR_BREAKDOWN && h.iter == 0) {
@@ -742,8 +781,8 @@ fe_status solve_reliable(const fe_mesh* m, CgWork* w, int op, const double* b, d
     // true FP64 residual of the current iterate; w = S r for the inner right-hand side
     ApplyLaunch L{m, op, w->x, w->q, w->st, nullptr};
     FE_TRY(fe_launch_apply_f64dw(L));
-    k_residual<<<grid_for(n), 256, 0, w->st>>>(b, w->q, w->r, n);
-    FE_TRY(residual_norm<double>(m, w, w->r, w->w, &w->sc[0], FIN_NORM));
+    k_residual<<<grid_for(n), 256, 0, w->st>>>(b, w->q, w->w, n);
+    FE_TRY(residual_norm<double>(m, w, nullptr, w->w, &w->sc[0], FIN_NORM));
     FE_TRY(read_scal(w, 0, &h));
     const double rel = sqrt(h.rnorm2 / bnorm2);
     res->rel_res = rel;
@@ -762,34 +801,14 @@ fe_status solve_reliable(const fe_mesh* m, CgWork* w, int op, const double* b, d
     // run the FP32 iteration down to delta, or to just below the outer target
     const double irtol = std::max(delta, 0.5 * opts->rtol / rel);
     FE_TRY(set_scal(w, 1, opts->maxit - total, 0, irtol));
-    // r32 = s (S r) / mult, d32 = 0
+    // p := z + beta p in the new scale (p and rz_old were in units of s_old):
+    // beta = <r', z'> / (rz_old (s / s_old)^2), times s / s_old for p
     const double s = 1.0 / sqrt(h.rnorm2);
-    k_to_inner<<<grid_for(n), 256, 0, w->st>>>(w->w, w->invmult, w->r32, w->d32, s, n);
-    FE_TRY(residual_norm<float>(m, w, w->r32, w->w32, &w->sc[1], FIN_INIT_B));
-    if (!have_p) {
-      FE_TRY(init_direction<float>(m, w, w->r32, w->z32, w->p32, w->w32, w->invdiag32, &w->sc[1],
-                                   irtol));
-      FE_TRY(read_scal(w, 1, &h));
-    } else {
-      // z = P r', <r', z>; p = z + beta p in the new scale (p and rz_old were in units of s_old)
-      FE_CUDA(cudaMemcpyAsync(w->w32, w->r32, n * sizeof(float), cudaMemcpyDeviceToDevice, w->st),
-              "cg copy");
-      FE_TRY(launch_precond<float>(m, w, w->w32, w->r32, nullptr, w->invdiag32, w->z32, &w->sc[1], 0, 1,
-                                   {irtol, FIN_INIT_R, 0, nullptr}));
-      FE_TRY(read_scal(w, 1, &h));
-      const double ratio = s / s_old;
-      const double beta = h.rz / (rz_old * ratio * ratio);
-      w->hsc[1].beta = beta * ratio;  // the run's first iteration forms z + (beta ratio) p
-      FE_CUDA(cudaMemcpyAsync(&w->sc[1].beta, &w->hsc[1].beta, sizeof(double), cudaMemcpyHostToDevice,
-                              w->st),
-              "keep direction");
-    }
-    if (!h.done) {
-      if (!w->g32[0])
-        FE_TRY((build_graph<float, float>(m, w, op, false, w->d32, w->r32, w->z32, w->p32, w->q32,
-                                          w->w32, w->invdiag32, &w->sc[1], nullptr, &w->g32[0])));
-      FE_TRY(run_until_done(w, w->g32[0], 1, &h));
-    }
+    FE_TRY(launch_start_run(w, s, !have_p, have_p ? s_old / (rz_old * s) : 0.0));
+    if (!w->g32[0])
+      FE_TRY((build_graph<float, float>(m, w, op, false, w->d32, w->r32, w->z32, w->p32, w->q32, w->w32,
+                                        w->invdiag32, &w->sc[1], nullptr, &w->g32[0])));
+    FE_TRY(run_until_done(w, w->g32[0], 1, &h));
     if (h.status == FE_ERR_BREAKDOWN) {
       *status = FE_ERR_BREAKDOWN;
       break;

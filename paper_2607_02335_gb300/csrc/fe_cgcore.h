@@ -17,12 +17,14 @@ struct CgScal {
 };
 
 // FIN_INIT_B: ||G^T b||^2.  FIN_INIT_R: initial residual, <r,z>.  FIN_ITER: residual, convergence,
-// beta.  FIN_NORM: residual only.  FIN_OUTER: residual, outer count, convergence.
-enum { FIN_INIT_B = 0, FIN_INIT_R = 1, FIN_ITER = 2, FIN_NORM = 3, FIN_OUTER = 4 };
+// beta.  FIN_NORM: residual only.  FIN_OUTER: residual, outer count, convergence.  FIN_START: FIN_INIT_B
+// and FIN_INIT_R of a run whose right-hand side is its initial residual.
+enum { FIN_INIT_B = 0, FIN_INIT_R = 1, FIN_ITER = 2, FIN_NORM = 3, FIN_OUTER = 4, FIN_START = 5 };
 
 // relative residual and beta of the new values
-__device__ __forceinline__ double fin_rel(const CgScal* sc, double rn2) {
-  return sc->bnorm2 > 0.0 ? sqrt(rn2 / sc->bnorm2) : 0.0;
+__device__ __forceinline__ double fin_rel(const CgScal* sc, double rn2, int mode) {
+  const double b = mode == FIN_START ? rn2 : sc->bnorm2;
+  return b > 0.0 ? sqrt(rn2 / b) : 0.0;
 }
 __device__ __forceinline__ double fin_new_beta(const CgScal* sc, double rz, double qz, int flexible) {
   return flexible ? -qz / sc->qp : rz / sc->rz;
@@ -33,6 +35,7 @@ __device__ __forceinline__ void fin_scalars(CgScal* sc, double rn2, double rz, d
     sc->bnorm2 = rn2;
     return;
   }
+  if (mode == FIN_START) sc->bnorm2 = rn2;
   sc->rnorm2 = rn2;
   sc->relres = rel;
   if (mode == FIN_NORM) return;
@@ -47,7 +50,7 @@ __device__ __forceinline__ void fin_scalars(CgScal* sc, double rn2, double rz, d
     }
     return;
   }
-  if (mode == FIN_INIT_R) {
+  if (mode == FIN_INIT_R || mode == FIN_START) {
     sc->rz = rz;
     sc->best = rel;
     sc->stall = 0;

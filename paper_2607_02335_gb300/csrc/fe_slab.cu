@@ -256,7 +256,7 @@ __global__ void k_fin(const double* __restrict__ red_all, int size, int nslots, 
   const int k = sc->iter;
   const double alpha_used = sc->alpha;
   // FIN_ITER: beta = gamma / gamma_old
-  fin_scalars(sc, rho, gamma, fin_rel(sc, rho),
+  fin_scalars(sc, rho, gamma, fin_rel(sc, rho, mode),
               mode == FIN_ITER ? fin_new_beta(sc, gamma, 0.0, 0) : 0.0, rtol, mode);
   if (mode == FIN_ITER && hist) {
     hist[3 * k + 0] = alpha_used;
