@@ -200,8 +200,34 @@ static fe_status launch_one(const ApplyArgs<N, V>& a, cudaStream_t st) {
   return launch_shape<N, V, OP, GEOM, MODE, Shape<N, V>>(a, st);
 }
 
-// Recompute mode: per chunk of cells, the metric into the L2-sized scratch, then the stored-metric
-// apply on the chunk.
+// the metric of cells [cell0, cell_end) on the fly
+template <int N, class V>
+static RecomputeArgs<N, V> recompute_args(const HostTab& tab, const typename RV<V>::GV* xyz,
+                                          typename NT<V>::GV* geo, const int* skip) {
+  RecomputeArgs<N, V> r;
+  std::memset(&r, 0, sizeof(r));
+  r.xyz = xyz;
+  r.geo = geo;
+  r.skip = skip;
+  for (int q = 0; q < N; ++q) r.tab.W_[q] = fe_cast<V>(tab.w[q]);
+  fill_eo<N, V>(r.tab.eV, tab.V, false);
+  fill_eo<N, V>(r.tab.eD, tab.D, false);
+  fill_full<RecomputeTab<N, V>, typename NT<V>::CV, N>(r.tab, tab);
+  return r;
+}
+template <int N, class V, int OP>
+static fe_status launch_metric(const RecomputeArgs<N, V>& r, cudaStream_t st) {
+  using G = RecCfg<N, V>;
+  auto kern = k_recompute<N, V, OP>;
+  FE_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM),
+          "recompute smem attribute");
+  const long long blocks = (r.cell_end - r.cell0 + G::CELLS - 1) / G::CELLS;
+  kern<<<(unsigned)blocks, G::THREADS, G::SMEM, st>>>(r);
+  return fe_cuda_check(cudaGetLastError(), "recompute kernel launch");
+}
+
+// Recompute mode: per chunk of cells, the metric into the scratch, then the stored-metric apply on the
+// chunk.
 template <int N, class V, int OP>
 static fe_status launch_recompute(ApplyArgs<N, V> a, const ApplyLaunch& L,
                                   const typename RV<V>::GV* xyz, typename NT<V>::GV* scratch) {
@@ -210,25 +236,14 @@ static fe_status launch_recompute(ApplyArgs<N, V> a, const ApplyLaunch& L,
     fe_set_error("apply: recompute-mode buffers missing for this arithmetic");
     return FE_ERR_INVALID;
   }
-  using G = GeoCfg<N>;
-  using W = typename RV<V>::T;
-  const long long chunk = fe_rc_chunk_cells(N, m->ncells, sizeof(typename NT<W>::GV));
-  RecomputeArgs<N, W> r;
-  std::memset(&r, 0, sizeof(r));
-  r.xyz = xyz;
-  r.geo = reinterpret_cast<typename NT<W>::GV*>(scratch);
-  r.skip = L.skip;
-  for (int q = 0; q < N; ++q) r.tab.W_[q] = fe_cast<W>(m->tab.w[q]);
-  fill_full<RecomputeTab<N, W>, W, N>(r.tab, m->tab);
+  const long long chunk = fe_rc_chunk_cells(N, m->ncells, RecCfg<N, V>::POINT_BYTES);
+  RecomputeArgs<N, V> r = recompute_args<N, V>(m->tab, xyz, scratch, L.skip);
   a.c.geo = scratch;
   for (long long c0 = 0; c0 < m->ncells; c0 += chunk) {
     const long long c1 = c0 + chunk < m->ncells ? c0 + chunk : m->ncells;
     r.cell0 = c0;
     r.cell_end = c1;
-    const long long gblocks = (c1 - c0 + G::CPB - 1) / G::CPB;
-    k_recompute<N, W, OP>
-        <<<(unsigned)gblocks, G::THREADS, recompute_smem_bytes<N, W>(), L.st>>>(r);
-    FE_CUDA(cudaGetLastError(), "recompute kernel launch");
+    FE_TRY((launch_metric<N, V, OP>(r, L.st)));
     a.c.cell_base = c0;
     a.c.geo_cell0 = c0;
     a.c.ncells = c1;
@@ -357,10 +372,17 @@ static fe_status launch_apply_n(const ApplyLaunch& L, const typename NT<V>::GV* 
   const bool fuse = L.assemble && N <= FE_FUSE_MAXN;
   // single cells where pairs would leave the SMs part-empty (the unfused layouts only)
   if constexpr (std::is_same<V, dw2>::value) {
-    if (!fuse && !m->packed && m->d.geom_mode != FE_GEOM_RECOMPUTE &&
+    const bool recompute = m->d.geom_mode == FE_GEOM_RECOMPUTE;
+    if ((!fuse || recompute) && !m->packed &&
         pair_shape<N>(m->ncells, fe_sm_count()) == TILE_SINGLE) {
       ApplyArgs<N, dw> one;
-      fill_args<N, dw>(one, L, geo);
+      fill_args<N, dw>(one, L, reinterpret_cast<const float2*>(geo));
+      if (recompute) {
+        float2* sc = reinterpret_cast<float2*>(scratch);
+        FE_TRY((L.op == FE_LAPLACE ? launch_recompute<N, dw, FE_LAPLACE>(one, L, xyz, sc)
+                                   : launch_recompute<N, dw, FE_MASS>(one, L, xyz, sc)));
+        return finish_unfused(L, FE_F64);
+      }
       FE_TRY((launch_geom<N, dw, MODE_CELLS>(one, L.op, affine, L.st)));
       return finish_unfused(L, FE_F64);
     }

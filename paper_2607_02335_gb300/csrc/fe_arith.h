@@ -442,7 +442,7 @@ struct NT<dw> {
   __device__ static __forceinline__ dw keep(dw a) { return a; }
   __device__ static __forceinline__ dw mul(dw a, dw b) { return dw_mul(a, b); }
   __device__ static __forceinline__ dw add(dw a, dw b) { return dw_add(a, b); }
-  __device__ static __forceinline__ dw sub(dw a, dw b) { return dw_add(a, {-b.h, -b.l}); }
+  __device__ static __forceinline__ dw neg(dw a) { return {-a.h, -a.l}; }
   // one Newton step from the float reciprocal: r = r0 + r0 (1 - a r0)
   __device__ static __forceinline__ dw recip(dw a) {
     const float r0 = __frcp_rn(a.h);
@@ -471,8 +471,17 @@ struct NT<dw2> {
   __device__ static __forceinline__ dw2 addk(dw2n a, dw2n b) { return dw2_addk(a, b); }
   __device__ static __forceinline__ dw2 subk(dw2n a, dw2n b) { return dw2_subk(a, b); }
   __device__ static __forceinline__ dw2 keep(dw2n a) { return {a.h, f2_neg(a.nl)}; }
+  __device__ static __forceinline__ dw2 fin(dw2 a) { return dw2_fast_two_sum(a.h, a.l); }
+  __device__ static __forceinline__ dw2 neg(dw2 a) { return {f2_neg(a.h), f2_neg(a.l)}; }
   __device__ static __forceinline__ dw2 mul(dw2 a, dw2 b) { return dw2_mul(a, b); }
   __device__ static __forceinline__ dw2 add(dw2 a, dw2 b) { return dw2_add(a, b); }
+  // one Newton step from the float reciprocal: r = r0 + r0 (1 - a r0)
+  __device__ static __forceinline__ dw2 recip(dw2 a) {
+    const float2 h = f2_unpack(a.h);
+    const dw2 r0 = {f2_pack(__frcp_rn(h.x), __frcp_rn(h.y)), 0ull};
+    const dw2 e = dw2_add({f2_pack(1.0f, 1.0f), 0ull}, neg(dw2_mul(a, r0)));
+    return dw2_add(r0, dw2_mul(r0, e));
+  }
 };
 template <>
 struct NT<bfv> : NT16<bfv> {};

@@ -32,9 +32,12 @@ Tab1D<N, V> make_tab(const HostTab& h);
 #define FE_GEO_COMPS 7  // xx, yy, zz, xy, xz, yz of w detJ J^{-1}J^{-T}, then w detJ
 
 // Recompute mode: cells per chunk of the metric scratch (about FE_RC_CHUNK_BYTES, a multiple of the
-// apply's cells per CTA), for a metric value of gv_bytes bytes.
+// apply's cells per CTA), for a metric value of gv_bytes bytes.  A chunk is two launches whose first and
+// last CTAs leave the SMs part-empty, which costs more than the scratch's trips to HBM: Laplace Q3 48^3
+// (396 MB of metric) 0.62 ms in chunks of 24 MB, 0.50 of 48 MB and 0.44 of 96 MB, which L2 would hold, 0.41
+// of 256 MB, 0.39 in one; Q6 28^3 1.08, 0.88, 0.81, 0.73 and 0.70 ms.
 #ifndef FE_RC_CHUNK_BYTES
-#define FE_RC_CHUNK_BYTES (48LL << 20)
+#define FE_RC_CHUNK_BYTES (256LL << 20)
 #endif
 inline long long fe_rc_chunk_cells(int n, long long ncells, size_t gv_bytes) {
   const long long per_cell = (long long)FE_GEO_COMPS * n * n * n * (long long)gv_bytes;
@@ -68,7 +71,7 @@ struct fe_mesh {
   // side; otherwise the cells with sn = n) -- what the DSS passes walk
   bool packed = false;
   int sgx = 0, sgy = 0, sgz = 0, sn = 0;
-  // recompute mode: nodal coordinates [cell][3][n3], and an L2-sized scratch for the metric of one
+  // recompute mode: nodal coordinates [cell][3][n3], and a scratch for the metric of one
   // chunk of cells (per arithmetic: 0 double-word, 1 FP64, 2 FP32)
   double* xyz64 = nullptr;
   float2* xyzdw = nullptr;

@@ -1,7 +1,7 @@
 // fe_vec.cu -- structured DSS, Jacobi diagonal, duality pairings and cell-wise vector kernels.
 #include <cstring>
 
-#include "fe_recompute.cuh"
+#include "fe_apply_launch.cuh"
 #include "fe_vec.cuh"
 
 // ---------------------------------------------------------------------------------------------
@@ -382,37 +382,21 @@ static fe_status launch_diag_chunk(const DiagArgs& a, cudaStream_t st) {
 template <int N>
 static fe_status launch_diag_n(const fe_mesh* m, DiagArgs a, cudaStream_t st) {
   if (m->d.geom_mode != FE_GEOM_RECOMPUTE) return launch_diag_chunk<N>(a, st);
-  using G = GeoCfg<N>;
   double* scratch = static_cast<double*>(m->rc_scratch[1]);
   if (!scratch || !m->xyz64) {
     fe_set_error("diag: recompute-mode buffers missing");
     return FE_ERR_INVALID;
   }
   const long long chunk = fe_rc_chunk_cells(N, m->ncells, sizeof(double));
-  RecomputeArgs<N, double> r;
-  std::memset(&r, 0, sizeof(r));
-  r.xyz = m->xyz64;
-  r.geo = scratch;
-  for (int q = 0; q < N; ++q) {
-    r.tab.W_[q] = m->tab.w[q];
-    for (int i = 0; i < N; ++i) {
-      r.tab.V_[q][i] = m->tab.V[q][i];
-      r.tab.D_[q][i] = m->tab.D[q][i];
-    }
-  }
+  RecomputeArgs<N, double> r = recompute_args<N, double>(m->tab, m->xyz64, scratch, nullptr);
   a.geo = scratch;
   const long long total = m->ncells;
   for (long long c0 = 0; c0 < total; c0 += chunk) {
     const long long c1 = c0 + chunk < total ? c0 + chunk : total;
     r.cell0 = c0;
     r.cell_end = c1;
-    const unsigned gb = (unsigned)((c1 - c0 + G::CPB - 1) / G::CPB);
-    const size_t gs = recompute_smem_bytes<N, double>();
-    if (a.op == FE_LAPLACE)
-      k_recompute<N, double, FE_LAPLACE><<<gb, G::THREADS, gs, st>>>(r);
-    else
-      k_recompute<N, double, FE_MASS><<<gb, G::THREADS, gs, st>>>(r);
-    FE_CUDA(cudaGetLastError(), "recompute kernel launch");
+    FE_TRY((a.op == FE_LAPLACE ? launch_metric<N, double, FE_LAPLACE>(r, st)
+                               : launch_metric<N, double, FE_MASS>(r, st)));
     a.cell_base = c0;
     a.geo_cell0 = c0;
     a.ncells = c1;

@@ -93,6 +93,25 @@ def test_recompute_several_chunks(fe, p, m):
         assert np.abs(got - ref).max() <= TOL64 * scale, op
 
 
+@pytest.mark.parametrize("p,m", [(1, (65, 63, 67)), (2, (35, 35, 37)), (3, (25, 25, 27)),
+                                 (4, (19, 19, 21)), (5, (15, 17, 17)), (6, (13, 13, 15)),
+                                 (7, (13, 13, 15)), (3, (44, 45, 47))])
+def test_recompute_pairs_and_ragged_chunks(fe, p, m):
+    """Meshes large enough for the kernels on pairs of cells, with an odd number of cells (the last
+    pair has one cell), and one whose metric spans two scratch chunks: recompute equals stored.  The
+    bounds are those of the oracle comparisons above, which both sides meet."""
+    gr = fe.Mesh(m, p, deform_amp=0.1, geom_mode=fe.FE_GEOM_RECOMPUTE)
+    gs = fe.Mesh(m, p, deform_amp=0.1)
+    x = torch.from_numpy(S.dual_cellwise(m, p, seed=4)).cuda()
+    for op in (fe.FE_LAPLACE, fe.FE_MASS):
+        for kw, v, tol in (({}, x, TOL64), ({"prec": fe.FE_F32}, x.float(), TOL32)):
+            ys = gs.apply(v, op=op, **kw)
+            err = (gr.apply(v, op=op, **kw) - ys).abs().max().item()
+            assert err <= tol * ys.abs().max().item(), (op, kw)
+    gr.close()
+    gs.close()
+
+
 def test_recompute_cg_matches_stored(fe):
     """Jacobi-PCG on a recompute mesh takes the same path as on the stored mesh."""
     m, p = (5, 4, 3), 3
