@@ -254,7 +254,7 @@ def run_reference(args, rank):
 # ---------------------------------------------------------------- our arm
 def kernel_source_sha():
     h = hashlib.sha256()
-    for f in ("fe_apply_kernel.cuh", "fe_arith.h", "fe_apply_launch.cuh"):
+    for f in ("fe_apply_kernel.cuh", "fe_apply_pair.cuh", "fe_arith.h", "fe_apply_launch.cuh"):
         with open(os.path.join(ROOT, "paper_2607_02335_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -427,7 +427,7 @@ def run_ours(args, rank, world):
     achieved = dom["volumetric_gbs"]
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                 "frac": round(achieved / peak, 4), "traffic": committed_traffic(),
-                "kernel": f"k_apply<{dom['degree'] + 1},dw,{dom['op']},stored>",
+                "kernel": f"k_apply_pair<{dom['degree'] + 1},{dom['op']},stored>",
                 "peak_source": f"{peak_kind} hbm_gbs (burst copy)",
                 "alg_bytes_per_launch": dom["volumetric_alg_bytes"],
                 "issue": issue_roofline(dom["volumetric_ms"], dom["cellwise_dofs"])}

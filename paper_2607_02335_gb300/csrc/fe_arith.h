@@ -37,20 +37,10 @@ __device__ __forceinline__ dw dw_fast_two_sum(float a, float b) {  // requires |
   float e = __fsub_rn(b, __fsub_rn(s, a));
   return {s, e};
 }
-// unnormalised accumulator acc + c*v: exact product error and a full TwoSum, low parts summed in
-// float (12 operations)
-__device__ __forceinline__ dw dw_mac12(dw acc, dw c, dw v) {
-  float p = __fmul_rn(c.h, v.h);
-  float e = __fmaf_rn(c.h, v.h, -p);
-  e = __fmaf_rn(c.h, v.l, e);
-  e = __fmaf_rn(c.l, v.h, e);
-  dw s = dw_two_sum(acc.h, p);
-  return {s.h, __fadd_rn(acc.l, __fadd_rn(s.l, e))};
-}
-// The same in 10 operations.  s = acc.h + p with p = fl(c.h v.h); of the TwoSum error, acc.h's share
-// t1 = acc.h - (s - bb) is exact (bb = s - acc.h), and p's share p - bb plus the product error c.h v.h
-// - p is c.h v.h - bb, one fma (a small value rounded once, an error of order 2^-24 ulp(s)).  The low
-// parts and cross products go in float.
+// unnormalised accumulator acc + c*v (10 operations).  s = acc.h + p with p = fl(c.h v.h); of the TwoSum
+// error, acc.h's share t1 = acc.h - (s - bb) is exact (bb = s - acc.h), and p's share p - bb plus the
+// product error c.h v.h - p is c.h v.h - bb, one fma (a small value rounded once, an error of order
+// 2^-24 ulp(s)).  The low parts and cross products go in float.
 __device__ __forceinline__ dw dw_mac(dw acc, dw c, dw v) {
   const float p = __fmul_rn(c.h, v.h);
   const float s = __fadd_rn(acc.h, p);
@@ -325,7 +315,6 @@ struct NT<double> {
   static constexpr bool LOWP = false;
   __device__ static __forceinline__ double zero() { return 0.0; }
   __device__ static __forceinline__ double mac(double a, double c, double v) { return fma(c, v, a); }
-  __device__ static __forceinline__ double mac12(double a, double c, double v) { return fma(c, v, a); }
   __device__ static __forceinline__ double prod(double c, double v) { return c * v; }
   __device__ static __forceinline__ double addk(double a, double b) { return a + b; }
   __device__ static __forceinline__ double subk(double a, double b) { return a - b; }
@@ -333,7 +322,6 @@ struct NT<double> {
   __device__ static __forceinline__ double keep(double a) { return a; }
   __device__ static __forceinline__ double mul(double a, double b) { return a * b; }
   __device__ static __forceinline__ double add(double a, double b) { return a + b; }
-  __device__ static __forceinline__ double sub(double a, double b) { return a - b; }
   __device__ static __forceinline__ double recip(double a) { return 1.0 / a; }
   __device__ static __forceinline__ double neg(double a) { return -a; }
   __device__ static __forceinline__ double load(const double* p) { return __ldg(p); }
@@ -352,7 +340,6 @@ struct NT<float> {
   static constexpr bool LOWP = false;
   __device__ static __forceinline__ float zero() { return 0.0f; }
   __device__ static __forceinline__ float mac(float a, float c, float v) { return fmaf(c, v, a); }
-  __device__ static __forceinline__ float mac12(float a, float c, float v) { return fmaf(c, v, a); }
   __device__ static __forceinline__ float prod(float c, float v) { return c * v; }
   __device__ static __forceinline__ float addk(float a, float b) { return a + b; }
   __device__ static __forceinline__ float subk(float a, float b) { return a - b; }
@@ -360,7 +347,6 @@ struct NT<float> {
   __device__ static __forceinline__ float keep(float a) { return a; }
   __device__ static __forceinline__ float mul(float a, float b) { return a * b; }
   __device__ static __forceinline__ float add(float a, float b) { return a + b; }
-  __device__ static __forceinline__ float sub(float a, float b) { return a - b; }
   __device__ static __forceinline__ float recip(float a) { return 1.0f / a; }
   __device__ static __forceinline__ float neg(float a) { return -a; }
   __device__ static __forceinline__ float load(const float* p) { return __ldg(p); }
@@ -397,7 +383,6 @@ struct NT16 {
   }
   __device__ static __forceinline__ W zero() { return {0.0f}; }
   __device__ static __forceinline__ W mac(W a, W c, W x) { return {fmaf(c.v, x.v, a.v)}; }
-  __device__ static __forceinline__ W mac12(W a, W c, W x) { return {fmaf(c.v, x.v, a.v)}; }
   __device__ static __forceinline__ W prod(W c, W x) { return {c.v * x.v}; }
   __device__ static __forceinline__ W addk(W a, W b) { return {rnd(a.v + b.v)}; }
   __device__ static __forceinline__ W subk(W a, W b) { return {rnd(a.v - b.v)}; }
@@ -405,7 +390,6 @@ struct NT16 {
   __device__ static __forceinline__ W keep(W a) { return {rnd(a.v)}; }
   __device__ static __forceinline__ W mul(W a, W b) { return {a.v * b.v}; }
   __device__ static __forceinline__ W add(W a, W b) { return {a.v + b.v}; }
-  __device__ static __forceinline__ W sub(W a, W b) { return {a.v - b.v}; }
   __device__ static __forceinline__ W recip(W a) { return {1.0f / a.v}; }
   __device__ static __forceinline__ W neg(W a) { return {-a.v}; }
   __device__ static __forceinline__ W load(const float* p) { return {rnd(__ldg(p))}; }
@@ -434,8 +418,6 @@ struct NT<dw> {
   // the double-word level of the operands, which is all the following products need
   __device__ static __forceinline__ dw addk(dw a, dw b) { return dw_add_keep(a, b); }
   __device__ static __forceinline__ dw subk(dw a, dw b) { return dw_add_keep(a, {-b.h, -b.l}); }
-  // the 12-operation form, for the geometry terms (their error reaches every output)
-  __device__ static __forceinline__ dw mac12(dw a, dw c, dw v) { return dw_mac12(a, c, v); }
   __device__ static __forceinline__ dw fin(dw a) { return dw_norm(a); }
   // intermediate results of the sweeps stay unnormalised: |lo| stays below a few ulp(hi), and the
   // next products use lo only in FP32 cross terms (relative effect ~2^-45)
