@@ -299,8 +299,8 @@ def issue_roofline(kernel_ms, cellwise_dofs):
     peak = 152 * 4 * mhz * 1e6 / 1e12
     return {"unit": "T warp-instructions/s", "achieved": round(achieved, 4), "peak": round(peak, 4),
             "frac": round(achieved / peak, 4), "warp_instructions_per_cellwise_dof": per_dof,
-            "note": "the kernel is bound by instruction issue (double-word FP64 arithmetic on the "
-                    "FP32 pipe); frac is its share of the issue peak"}
+            "note": "FP64-accurate double-word arithmetic in packed FP32 instructions, each of which "
+                    "holds the FP32 pipe for two issue slots; frac is the share of the issue peak"}
 
 
 def max_over_ranks(x, world, device):
