@@ -496,7 +496,9 @@ template <class S>
 __global__ void __launch_bounds__(BT)
     kb_precond(const BProb* __restrict__ probs, const Chunk* __restrict__ chunks, int nchunks,
                int slot, int pmode, int mode, double* partials, unsigned* arrive) {
-  using V = Vec<S, 2>;
+  // one 16-byte group per vector in flight: two need 80 registers, and a third of the warps goes (64
+  // problems of 4^3 to 32^3: 3.62 s against 3.47; 32 of up to 20^3, FP64: 0.670 against 0.653)
+  using V = Vec<S, 1>;
   __shared__ double sh[SUM_MAX * SUM_THREADS];
   for (int c = blockIdx.x; c < nchunks; c += gridDim.x) {
     const Chunk C = chunks[c];
