@@ -264,19 +264,27 @@ __device__ __forceinline__ dw dw_from_doubles(double a, const ExpShift& s) {
   return {v.hi[0], __fmul_rn(lo, v.sc[0])};
 }
 
-// (h + l) 2^sh as binary64 (`plain`): both parts widened on the integer pipe, one FP64 addition
+// (h + l) 2^sh as binary64, rounded once.  Where the CTA's inputs are `plain` and the parts finite (in_range)
+// both are widened on the integer pipe, subnormal floats to zero, and one FP64 addition rounds; the rest goes
+// out of line and gets the same bits wherever both are right, so that a cell's values do not depend on what
+// else its tile holds.  Finite inputs can still overflow float on the way, in a metric beyond its range or
+// in the sweeps, and an infinity or NaN then has to arrive as one.
+__device__ __forceinline__ bool in_range(dw v) {
+  const float inf = __uint_as_float(0x7F800000u);
+  return fabsf(v.h) < inf && fabsf(v.l) < inf;
+}
 __device__ __forceinline__ double dw_to_double_plain(dw v, int sh) {
   const unsigned k = (unsigned)(896 + sh) << 20;
   auto wide = [&](float f) {
     const unsigned u = __float_as_uint(f);
-    const unsigned h = (u & 0x7F800000u) == 0u ? 0u : ((unsigned)((int)u >> 3) & 0x8FFFFFFFu) + k;
-    return __hiloint2double((int)h, (int)(u << 29));
+    const bool zero = (u & 0x7F800000u) == 0u;
+    const unsigned h = ((unsigned)((int)u >> 3) & 0x8FFFFFFFu) + k;
+    return __hiloint2double(zero ? 0 : (int)h, zero ? 0 : (int)(u << 29));
   };
   return wide(v.h) + wide(v.l);
 }
-
 static __device__ __noinline__ double dw_to_double_general(dw v, int sh) {
-  return dw_to_double_sh(v, sh);
+  return scalbn(f2d_bits(v.h) + f2d_bits(v.l), sh);
 }
 
 // the two cells of pair slot pl of the tile at cell0 (cell_pos's tile modes)
@@ -659,16 +667,24 @@ __device__ __forceinline__ void apply_pairs(const CellArgs<N, typename PairCfg<N
   tile_sync<N>();
 
   // ---- outputs, binary64
-  auto out = [&](V v, int c, int k) -> double {
-    dw x;
+  auto out = [&](V v, int k, double (&q)[W]) {
+    dw x[W];
     if constexpr (W == 2) {
       const float2 h = f2_unpack(v.h), l = f2_unpack(v.l);
-      x = c == 0 ? dw{h.x, l.x} : dw{h.y, l.y};
+      x[0] = {h.x, l.x};
+      x[1] = {h.y, l.y};
     } else {
-      x = v;
+      x[0] = v;
     }
-    const dw m = masked(c, k) ? dw{0.0f, 0.0f} : x;
-    return es.plain ? dw_to_double_plain(m, es.sh) : dw_to_double_general(m, es.sh);
+    bool plain = es.plain;
+#pragma unroll
+    for (int c = 0; c < W; ++c) {
+      if (masked(c, k)) x[c] = {0.0f, 0.0f};
+      plain = plain && in_range(x[c]);
+    }
+#pragma unroll
+    for (int c = 0; c < W; ++c)
+      q[c] = plain ? dw_to_double_plain(x[c], es.sh) : dw_to_double_general(x[c], es.sh);
   };
   if constexpr (MODE != MODE_CELLS && warp_tile<N>()) __syncthreads();
   if constexpr (MODE == MODE_BRICK || MODE == MODE_BRICKZ) pair_brick_sums<N>(s0, a, cell0);
@@ -676,29 +692,31 @@ __device__ __forceinline__ void apply_pairs(const CellArgs<N, typename PairCfg<N
     // The z-interface with the previous layer of the chunk: the structured DSS's z-pass pair sum
     // (lower + upper copy), formed on the stored values, so the result is that of the pass.
     // The x/y sums inside the brick came first, as they do before the pass.
-    const dw2 vb = s0.get(bz), vt = s0.get(bz + (N - 1) * PS);
+    double qb[W], qt[W];
+    out(s0.get(bz), 0, qb);
+    out(s0.get(bz + (N - 1) * PS), N - 1, qt);
 #pragma unroll
     for (int c = 0; c < W; ++c) {
       if (!act[c]) continue;
       double* y = a.y + cell[c] * N3 + lt;
-      double bottom = out(vb, c, 0);
+      double bottom = qb[c];
       if (zc->pending) {
         bottom = zc->top[c] + bottom;
         __stcs(y - (long long)a.mx * a.my * N3 + (N - 1) * N2, bottom);
       }
       __stcs(y, bottom);
-      const double top = out(vt, c, N - 1);
       if (zc->last)
-        __stcs(y + (N - 1) * N2, top);
+        __stcs(y + (N - 1) * N2, qt[c]);
       else
-        zc->top[c] = top;
+        zc->top[c] = qt[c];
     }
 #pragma unroll
     for (int k = 1; k < N - 1; ++k) {
-      const dw2 v = s0.get(bz + k * PS);
+      double q[W];
+      out(s0.get(bz + k * PS), k, q);
 #pragma unroll
       for (int c = 0; c < W; ++c)
-        if (act[c]) __stcs(a.y + cell[c] * N3 + lt + k * N2, out(v, c, k));
+        if (act[c]) __stcs(a.y + cell[c] * N3 + lt + k * N2, q[c]);
     }
     zc->pending = !zc->last;
     return;
@@ -729,15 +747,15 @@ __device__ __forceinline__ void apply_pairs(const CellArgs<N, typename PairCfg<N
     }
     __syncthreads();
     if (act[0] && (sy == 0 || lb > 0)) {
+      double* yu = a.y + (cell0 + pl / 4) * Packed<N>::NU3 + (long long)(sy * P + lb) * NU + la;
 #pragma unroll
-      for (int c = 0; c < W; ++c) {
-        if (c == 1 && la == 0) continue;
-        double* yu = a.y + (cell0 + pl / 4) * Packed<N>::NU3 + (long long)(sy * P + lb) * NU + c * P + la;
+      for (int k = 0; k < N; ++k) {
+        if (sz == 1 && k == 0) continue;
+        double q[W];
+        out(s0.get(bz + k * PS), k, q);
 #pragma unroll
-        for (int k = 0; k < N; ++k) {
-          if (sz == 1 && k == 0) continue;
-          __stcs(yu + (long long)(sz * P + k) * NU * NU, out(s0.get(bz + k * PS), c, k));
-        }
+        for (int c = 0; c < W; ++c)
+          if (c == 0 || la > 0) __stcs(yu + (long long)(sz * P + k) * NU * NU + c * P, q[c]);
       }
     }
     return;
@@ -745,14 +763,14 @@ __device__ __forceinline__ void apply_pairs(const CellArgs<N, typename PairCfg<N
   Acc<double> qp;
 #pragma unroll 1
   for (int k = 0; k < N; ++k) {
-    const V v = s0.get(bz + k * PS);
+    double q[W];
+    out(s0.get(bz + k * PS), k, q);
 #pragma unroll
     for (int c = 0; c < W; ++c) {
       if (!act[c]) continue;
       const long long e = cell[c] * N3 + lt + k * N2;
-      const double q = out(v, c, k);
-      __stcs(a.y + e, q);
-      if constexpr (CG) qp.add_prod(q, *(volatile const double*)(a.x + e));
+      __stcs(a.y + e, q[c]);
+      if constexpr (CG) qp.add_prod(q[c], *(volatile const double*)(a.x + e));
     }
   }
   if constexpr (CG) cg_finish_apply(*cg, qp);

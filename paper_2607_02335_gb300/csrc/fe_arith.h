@@ -137,48 +137,6 @@ __device__ __forceinline__ double f2d_bits(float f) {
   return (double)f;  // inf / nan
 }
 __device__ __forceinline__ double dw_to_double(dw a) { return f2d_bits(a.h) + f2d_bits(a.l); }
-static __device__ __noinline__ double dw_to_double_slow(dw a) { return f2d_bits(a.h) + f2d_bits(a.l); }
-
-// binary64 of h + l on the integer and FP32 pipes (no FP64 add): after a TwoSum |l| <= ulp(h)/2,
-// so l is at most 2^28 units of 2^(e-52), e the exponent of h; those units, truncated to an
-// integer, are added to (or, for opposite signs, subtracted from) the bit pattern of h, whose
-// low 29 mantissa bits are zero.  Subtracting from a power of two crosses into the binade below,
-// where the unit is half as large.  Result within 2^(e-52) of h + l (about one double ulp).
-// Zero and the exponent range outside 2^-75 .. 2^127 take the FP64 path.
-__device__ __forceinline__ double dw_to_double_int(dw a) {
-  const dw s = dw_two_sum(a.h, a.l);
-  const unsigned hb = __float_as_uint(s.h);
-  const unsigned e8 = (hb >> 23) & 0xFFu;
-  if (s.h == 0.0f) return 0.0;
-  if (e8 - 52u > 202u) return dw_to_double_slow(s);
-  const unsigned long long dh = ((unsigned long long)(hb & 0x80000000u) << 32) |
-                                ((unsigned long long)(e8 + 896u) << 52) |
-                                ((unsigned long long)(hb & 0x7FFFFFu) << 29);
-  const float v = __fmul_rn(fabsf(s.l), __uint_as_float((306u - e8) << 23));
-  const unsigned vb = __float_as_uint(v);
-  const int ev = (int)(vb >> 23) - 127;
-  const unsigned mv = (vb & 0x7FFFFFu) | 0x800000u;
-  const unsigned li = ev >= 23 ? (mv << (ev - 23)) : (ev >= 0 ? (mv >> (23 - ev)) : 0u);
-  unsigned long long out;
-  if (((hb ^ __float_as_uint(s.l)) & 0x80000000u) == 0u)
-    out = dh + li;
-  else
-    out = dh - ((hb & 0x7FFFFFu) == 0u ? 2ull * li : (unsigned long long)li);
-  return __longlong_as_double((long long)out);
-}
-
-// (h + l) * 2^sh as binary64: dw_to_double_int, then sh added to the exponent field; results
-// that leave the normal binary64 range take the FP64 path (out of line).
-static __device__ __noinline__ double dw_to_double_sh_slow(double v, int sh) { return scalbn(v, sh); }
-__device__ __forceinline__ double dw_to_double_sh(dw a, int sh) {
-  const double v = dw_to_double_int(a);
-  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-  const unsigned e = (unsigned)(b >> 52) & 0x7FFu;
-  if (e == 0u || sh == 0) return v;
-  if (e != 0x7FFu && (e + (unsigned)sh) - 1u < 2046u)
-    return __longlong_as_double((long long)(b + ((unsigned long long)(long long)sh << 52)));
-  return dw_to_double_sh_slow(v, sh);
-}
 
 // ---------------------------------------------------------------------------------------------
 // packed double-word arithmetic: two values per operand (the two cells of a pair)
