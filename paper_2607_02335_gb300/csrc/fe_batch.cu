@@ -511,7 +511,7 @@ __global__ void __launch_bounds__(BT)
     const S* idg = (sizeof(S) == 8) ? (const S*)P.invdiag64 : (const S*)P.invdiag32;
     const float* im = P.invmult;
     const bool dir = pmode & 1, redist = pmode & 2, flex = pmode & 4;
-    Sum2 a0, a1, a2;
+    DwSum a0, a1, a2;
     auto body = [&](S we, float ime, S dg, S& re, S qe) -> S {  // returns z, updates r
       const dw w2 = prod_dw(we, we);
       a0.add({w2.h * ime, w2.l * ime});
@@ -645,7 +645,7 @@ __global__ void __launch_bounds__(BT)
     const BProb& P = probs[C.prob];
     if (*(volatile const int*)&P.sc[0].done) continue;
     const double s = by_one_thread(&scale, [&] { return 1.0 / sqrt(P.sc[0].rnorm2); });
-    Sum2 a0;
+    DwSum a0;
     Acc<float> a1;
     for (long long e = C.lo + threadIdx.x; e < C.hi; e += RED_U * BT) {
       double wv[RED_U];

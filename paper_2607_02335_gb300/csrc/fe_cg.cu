@@ -188,7 +188,7 @@ __global__ void k_update_p(S* __restrict__ p, const S* __restrict__ z, const CgS
 // diag (measured: binary64 FMAs for <r,z> there made it slower, 165 -> 202 us at Q3 64^3)
 template <class S>
 struct AccDw {
-  Sum2 v;
+  DwSum v;
   __device__ __forceinline__ void add_prod(S a, S b) { v.add(prod_dw(a, b)); }
   __device__ __forceinline__ double value() const { return v.value(); }
 };
@@ -281,7 +281,7 @@ __global__ void __launch_bounds__(RED_THREADS)
       return w[f];
   };
   __shared__ double sh[SUM_MAX * SUM_THREADS];
-  Sum2 a0;
+  DwSum a0;
   AccDw<S> a1, a2;
   auto body = [&](long long e, S we, float im, S idg, S rv, S qv) {
     const dw w2 = prod_dw(we, we);
@@ -352,7 +352,7 @@ __global__ void __launch_bounds__(RED_THREADS)
                 float* __restrict__ z, float* __restrict__ d, float* __restrict__ p, double* partials,
                 unsigned* count, CgScal* sc, long long n, const FinBeta fin) {
   __shared__ double sh[SUM_MAX * SUM_THREADS];
-  Sum2 a0;
+  DwSum a0;
   Acc<float> a1;
   const long long STRIDE = (long long)gridDim.x * RED_THREADS;
   for (long long e = (long long)blockIdx.x * RED_THREADS + threadIdx.x; e < n; e += RED_U * STRIDE) {

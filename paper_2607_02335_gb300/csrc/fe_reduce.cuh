@@ -126,18 +126,14 @@ __device__ __forceinline__ void fin_alpha(const double* partials, int nparts, Cg
   }
 }
 
-// A thread's running sum of double-word terms, compensated (Dot2 of Ogita, Rump and Oishi, "Accurate sum
-// and dot product", SIAM J. Sci. Comput. 2005: the accuracy of a sum in twice the working precision):
-// the TwoSum error and the term's low part go to a second float.  8 operations a term where a
-// normalised double-word sum takes 20.
-struct Sum2 {
-  float h = 0.0f, l = 0.0f;
-  __device__ __forceinline__ void add(dw t) {
-    const dw s = dw_two_sum(h, t.h);
-    h = s.h;
-    l = __fadd_rn(l, __fadd_rn(s.l, t.l));
-  }
-  __device__ __forceinline__ double value() const { return dw_to_double({h, l}); }
+// A thread's running sum of double-word terms, normalised after every term: the low part then stays below
+// an ulp of the high part and its rounding errors near 2^-48 of the sum each, whatever the number of terms.
+// Left unnormalised (8 operations a term instead of 11) the low part grows with the sum of the errors it
+// holds: 1.7 times the error at 16 terms, 3 at 108, 6 at 640 (positive terms).
+struct DwSum {
+  dw v = {0.0f, 0.0f};
+  __device__ __forceinline__ void add(dw t) { v = dw_add(v, t); }
+  __device__ __forceinline__ double value() const { return dw_to_double(v); }
 };
 
 // A thread's running sum of products in a pairing: float vectors in double-word (exact products);
@@ -154,7 +150,7 @@ template <class S>
 struct Acc;
 template <>
 struct Acc<float> {
-  Sum2 v;
+  DwSum v;
   __device__ __forceinline__ void add_prod(float a, float b) { v.add(prod_dw(a, b)); }
   __device__ __forceinline__ double value() const { return v.value(); }
 };
