@@ -2,7 +2,7 @@
 #include "fe_apply_launch.cuh"
 
 fe_status fe_launch_apply_f64dw(const ApplyLaunch& L) {
-  return launch_apply_v<dw2>(L, L.m->geodw, L.m->xyzdw, static_cast<float*>(L.m->rc_scratch[0]));
+  return launch_apply_v<dw2>(L, L.m->geodw, L.m->xyzdw, static_cast<float*>(L.m->rc_scratch));
 }
 
 // The fused kernel saves the launches and passes of the p update and of <q,p>, and pays for them with a

@@ -2,5 +2,5 @@
 #include "fe_apply_launch.cuh"
 
 fe_status fe_launch_apply_f32(const ApplyLaunch& L) {
-  return launch_apply_v<float>(L, L.m->geo32, L.m->xyz32, static_cast<float*>(L.m->rc_scratch[2]));
+  return launch_apply_v<float>(L, L.m->geo32, L.m->xyz32, static_cast<float*>(L.m->rc_scratch));
 }

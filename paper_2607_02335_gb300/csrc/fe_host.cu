@@ -144,7 +144,8 @@ void make_view(const fe_mesh* m, int z0, int z1, fe_mesh* v) {
   v->xyz64 = nullptr;
   v->xyzdw = nullptr;
   v->xyz32 = nullptr;
-  for (void*& r : v->rc_scratch) r = nullptr;
+  v->rc_scratch = nullptr;
+  v->rc_diag = nullptr;
   for (int k = 0; k < 2; ++k) {
     v->diag64[k] = nullptr;
     v->invdiag32[k] = nullptr;

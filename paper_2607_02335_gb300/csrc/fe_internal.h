@@ -31,19 +31,25 @@ Tab1D<N, V> make_tab(const HostTab& h);
 // ---------------------------------------------------------------------------------------------
 #define FE_GEO_COMPS 7  // xx, yy, zz, xy, xz, yz of w detJ J^{-1}J^{-T}, then w detJ
 
-// Recompute mode: cells per chunk of the metric scratch (about FE_RC_CHUNK_BYTES, a multiple of the
-// apply's cells per CTA), for a metric value of gv_bytes bytes.  A chunk is two launches whose first and
-// last CTAs leave the SMs part-empty, which costs more than the scratch's trips to HBM: Laplace Q3 48^3
-// (396 MB of metric) 0.62 ms in chunks of 24 MB, 0.50 of 48 MB and 0.44 of 96 MB, which L2 would hold, 0.41
-// of 256 MB, 0.39 in one; Q6 28^3 1.08, 0.88, 0.81, 0.73 and 0.70 ms.
+// Recompute mode: cells per chunk of the metric scratch (about `limit` bytes, whole tiles of cells or pairs),
+// for a metric value of gv_bytes bytes.  A chunk is two launches whose first and last CTAs leave the SMs
+// part-empty, which costs more than the scratch's trips to HBM: Laplace Q3 48^3 (396 MB of metric) 0.62 ms
+// in chunks of 24 MB, 0.50 of 48 MB and 0.44 of 96 MB, which L2 would hold, 0.41 of 256 MB, 0.39 in one; Q6
+// 28^3 1.08, 0.88, 0.81, 0.73 and 0.70 ms.  All arithmetics of the apply share one scratch: applies on a
+// recompute mesh do not overlap.  The diagonal, formed once per mesh and operator in most programs, has a
+// small one of its own, so that it may run beside an apply.
 #ifndef FE_RC_CHUNK_BYTES
 #define FE_RC_CHUNK_BYTES (256LL << 20)
 #endif
-inline long long fe_rc_chunk_cells(int n, long long ncells, size_t gv_bytes) {
+#ifndef FE_RC_DIAG_BYTES
+#define FE_RC_DIAG_BYTES (48LL << 20)
+#endif
+inline long long fe_rc_chunk_cells(int n, long long ncells, size_t gv_bytes,
+                                   long long limit = FE_RC_CHUNK_BYTES) {
   const long long per_cell = (long long)FE_GEO_COMPS * n * n * n * (long long)gv_bytes;
-  const long long cpb = 256 / (n * n);
-  long long c = FE_RC_CHUNK_BYTES / per_cell;
-  c = c >= cpb ? c / cpb * cpb : (c > 0 ? c : 1);
+  const long long tile = 2 * (256 / (n * n));
+  long long c = limit / per_cell;
+  c = c >= tile ? c / tile * tile : (c > 0 ? c : 1);
   return c < ncells ? c : (ncells > 0 ? ncells : 1);
 }
 
@@ -71,12 +77,13 @@ struct fe_mesh {
   // side; otherwise the cells with sn = n) -- what the DSS passes walk
   bool packed = false;
   int sgx = 0, sgy = 0, sgz = 0, sn = 0;
-  // recompute mode: nodal coordinates [cell][3][n3], and a scratch for the metric of one
-  // chunk of cells (per arithmetic: 0 double-word, 1 FP64, 2 FP32)
+  // recompute mode: nodal coordinates [cell][3][n3], and scratches for the metric of one chunk of cells, the
+  // applies' and the diagonal's
   double* xyz64 = nullptr;
   float2* xyzdw = nullptr;
   float* xyz32 = nullptr;
-  void* rc_scratch[3] = {nullptr, nullptr, nullptr};
+  void* rc_scratch = nullptr;
+  double* rc_diag = nullptr;
   long long rc_cells = 0;  // cells per chunk
   // Jacobi diagonal caches (cell-wise, continuous), per operator
   double* diag64[2] = {nullptr, nullptr};
@@ -123,6 +130,7 @@ fe_status fe_cuda_check(cudaError_t e, const char* what);
 #define FE_CUDA(expr, what) FE_TRY(fe_cuda_check((expr), (what)))
 
 fe_status fe_ensure_geometry(const fe_mesh* m, int prec, bool native);  // fe_mesh.cu
+fe_status fe_ensure_diag_scratch(const fe_mesh* m);                     // recompute mode (fe_mesh.cu)
 // fe_mesh_create with an optional trilinear block map (8 corners, 24 doubles; null = unit cube)
 // z0 < z1: build only the slab of layers [z0, z1) of the mesh d describes (z1 = 0: all of it)
 fe_status fe_mesh_create_impl(const fe_mesh_desc* d, const double* corners, void* stream,

@@ -6,6 +6,7 @@
 // J_ab = d x_a / d xi_b (xi in [0,1]^3) by sum factorization, then stores
 // G = w_q detJ J^{-1} J^{-T} (6 symmetric entries) and w_q detJ, in FP64, laid out
 // [cell][component][q] so that the apply kernels read them with coalesced loads.
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -310,10 +311,9 @@ static unsigned grid_for(long long n, int threads) {
 fe_status fe_ensure_geometry(const fe_mesh* cm, int prec, bool native) {
   fe_mesh* m = const_cast<fe_mesh*>(cm);
   if (m->d.geom_mode == FE_GEOM_RECOMPUTE) {
-    // coordinate copy in the arithmetic of the call, and that arithmetic's metric scratch
+    // coordinate copy in the arithmetic of the call, and the metric scratch (never larger for the 4-byte values)
     const long long n = m->ncells * 3 * m->n3;
     const int idx = prec == FE_F32 ? 2 : (native ? 1 : 0);
-    const size_t gv = idx == 2 ? sizeof(float) : (idx == 1 ? sizeof(double) : sizeof(float2));
     if (idx == 0 && !m->xyzdw) {
       FE_TRY(fe_dalloc((void**)&m->xyzdw, n * sizeof(float2), m->st, "coordinates (double-word)"));
       k_split_dw<<<grid_for(n, 256), 256, 0, m->st>>>(m->xyz64, m->xyzdw, n);
@@ -323,10 +323,11 @@ fe_status fe_ensure_geometry(const fe_mesh* cm, int prec, bool native) {
       k_to_f32<<<grid_for(n, 256), 256, 0, m->st>>>(m->xyz64, m->xyz32, n);
       FE_CUDA(cudaStreamSynchronize(m->st), "coordinates fp32 copy");
     }
-    if (!m->rc_scratch[idx]) {
-      const long long cells = fe_rc_chunk_cells(m->n, m->ncells, gv);
-      FE_TRY(fe_dalloc(&m->rc_scratch[idx], (size_t)cells * FE_GEO_COMPS * m->n3 * gv, m->st,
-                       "recompute metric scratch"));
+    if (!m->rc_scratch) {
+      size_t bytes = 0;
+      for (const size_t gv : {sizeof(float), sizeof(double)})
+        bytes = std::max(bytes, (size_t)fe_rc_chunk_cells(m->n, m->ncells, gv) * FE_GEO_COMPS * m->n3 * gv);
+      FE_TRY(fe_dalloc(&m->rc_scratch, bytes, m->st, "recompute metric scratch"));
       FE_CUDA(cudaStreamSynchronize(m->st), "recompute metric scratch");
     }
     return FE_OK;
@@ -388,6 +389,15 @@ fe_status fe_ensure_geometry(const fe_mesh* cm, int prec, bool native) {
   return FE_OK;
 }
 
+fe_status fe_ensure_diag_scratch(const fe_mesh* cm) {
+  fe_mesh* m = const_cast<fe_mesh*>(cm);
+  if (m->rc_diag) return FE_OK;
+  const long long cells = fe_rc_chunk_cells(m->n, m->ncells, sizeof(double), FE_RC_DIAG_BYTES);
+  FE_TRY(fe_dalloc((void**)&m->rc_diag, (size_t)cells * FE_GEO_COMPS * m->n3 * sizeof(double), m->st,
+                   "recompute diagonal scratch"));
+  return fe_cuda_check(cudaStreamSynchronize(m->st), "recompute diagonal scratch");
+}
+
 // ---------------------------------------------------------------------------------------------
 // mesh object
 // ---------------------------------------------------------------------------------------------
@@ -395,8 +405,7 @@ static void free_mesh(fe_mesh* m, cudaStream_t st) {
   if (!m) return;
   if (m->cg_work && m->cg_free) m->cg_free(m->cg_work, st);
   void* bufs[] = {m->geo64, m->geodw, m->geo32, m->geo16[0], m->geo16[1], m->xyz64, m->xyzdw,
-                  m->xyz32, m->rc_scratch[0],
-                  m->rc_scratch[1], m->rc_scratch[2], m->diag64[0],
+                  m->xyz32, m->rc_scratch, m->rc_diag, m->diag64[0],
                   m->diag64[1], m->invdiag32[0], m->invdiag32[1], m->invdiag64[0],
                   m->invdiag64[1], m->invmult64, m->red, m->hs_xu, m->hs_xc, m->hs_yc,
                   m->hs_yu[0], m->hs_yu[1], m->kron_tab[0][0], m->kron_tab[0][1],

@@ -382,12 +382,12 @@ static fe_status launch_diag_chunk(const DiagArgs& a, cudaStream_t st) {
 template <int N>
 static fe_status launch_diag_n(const fe_mesh* m, DiagArgs a, cudaStream_t st) {
   if (m->d.geom_mode != FE_GEOM_RECOMPUTE) return launch_diag_chunk<N>(a, st);
-  double* scratch = static_cast<double*>(m->rc_scratch[1]);
+  double* scratch = m->rc_diag;
   if (!scratch || !m->xyz64) {
     fe_set_error("diag: recompute-mode buffers missing");
     return FE_ERR_INVALID;
   }
-  const long long chunk = fe_rc_chunk_cells(N, m->ncells, sizeof(double));
+  const long long chunk = fe_rc_chunk_cells(N, m->ncells, sizeof(double), FE_RC_DIAG_BYTES);
   RecomputeArgs<N, double> r = recompute_args<N, double>(m->tab, m->xyz64, scratch, nullptr);
   a.geo = scratch;
   const long long total = m->ncells;
@@ -447,7 +447,7 @@ fe_status fe_launch_diag(const fe_mesh* m, int op, double* d, cudaStream_t st) {
       a.tab.DV[q][i] = m->tab.Dh[q][i] * m->tab.V[q][i];
     }
   }
-  if (m->d.geom_mode == FE_GEOM_RECOMPUTE) FE_TRY(fe_ensure_geometry(m, FE_F64, true));
+  if (m->d.geom_mode == FE_GEOM_RECOMPUTE) FE_TRY(fe_ensure_diag_scratch(m));
   if (!a.affine && !a.geo && m->d.geom_mode != FE_GEOM_RECOMPUTE) {
     fe_set_error("diag: the stored metric has been released");
     return FE_ERR_INVALID;

@@ -141,3 +141,25 @@ def test_recompute_not_accepted_by_batched(fe):
     x = torch.zeros_like(b)
     with pytest.raises(fe.FeError):
         fe.fe_cg_solve_batched([gm.handle], [b], [x], fe.fe_cg_opts(1e-8, 10, 0, 0, 1e-2, None))
+
+
+def test_scratch_is_shared_between_arithmetics(fe):
+    """What a recompute mesh holds on the device after applies in every arithmetic and a diagonal: the
+    coordinate copies, one metric scratch of 256 MB (allocated with the mesh) and the diagonal's 48 MB."""
+    gm = fe.Mesh((54, 54, 53), 3, deform_amp=0.1, geom_mode=fe.FE_GEOM_RECOMPUTE)
+    n = gm.cellwise_len
+    assert 7 * 4 * n > 256 << 20  # the metric is beyond the scratch in FP32 too
+    x = torch.rand(n, dtype=torch.float64, device="cuda")
+    y, x32, y32 = torch.empty_like(x), x.float(), torch.empty(n, dtype=torch.float32, device="cuda")
+    gm.apply(x, y=y)
+    torch.cuda.synchronize()
+    free0 = torch.cuda.mem_get_info()[0]
+    gm.apply(x32, prec=fe.FE_F32, y=y32)
+    gm.apply(x, flags=fe.FE_NATIVE_F64, y=y)
+    fe.fe_diag(gm.handle, fe.FE_LAPLACE, y)
+    torch.cuda.synchronize()
+    used = free0 - torch.cuda.mem_get_info()[0]
+    coords32 = 3 * 4 * n
+    # 128 MB: the device pool's growth in large steps, and the kernels loaded by their first launch
+    assert used <= coords32 + (48 << 20) + (128 << 20), used / 2 ** 20
+    gm.close()
