@@ -2,8 +2,11 @@
 Sec. 6.2) against the FP64 CPU oracle and against the stored-metric mode of the same mesh.
 
 The two modes describe the same operator, so they must agree to the FP64 bar (1e-12 relative
-max-norm).  Meshes of the chunked sizes make the apply walk several L2-sized chunks of cells with
-a ragged last chunk."""
+max-norm).  Meshes whose metric is larger than the scratch make the apply walk several chunks of cells
+with a ragged last one."""
+import os
+import re
+
 import numpy as np
 import pytest
 
@@ -29,6 +32,13 @@ def fe():
 
 def to_host(t):
     return t.detach().cpu().numpy().astype(np.float64)
+
+
+def scratch_bytes(name):
+    """A scratch size of the library's source."""
+    src = open(os.path.join(os.path.dirname(os.path.abspath(__file__)), os.pardir, "paper_2607_02335_gb300",
+                            "csrc", "fe_internal.h")).read()
+    return int(re.search(rf"#define {name} \((\d+)LL << 20\)", src).group(1)) << 20
 
 
 @pytest.mark.parametrize("p", [1, 2, 3, 4, 5, 6, 7])
@@ -64,11 +74,12 @@ def test_recompute_assembled_dirichlet_and_diag(fe, p, m):
         assert rel_max_err(to_host(gm.diag(op)), dref) <= TOL64, op
 
 
-@pytest.mark.parametrize("p,m", [(3, 32), (7, (14, 14, 15)), (1, 64)])
+@pytest.mark.parametrize("p,m", [(3, 54), (7, (26, 27, 28)), (1, 108)])
 def test_recompute_several_chunks(fe, p, m):
     """Sizes whose metric spans several scratch chunks (the last one ragged): recompute equals
     stored over the whole vector in every arithmetic, and sampled entries match the oracle."""
     gr = fe.Mesh(m, p, deform_amp=0.1, geom_mode=fe.FE_GEOM_RECOMPUTE)
+    assert 7 * 4 * gr.cellwise_len > scratch_bytes("FE_RC_CHUNK_BYTES")  # in FP32, the smaller one
     gs = fe.Mesh(m, p, deform_amp=0.1)
     xg = S.primal_unique(m, p, seed=2)
     x = gr.gather(xg)
@@ -108,6 +119,31 @@ def test_recompute_pairs_and_ragged_chunks(fe, p, m):
             ys = gs.apply(v, op=op, **kw)
             err = (gr.apply(v, op=op, **kw) - ys).abs().max().item()
             assert err <= tol * ys.abs().max().item(), (op, kw)
+    gr.close()
+    gs.close()
+
+
+# odd and even n, more than 256 MB of FP32 metric, the last chunk ragged
+@pytest.mark.parametrize("p,m", [(2, (71, 73, 71)), (3, (54, 55, 53)), (4, (43, 43, 45)), (5, (37, 35, 37))])
+def test_recompute_several_chunks_in_every_arithmetic(fe, p, m):
+    """Meshes whose metric spans several scratch chunks in FP64, on the FP64 pipe, in FP32 and for the
+    diagonal: recompute equals stored, unassembled and assembled.  The bounds are those of the oracle
+    comparisons above, which both sides meet."""
+    gr = fe.Mesh(m, p, deform_amp=0.1, geom_mode=fe.FE_GEOM_RECOMPUTE)
+    gs = fe.Mesh(m, p, deform_amp=0.1)
+    entries = gr.cellwise_len
+    assert 7 * 4 * entries > scratch_bytes("FE_RC_CHUNK_BYTES")
+    assert 7 * 8 * entries > scratch_bytes("FE_RC_DIAG_BYTES")
+    g = torch.Generator(device="cuda").manual_seed(p)
+    x = torch.rand(entries, generator=g, dtype=torch.float64, device="cuda") - 0.5
+    for op in (fe.FE_LAPLACE, fe.FE_MASS):
+        for kw, v, tol in (({}, x, TOL64), ({"flags": fe.FE_ASSEMBLE}, x, TOL64),
+                           ({"flags": fe.FE_NATIVE_F64}, x, TOL64), ({"prec": fe.FE_F32}, x.float(), TOL32)):
+            ys = gs.apply(v, op=op, **kw)
+            err = (gr.apply(v, op=op, **kw) - ys).abs().max().item()
+            assert err <= tol * ys.abs().max().item(), (op, kw)
+        ds = gs.diag(op)
+        assert (gr.diag(op) - ds).abs().max().item() <= TOL64 * ds.abs().max().item(), op
     gr.close()
     gs.close()
 
