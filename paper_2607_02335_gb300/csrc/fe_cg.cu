@@ -460,6 +460,25 @@ fe_status fe_launch_invmult(const fe_mesh* m, float* out, cudaStream_t st) {
   return fe_cuda_check(cudaGetLastError(), "invmult launch");
 }
 
+static fe_status alloc_work(const fe_mesh* m, CgWork* w) {
+  const long long n = m->ncw;
+  w->n = n;
+  FE_CUDA(cudaStreamCreateWithFlags(&w->st, cudaStreamNonBlocking), "cg stream");
+  double** d[] = {&w->x, &w->r, &w->z, &w->p, &w->q, &w->w, &w->bs, &w->invdiag64};
+  for (double** v : d) FE_TRY(fe_dalloc((void**)v, n * sizeof(double), w->st, "cg vector"));
+  FE_TRY(fe_dalloc((void**)&w->invdiag32, n * sizeof(float), w->st, "cg vector"));
+  FE_TRY(fe_dalloc((void**)&w->invmult, n * sizeof(float), w->st, "cg vector"));
+  FE_TRY(fe_dalloc((void**)&w->partials,
+                   ((size_t)RED_BLOCKS * RED_SLOTS + m->ncells / 2 + 1) * sizeof(double), w->st,
+                   "cg partials"));
+  FE_TRY(fe_dalloc((void**)&w->count, sizeof(unsigned), w->st, "cg counter"));
+  FE_CUDA(cudaMemsetAsync(w->count, 0, sizeof(unsigned), w->st), "cg counter");
+  FE_TRY(fe_dalloc((void**)&w->sc, 2 * sizeof(CgScal), w->st, "cg scalars"));
+  FE_CUDA(cudaMallocHost(&w->hsc, 2 * sizeof(CgScal)), "cudaMallocHost cg scalars");
+  return fe_launch_invmult(m, w->invmult, w->st);
+}
+
+// the mesh keeps a workspace only once it is whole: after a failed allocation the next solve starts anew
 fe_status fe_cg_get_work(const fe_mesh* cm, bool mixed, CgWork** out) {
   fe_mesh* m = const_cast<fe_mesh*>(cm);
   CgWork* w = static_cast<CgWork*>(m->cg_work);
@@ -469,27 +488,18 @@ fe_status fe_cg_get_work(const fe_mesh* cm, bool mixed, CgWork** out) {
       fe_set_error("fe_cg_solve: host allocation failed");
       return FE_ERR_OOM;
     }
+    const fe_status s = alloc_work(m, w);
+    if (s != FE_OK) {
+      free_work(w, w->st);
+      return s;
+    }
     m->cg_work = w;
     m->cg_free = [](void* p, cudaStream_t st) { free_work(static_cast<CgWork*>(p), st); };
-    const long long n = m->ncw;
-    w->n = n;
-    FE_CUDA(cudaStreamCreateWithFlags(&w->st, cudaStreamNonBlocking), "cg stream");
-    double** d[] = {&w->x, &w->r, &w->z, &w->p, &w->q, &w->w, &w->bs, &w->invdiag64};
-    for (double** v : d) FE_TRY(fe_dalloc((void**)v, n * sizeof(double), w->st, "cg vector"));
-    FE_TRY(fe_dalloc((void**)&w->invdiag32, n * sizeof(float), w->st, "cg vector"));
-    FE_TRY(fe_dalloc((void**)&w->invmult, n * sizeof(float), w->st, "cg vector"));
-    FE_TRY(fe_dalloc((void**)&w->partials,
-                     ((size_t)RED_BLOCKS * RED_SLOTS + m->ncells / 2 + 1) * sizeof(double), w->st,
-                     "cg partials"));
-    FE_TRY(fe_dalloc((void**)&w->count, sizeof(unsigned), w->st, "cg counter"));
-    FE_CUDA(cudaMemsetAsync(w->count, 0, sizeof(unsigned), w->st), "cg counter");
-    FE_TRY(fe_dalloc((void**)&w->sc, 2 * sizeof(CgScal), w->st, "cg scalars"));
-    FE_CUDA(cudaMallocHost(&w->hsc, 2 * sizeof(CgScal)), "cudaMallocHost cg scalars");
-    FE_TRY(fe_launch_invmult(m, w->invmult, w->st));
   }
-  if (mixed && !w->r32) {
+  if (mixed) {
     float** f[] = {&w->r32, &w->z32, &w->p32, &w->q32, &w->w32, &w->d32};
-    for (float** v : f) FE_TRY(fe_dalloc((void**)v, w->n * sizeof(float), w->st, "cg fp32 vector"));
+    for (float** v : f)
+      if (!*v) FE_TRY(fe_dalloc((void**)v, w->n * sizeof(float), w->st, "cg fp32 vector"));
   }
   *out = w;
   return FE_OK;

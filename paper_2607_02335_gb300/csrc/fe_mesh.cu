@@ -30,6 +30,7 @@ void fe_set_error(const char* fmt, ...) {
 
 fe_status fe_cuda_check(cudaError_t e, const char* what) {
   if (e == cudaSuccess) return FE_OK;
+  cudaGetLastError();  // reported here: the next launch's check must not find it again
   fe_set_error("%s: %s", what, cudaGetErrorString(e));
   return e == cudaErrorMemoryAllocation ? FE_ERR_OOM : FE_ERR_CUDA;
 }
