@@ -985,14 +985,20 @@ static fe_status launch_apply_batched(FeBatch* B, int slot, int src = 0) {
     for (int k = 0; k < forks; ++k)
       FE_CUDA(cudaStreamWaitEvent(B->fork_st[k], B->fork_ev[forks], 0), "batch fork");
   }
-  for (int k = 0; k < nd; ++k)
-    FE_TRY((launch_apply_degree<V>(B, deg[k], slot, src,
-                                   k == 0 ? B->st : B->fork_st[(k - 1) % FeBatch::FORKS])));
+  fe_status status = FE_OK;
+  for (int k = 0; k < nd && status == FE_OK; ++k)
+    status = launch_apply_degree<V>(B, deg[k], slot, src,
+                                    k == 0 ? B->st : B->fork_st[(k - 1) % FeBatch::FORKS]);
+  // joined also after a failure: the batch's buffers are freed or rebuilt in the order of st
   for (int k = 0; k < forks; ++k) {
-    FE_CUDA(cudaEventRecord(B->fork_ev[k], B->fork_st[k]), "batch join");
-    FE_CUDA(cudaStreamWaitEvent(B->st, B->fork_ev[k], 0), "batch join");
+    cudaError_t e = cudaEventRecord(B->fork_ev[k], B->fork_st[k]);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(B->st, B->fork_ev[k], 0);
+    if (e == cudaSuccess) continue;
+    cudaStreamSynchronize(B->fork_st[k]);
+    const fe_status s = fe_cuda_check(e, "batch join");
+    if (status == FE_OK) status = s;
   }
-  return FE_OK;
+  return status;
 }
 
 template <class S>

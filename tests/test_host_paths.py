@@ -75,3 +75,24 @@ def test_a_solve_after_a_failed_allocation(lib, mixed):
         seen.clear()
         lib.fe_mesh_destroy(h)
     assert 15 < failed < 39  # every failable call of the solve, and a few solves beyond the last
+
+
+def test_nothing_is_freed_under_a_forked_apply(lib):
+    """A batched solve of three degrees, with each of its first calls that allocate, launch, fork or join
+    failing in turn: the error is reported, and no buffer is freed while a forked stream still holds kernels
+    that nothing orders before the free."""
+    from paper_2607_02335_gb300 import fe
+    shapes = [((2, 2, 2), 1), ((2, 2, 2), 2), ((2, 2, 2), 4)]
+    meshes = [mesh(fe, lib, m, p) for m, p in shapes]
+    vecs = [[aligned(8 * (p + 1) ** 3) for _, p in shapes] for _ in range(2)]
+    arr = [(ctypes.c_void_p * 3)(*[v.ctypes.data for v in vs]) for vs in vecs]
+    hs = (ctypes.c_void_p * 3)(*meshes)
+    for mixed in (0, fe.FE_F32):
+        opts = fe.fe_cg_opts(1e-10, 100, mixed, 0, 0.1, None)
+        for n in range(1, 160):
+            res = (fe.fe_cg_result * 3)()
+            lib.fake_fail_at(n)
+            st = lib.fe_cg_solve_batched(3, hs, arr[0], arr[1], ctypes.byref(opts), res, None)
+            lib.fake_fail_at(0)
+            assert st != 0, (mixed, n)
+            assert lib.fake_unordered_frees() == 0, (mixed, n)
