@@ -170,6 +170,9 @@ static fe_status launch_shape(const ApplyArgs<N, V>& a, cudaStream_t st) {
             "apply smem attribute");
     if (dev >= 0 && dev < 64) attr_done[dev] = true;
   }
+  if constexpr (CG) {
+    if (a.cg.prepare) return FE_OK;
+  }
   long long blocks;
   int threads = Sh::THREADS;
   if constexpr (MODE == MODE_BRICK) {

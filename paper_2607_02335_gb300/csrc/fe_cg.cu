@@ -558,6 +558,13 @@ fe_status launch_precond(const fe_mesh* m, CgWork* w, S* wv, S* r, const S* q, c
   return fe_cuda_check(cudaGetLastError(), "preconditioner launch");
 }
 
+// whether the operator takes its neighbours of the iteration into its kernel
+template <class S>
+bool fuses(const fe_mesh* m, const CgWork* w) {
+  return sizeof(S) == 8 ? fe_apply_fuses_cg(m, FE_F64)
+                        : w->inner_prec == FE_F32 && fe_apply_fuses_cg(m, FE_F32);
+}
+
 // one PCG iteration on vectors of type S, solution of type U, scalars sc
 template <class S, class U>
 fe_status enqueue_iteration(const fe_mesh* m, CgWork* w, int op, bool flexible, U* u, S* r, S* z,
@@ -567,9 +574,8 @@ fe_status enqueue_iteration(const fe_mesh* m, CgWork* w, int op, bool flexible, 
   // FP32 iterations redistribute: r = (S r)/mult is formed by the preconditioner
   const int redistribute = sizeof(S) == 4 ? 1 : 0;
   const unsigned grid = red_grid(n);
-  const CgApply cg{z, sc, w->partials + (size_t)RED_BLOCKS * RED_SLOTS, w->count, hist};
-  const bool fused = sizeof(S) == 8 ? fe_apply_fuses_cg(m, FE_F64)
-                                    : w->inner_prec == FE_F32 && fe_apply_fuses_cg(m, FE_F32);
+  const CgApply cg{z, sc, w->partials + (size_t)RED_BLOCKS * RED_SLOTS, w->count, hist, 0};
+  const bool fused = fuses<S>(m, w);
   if (fused)
     L.cg = &cg;
   else
@@ -595,8 +601,10 @@ fe_status build_graph(const fe_mesh* m, CgWork* w, int op, bool flexible, U* u, 
                       S* q, S* wv, const S* invdiag, CgScal* sc, double* hist,
                       cudaGraphExec_t* exec) {
   cudaGraph_t g = nullptr;
-  {  // one uncaptured apply first, so that per-kernel attributes are set outside the capture
+  {  // per-kernel attributes are set outside the capture: by one apply first, the fused one's without a launch
     ApplyLaunch L{m, op, p, q, w->st, &sc->done};
+    const CgApply cg{z, sc, nullptr, nullptr, nullptr, 1};
+    if (fuses<S>(m, w)) L.cg = &cg;
     FE_TRY(sizeof(S) == 8 ? fe_launch_apply_f64dw(L) : launch_inner_apply(L, w));
   }
   FE_CUDA(cudaStreamBeginCapture(w->st, cudaStreamCaptureModeThreadLocal), "begin capture");

@@ -155,6 +155,7 @@ struct CgApply {
   double* partials;  // one per CTA: at least n_cells / 2 + 1
   unsigned* count;   // 0 between launches
   double* hist;      // alpha history or null
+  int prepare;       // nonzero: set the kernel's attributes and launch nothing (before a stream capture)
 };
 // apply (fe_apply.cu / fe_apply_*.cu)
 struct ApplyLaunch {

@@ -96,3 +96,35 @@ def test_nothing_is_freed_under_a_forked_apply(lib):
             lib.fake_fail_at(0)
             assert st != 0, (mixed, n)
             assert lib.fake_unordered_frees() == 0, (mixed, n)
+
+
+class Scal(ctypes.Structure):  # the start of CgScal (fe_cgcore.h)
+    _fields_ = [(k, ctypes.c_double) for k in ("rz", "rz_new", "qp", "qz", "alpha", "beta", "rnorm2", "bnorm2",
+                                               "relres", "best")] + [("done", ctypes.c_int)]
+
+
+# single cells and pairs in FP64 (fused and separate iterations), FP32
+@pytest.mark.parametrize("p,m,mixed", [(3, (2, 2, 2), False), (6, (2, 2, 2), False), (3, (24, 24, 24), False),
+                                       (2, (3, 3, 3), True), (7, (2, 2, 2), True)])
+def test_no_kernel_attribute_is_set_inside_a_capture(lib, p, m, mixed):
+    """The iteration graph's capture holds launches only: each kernel was loaded and had its attributes set
+    before."""
+    from paper_2607_02335_gb300 import fe
+    n = m[0] * m[1] * m[2] * (p + 1) ** 3
+    b, x = aligned(n), aligned(n)
+    opts = fe.fe_cg_opts(1e-10, 100, fe.FE_F32 if mixed else 0, 0, 0.1, None)
+
+    def on_launch(name, args):
+        if b"k_precond" in name:  # a right-hand side that is not zero, and a residual to iterate on
+            sc = ctypes.cast(pointer_arg(args, 8), ctypes.POINTER(Scal))[0]
+            sc.bnorm2 = sc.rnorm2 = sc.rz = sc.relres = 1.0
+
+    hook = HOOK(on_launch)
+    h, res, graphs = mesh(fe, lib, m, p), fe.fe_cg_result(), lib.fake_graphs()
+    lib.fake_hook(hook)
+    lib.fe_cg_solve(h, ctypes.c_void_p(b.ctypes.data), ctypes.c_void_p(x.ctypes.data), ctypes.byref(opts),
+                    ctypes.byref(res), None)  # ends at the first replay, which the stand-in refuses
+    lib.fake_hook(None)
+    lib.fe_mesh_destroy(h)
+    assert lib.fake_graphs() == graphs + 1
+    assert lib.fake_attr_in_capture() == 0
