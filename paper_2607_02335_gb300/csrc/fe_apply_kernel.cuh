@@ -379,16 +379,15 @@ __host__ __device__ constexpr int apply_narr(int op) { return op == FE_LAPLACE ?
 
 template <int N, class V, int OP, int GEOM, int MODE>
 __device__ __forceinline__ void apply_cells_rolled(const CellArgs<N, V>& a, const Tab1D<N, V>& tab,
-                                                   long long cell0, unsigned char* smraw,
-                                                   int tile_stride) {
+                                                   long long cell0, unsigned char* smraw) {
   constexpr int RU = roll_unroll<N, OP>();
   using T = NT<V>;
   using C = Cfg<N>;
   constexpr int N2 = C::N2, N3 = C::N3, RS = C::RS, PS = C::PS;
   constexpr int NARR = (OP == FE_LAPLACE) ? 3 : 1;
-  const Sm<V> s0(smraw, NARR, 0, tile_stride);
-  const Sm<V> s1(smraw, NARR, NARR > 1 ? 1 : 0, tile_stride);
-  const Sm<V> s2(smraw, NARR, NARR > 2 ? 2 : 0, tile_stride);
+  const Sm<V> s0(smraw, NARR, 0, Cfg<N>::TILE);
+  const Sm<V> s1(smraw, NARR, NARR > 1 ? 1 : 0, Cfg<N>::TILE);
+  const Sm<V> s2(smraw, NARR, NARR > 2 ? 2 : 0, Cfg<N>::TILE);
 
   const int t = threadIdx.x;
   const int cl = t / N2;
@@ -538,23 +537,22 @@ __device__ __forceinline__ void apply_cells_rolled(const CellArgs<N, V>& a, cons
 template <int N, class V, int OP, int GEOM, int MODE = MODE_CELLS, bool CG = false>
 __device__ __forceinline__ void apply_cells(const CellArgs<N, V>& a, const Tab1D<N, V>& tab,
                                             long long cell0, unsigned char* smraw,
-                                            int tile_stride,
                                             ZCarry<typename NT<V>::SV>* zc = nullptr,
                                             const CgApply* cg = nullptr) {
   static_assert(MODE != MODE_PACKED || N < FE_ROLL_MINN, "packed units: unrolled degrees only");
   static_assert(MODE != MODE_BRICKZ || (N < FE_ROLL_MINN && !NT<V>::LOWP),
                 "z-carry bricks: unrolled degrees, FP64 / FP32 values");
   if constexpr (N >= roll_minn<V>() && MODE != MODE_PACKED) {
-    apply_cells_rolled<N, V, OP, GEOM, MODE>(a, tab, cell0, smraw, tile_stride);
+    apply_cells_rolled<N, V, OP, GEOM, MODE>(a, tab, cell0, smraw);
     return;
   }
   using T = NT<V>;
   using C = Cfg<N>;
   constexpr int N2 = C::N2, N3 = C::N3;
   constexpr int NARR = (OP == FE_LAPLACE) ? 3 : 1;
-  const Sm<V> s0(smraw, NARR, 0, tile_stride);
-  const Sm<V> s1(smraw, NARR, NARR > 1 ? 1 : 0, tile_stride);
-  const Sm<V> s2(smraw, NARR, NARR > 2 ? 2 : 0, tile_stride);
+  const Sm<V> s0(smraw, NARR, 0, Cfg<N>::TILE);
+  const Sm<V> s1(smraw, NARR, NARR > 1 ? 1 : 0, Cfg<N>::TILE);
+  const Sm<V> s2(smraw, NARR, NARR > 2 ? 2 : 0, Cfg<N>::TILE);
 
   const int t = threadIdx.x;
   const int cl = t / N2;
@@ -844,7 +842,7 @@ __global__ void __launch_bounds__(Cfg<N>::THREADS, 1) k_apply(const __grid_const
     cell0 = (long long)blockIdx.x * Packed<N>::UPB;
   else
     cell0 = a.c.cell_base + (long long)blockIdx.x * Cfg<N>::CPB;
-  apply_cells<N, V, OP, GEOM, MODE, CG>(a.c, a.tab, cell0, smraw, Cfg<N>::TILE, nullptr, &a.cg);
+  apply_cells<N, V, OP, GEOM, MODE, CG>(a.c, a.tab, cell0, smraw, nullptr, &a.cg);
 }
 
 // MODE_BRICKZ: blockIdx.x = chunk * (bricks per layer) + brick column; the CTA applies the layers
@@ -865,8 +863,7 @@ __global__ void __launch_bounds__(Cfg<N>::THREADS,
   zc.pending = false;
   for (int cz = z0; cz < z1; ++cz) {
     zc.last = cz == z1 - 1;
-    apply_cells<N, V, OP, GEOM, MODE_BRICKZ>(a.c, a.tab, (long long)cz * per_layer + col, smraw,
-                                             Cfg<N>::TILE, &zc);
+    apply_cells<N, V, OP, GEOM, MODE_BRICKZ>(a.c, a.tab, (long long)cz * per_layer + col, smraw, &zc);
     __syncthreads();  // the next layer refills the tile
   }
 }

@@ -102,7 +102,6 @@ Tab1D<N, V> make_tab(const HostTab& h) {
     fill_eob<N, V>(t.eB, h);
   } else {
     fill_eo<N, V>(t.eD, h.D, false);
-    fill_full<Tab1D<N, V>, V, N>(t, h);
   }
   return t;
 }
@@ -155,10 +154,16 @@ inline int fe_sm_count() {  // of the current device
 template <int N, class V, int OP, int GEOM, int MODE, class Sh, bool CG = false>
 static fe_status launch_shape(const ApplyArgs<N, V>& a, cudaStream_t st) {
   // the fused CG iteration is an instantiation of its own: its loads and sums take registers
-  if constexpr (!CG && OP == FE_LAPLACE && MODE == MODE_CELLS &&
-                (std::is_same<V, float>::value || std::is_same<V, dw>::value ||
-                 std::is_same<V, dw2>::value)) {
-    if (a.cg.sc) return launch_shape<N, V, OP, GEOM, MODE, Sh, true>(a, st);
+  if constexpr (!CG) {
+    if (a.cg.sc) {
+      if constexpr (OP == FE_LAPLACE && MODE == MODE_CELLS &&
+                    (std::is_same<V, float>::value || std::is_same<V, dw>::value)) {
+        return launch_shape<N, V, OP, GEOM, MODE, Sh, true>(a, st);
+      } else {  // fe_apply_fuses_cg does not ask for it
+        fe_set_error("apply: no fused CG iteration in this arithmetic or layout");
+        return FE_ERR_INVALID;
+      }
+    }
   }
   const size_t smem = Sh::smem(OP);
   auto kern = Sh::template kernel<OP, GEOM, MODE, CG>();
@@ -213,9 +218,12 @@ static RecomputeArgs<N, V> recompute_args(const HostTab& tab, const typename RV<
   r.geo = geo;
   r.skip = skip;
   for (int q = 0; q < N; ++q) r.tab.W_[q] = fe_cast<V>(tab.w[q]);
-  fill_eo<N, V>(r.tab.eV, tab.V, false);
-  fill_eo<N, V>(r.tab.eD, tab.D, false);
-  fill_full<RecomputeTab<N, V>, typename NT<V>::CV, N>(r.tab, tab);
+  if constexpr (rec_direct<N, V>()) {
+    fill_full<RecomputeTab<N, V>, typename NT<V>::CV, N>(r.tab, tab);
+  } else {
+    fill_eo<N, V>(r.tab.V_, tab.V, false);
+    fill_eo<N, V>(r.tab.D_, tab.D, false);
+  }
   return r;
 }
 template <int N, class V, int OP>

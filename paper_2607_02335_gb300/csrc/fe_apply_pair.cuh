@@ -390,6 +390,7 @@ __device__ __forceinline__ void apply_pairs(const CellArgs<N, typename PairCfg<N
                                             long long cell0, unsigned char* smraw,
                                             ZCarry2* zc = nullptr, const CgApply* cg = nullptr) {
   static_assert(SHAPE != TILE_SINGLE || MODE == MODE_CELLS, "single cells: consecutive cells only");
+  static_assert(!CG || SHAPE == TILE_SINGLE, "fused CG iteration: where single cells are taken");
   using C = PairCfg<N, SHAPE>;
   using V = typename C::V;
   using T = NT<V>;
@@ -779,7 +780,7 @@ __device__ __forceinline__ void apply_pairs(const CellArgs<N, typename PairCfg<N
 template <int N, int OP, int GEOM, int MODE, int SHAPE, bool CG>
 __global__ void __launch_bounds__(PairCfg<N, SHAPE>::THREADS,
                                   (SHAPE == TILE_PAIRS
-                                       ? (CG && N <= 4 ? 4 : pair_minb<N, OP, MODE>())
+                                       ? pair_minb<N, OP, MODE>()
                                        : 512 / ((PairCfg<N, SHAPE>::THREADS + 31) / 32 * 32)))
     k_apply_pair(const __grid_constant__ ApplyArgs<N, typename PairCfg<N, SHAPE>::V> a) {
   extern __shared__ __align__(16) unsigned char smraw[];

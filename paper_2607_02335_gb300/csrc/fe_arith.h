@@ -468,10 +468,10 @@ struct EOB {
 
 template <int N, class V>
 struct Tab1D {
-  V V_[N][N];  // V[q][i]  = l_i(s_q): GLL-node Lagrange basis at Gauss point q      (Sec. 2.3 "V")
-  V D_[N][N];  // D[q][r]  = derivative of the Gauss-point Lagrange basis r at s_q (collocation)
-  V W_[N];     // Gauss weights on [0,1]
-  EO<N, V> eV, eVT, eD, eDT;  // even-odd forms of V, V^T, D, D^T
+  V W_[N];  // Gauss weights on [0,1]
+  // even-odd forms of V[q][i] = l_i(s_q), the GLL-node Lagrange basis at Gauss point q (Sec. 2.3 "V"), of
+  // D[q][r], the derivative of the Gauss-point Lagrange basis r at s_q (collocation), and of V^T and D^T
+  EO<N, V> eV, eVT, eD, eDT;
 };
 
 // the tables of the FP64 apply (pairs and single cells): even-odd forms and weights

@@ -146,9 +146,9 @@ __device__ __forceinline__ void apply_item(const BProb& P, int prec, int src, lo
       apply_pairs<N, FE_LAPLACE, GEOM_STORED_K, MODE_CELLS>(a, tab_of<N, V>(), cell0, sm);
   } else {
     if (P.affine)
-      apply_cells<N, V, FE_LAPLACE, GEOM_AFFINE_K>(a, tab_of<N, V>(), cell0, sm, Cfg<N>::TILE);
+      apply_cells<N, V, FE_LAPLACE, GEOM_AFFINE_K>(a, tab_of<N, V>(), cell0, sm);
     else
-      apply_cells<N, V, FE_LAPLACE, GEOM_STORED_K>(a, tab_of<N, V>(), cell0, sm, Cfg<N>::TILE);
+      apply_cells<N, V, FE_LAPLACE, GEOM_STORED_K>(a, tab_of<N, V>(), cell0, sm);
   }
 }
 

@@ -45,11 +45,24 @@ struct RV<dw2> {
   using GV = float2;  // the halves of a double-word value side by side
 };
 
+// The plain product instead of the even-odd form: in single values (binary64, FP32) its operations cost
+// no more and its error is smaller (FP32 Q4, relative l2: 5.1e-7 against 7.8e-7); in double-word
+// values at n = 3 and 5, where the even-odd form saves little (Laplace, 64^3 and 40^3, one thread per
+// line: 0.471 against 0.486 ms, 0.650 against 0.719) and its error is the larger one (l2 3.6e-14
+// against 3.3e-14, 7.0e-14 against 5.7e-14; at n = 6: 1.0e-13 both, 0.677 against 0.830 ms).
 template <int N, class V>
+__host__ __device__ constexpr bool rec_direct() {
+  constexpr bool DW = std::is_same<V, dw2>::value || std::is_same<V, dw>::value;
+  return !DW || N == 3 || N == 5;
+}
+template <int N, class V, bool DIRECT = rec_direct<N, V>()>
 struct RecomputeTab {
-  using C = typename NT<V>::CV;
-  EO<N, V> eV, eD;
-  C V_[N][N], D_[N][N];
+  EO<N, V> V_, D_;
+  V W_[N];
+};
+template <int N, class V>
+struct RecomputeTab<N, V, true> {
+  typename NT<V>::CV V_[N][N], D_[N][N];
   V W_[N];
 };
 template <int N, class V>
@@ -79,31 +92,20 @@ __device__ __forceinline__ void tile_put<dw2>(dw2* p, dw2 v) {
   *reinterpret_cast<ulonglong2*>(p) = make_ulonglong2(v.h, v.l);
 }
 
-// The plain product instead of the even-odd form: in single values (binary64, FP32) its operations cost
-// no more and its error is smaller (FP32 Q4, relative l2: 5.1e-7 against 7.8e-7); in double-word
-// values at n = 3 and 5, where the even-odd form saves little (Laplace, 64^3 and 40^3, one thread per
-// line: 0.471 against 0.486 ms, 0.650 against 0.719) and its error is the larger one (l2 3.6e-14
-// against 3.3e-14, 7.0e-14 against 5.7e-14; at n = 6: 1.0e-13 both, 0.677 against 0.830 ms).
-template <int N, class V>
-__host__ __device__ constexpr bool rec_direct() {
-  constexpr bool DW = std::is_same<V, dw2>::value || std::is_same<V, dw>::value;
-  return !DW || N == 3 || N == 5;
-}
 // out = M in, normalised
-template <int N, class V, int SIG>
-__device__ __forceinline__ void rec_line(const EO<N, V>& eo, const typename NT<V>::CV (&full)[N][N],
-                                         const V (&in)[N], V (&out)[N]) {
+template <int N, class V, int SIG, class M>
+__device__ __forceinline__ void rec_line(const M& m, const V (&in)[N], V (&out)[N]) {
   using T = NT<V>;
   if constexpr (rec_direct<N, V>()) {
 #pragma unroll
     for (int q = 0; q < N; ++q) {
-      auto acc = T::prod(full[q][0], in[0]);
+      auto acc = T::prod(m[q][0], in[0]);
 #pragma unroll
-      for (int r = 1; r < N; ++r) acc = T::mac(acc, full[q][r], in[r]);
+      for (int r = 1; r < N; ++r) acc = T::mac(acc, m[q][r], in[r]);
       out[q] = T::fin(T::keep(acc));
     }
   } else {
-    eo_regs<N, V, SIG>(eo, in, out);
+    eo_regs<N, V, SIG>(m, in, out);
 #pragma unroll
     for (int q = 0; q < N; ++q) out[q] = T::fin(out[q]);
   }
@@ -165,33 +167,33 @@ __global__ void __launch_bounds__(RecCfg<N, V>::THREADS, RecCfg<N, V>::MINB)
     else
       in[k] = g[0];
   }
-  rec_line<N, V, 1>(a.tab.eV, a.tab.V_, in, out);
+  rec_line<N, V, 1>(a.tab.V_, in, out);
 #pragma unroll
   for (int k = 0; k < N; ++k) tile_put(s + bz + k * PS, out[k]);
   sync();
 #pragma unroll
   for (int r = 0; r < N; ++r) in[r] = tile_get(s + by + r * RS);
-  rec_line<N, V, 1>(a.tab.eV, a.tab.V_, in, out);
+  rec_line<N, V, 1>(a.tab.V_, in, out);
 #pragma unroll
   for (int r = 0; r < N; ++r) tile_put(s + by + r * RS, out[r]);
   sync();
 #pragma unroll
   for (int r = 0; r < N; ++r) in[r] = tile_get(s + bx + r);
-  rec_line<N, V, 1>(a.tab.eV, a.tab.V_, in, out);
+  rec_line<N, V, 1>(a.tab.V_, in, out);
 #pragma unroll
   for (int r = 0; r < N; ++r) tile_put(s + bx + r, out[r]);
-  rec_line<N, V, -1>(a.tab.eD, a.tab.D_, out, in);
+  rec_line<N, V, -1>(a.tab.D_, out, in);
 #pragma unroll
   for (int r = 0; r < N; ++r) tile_put(sx + d * G::TILE + bx + r, in[r]);
   sync();
 #pragma unroll
   for (int r = 0; r < N; ++r) in[r] = tile_get(s + by + r * RS);
-  rec_line<N, V, -1>(a.tab.eD, a.tab.D_, in, out);
+  rec_line<N, V, -1>(a.tab.D_, in, out);
 #pragma unroll
   for (int r = 0; r < N; ++r) tile_put(sy + d * G::TILE + by + r * RS, out[r]);
 #pragma unroll
   for (int k = 0; k < N; ++k) in[k] = tile_get(s + bz + k * PS);
-  rec_line<N, V, -1>(a.tab.eD, a.tab.D_, in, out);
+  rec_line<N, V, -1>(a.tab.D_, in, out);
   sync();  // the coordinates have been read
 #pragma unroll
   for (int k = 0; k < N; ++k) tile_put(s + bz + k * PS, out[k]);

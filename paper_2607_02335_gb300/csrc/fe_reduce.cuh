@@ -28,13 +28,6 @@ __device__ __forceinline__ dw block_reduce_dw(dw v, dw* sh /* [32] */) {
   return v;
 }
 
-template <class S>
-__device__ __forceinline__ dw to_dw(S v);
-template <>
-__device__ __forceinline__ dw to_dw<double>(double v) { return dw_from_double(v); }
-template <>
-__device__ __forceinline__ dw to_dw<float>(float v) { return {v, 0.0f}; }
-
 // CTA-wide binary64 sum in a fixed shuffle tree; result valid in thread 0
 __device__ __forceinline__ double block_reduce_f64(double v, double* sh /* [32] */) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
