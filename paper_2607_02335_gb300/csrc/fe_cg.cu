@@ -753,7 +753,7 @@ fe_status solve_fcg_outer(const fe_mesh* m, CgWork* w, int op, const double* b, 
     FE_TRY(read_scal(w, 0, &h));
     ++outer;
     res->rel_res = h.relres;
-    if (h.done) {  // breakdown flagged by k_fin_alpha
+    if (h.done) {  // breakdown flagged by fin_alpha
       *status = (fe_status)h.status;
       break;
     }

@@ -1,5 +1,5 @@
-"""The error-free building blocks of the FP64-accurate path, alone: a kernel compiled here from the
-library's headers runs them on given operands, against exact rational or correctly rounded sums."""
+"""The double-word building blocks of the FP64-accurate path, alone: kernels compiled here from the library's
+headers run them on given operands, against exactly rounded sums and against the scalar operations."""
 import ctypes
 import math
 import os
