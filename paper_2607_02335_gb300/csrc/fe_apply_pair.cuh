@@ -761,8 +761,12 @@ __device__ __forceinline__ void apply_pairs(const CellArgs<N, typename PairCfg<N
     }
     return;
   }
+  // two points per iteration from n = 5 on, so that one's conversion covers the other's branch and store: Q4
+  // 40^3 mass 73.8 -> 73.1 us, Q5 32^3 82.3 -> 81.4, Q7 32^3 190.1 -> 189.0; at n = 3 and 4 one is faster (Laplace
+  // Q2 64^3 145.3 against 146.8, Q3 64^3 328.8 against 331.2)
+  constexpr int OUT = N >= 5 ? 2 : 1;
   Acc<double> qp;
-#pragma unroll 1
+#pragma unroll(OUT)
   for (int k = 0; k < N; ++k) {
     double q[W];
     out(s0.get(bz + k * PS), k, q);
